@@ -23,9 +23,9 @@ NVCC_FLAGS = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC",
 CXX_FLAGS = ["-O2", "-std=c++17", "-fPIC", "-I", CSRC, "-I", INCLUDE]
 
 CU_SOURCES = ["api.cu", "factor.cu", "solve.cu", "update_tc.cu", "batch_api.cu", "batch_lu.cu", "selinv.cu",
-              "sweep.cu", "study.cu", "fqueue_f64.cu", "fqueue_tc.cu", "fqueue_ldlt.cu"]
+              "sweep.cu", "study.cu", "fqueue_f64.cu", "fqueue_tc.cu", "fqueue_ldlt.cu", "update_sl.cu"]
 CXX_SOURCES = ["analyze.cpp"]
-HEADERS = ["kernels.cuh", "spx_plan.h", "batch_kernel.cuh", "operand.cuh", "blocks.cuh", "tc_common.cuh", "fqueue.cuh"]
+HEADERS = ["kernels.cuh", "spx_plan.h", "batch_kernel.cuh", "operand.cuh", "blocks.cuh", "tc_common.cuh", "fqueue.cuh", "slices.cuh"]
 
 
 def _sources():

@@ -203,6 +203,20 @@ struct spx_handle_s {
     int opc_kind = -1;                // 0 tf32, 1 bf16, 2 split tf32
     alignas(64) unsigned char tmap[128];     // CUtensorMap over d_opc
     alignas(64) unsigned char tmap_lo[128];  // CUtensorMap over d_opc_lo
+    // FP64 updates and TRSM by error-free slices on the tensor cores
+    // (update_sl.cu): tiles and one-warp tasks per level, near targets first
+    // (sl_near, small_near: where the far ones begin),
+    // TRSM chunks, operand copies ([1]: the D L^T rows of LDL^T) with their row exponents
+    bool sl_ready = false, sl_failed = false;
+    std::vector<int64_t> sl_ptr, sl_near, small_ptr, small_near, slc_ptr;
+    spx::SlTile *d_sl_tiles = nullptr;
+    int32_t *d_sl_small = nullptr;
+    RowChunk *d_slc = nullptr;
+    int64_t *d_colbase = nullptr, *d_relbase = nullptr;   // per operand row: where its column goes
+    void *d_slop[2] = {nullptr, nullptr};
+    int32_t *d_slexp[2] = {nullptr, nullptr};
+    alignas(64) unsigned char tmap_sla[128];
+    alignas(64) unsigned char tmap_slb[128];
     int *d_tcerr = nullptr;
     double upd_flops_tc = 0, upd_elems_tc = 0, upd_op_elems_tc = 0;   // share of the tensor-core tasks
 
@@ -337,12 +351,34 @@ __global__ void set_tau_kernel(const unsigned long long *anorm_bits, double fixe
     *tau = fixed >= 0.0 ? fixed : scale * a;
 }
 
+// FP64 factorizations by slices: panels whose updates come to at least this
+// many multiply-adds (the lower triangle of their off-diagonal rows' product)
+// go to the tensor cores, the others' tasks to one warp each on the FP64 unit.
+constexpr double kSliceMinMacs = 8192.0;
+bool panel_slices(const spx::Plan &P, int32_t q)
+{
+    const double m = (double)P.ph[q] - P.pw[q];
+    return m * (m + 1.0) / 2.0 * P.pw[q] >= kSliceMinMacs;
+}
+// ... when the updates come to this many flops in all; smaller systems keep
+// the task queue (one launch).
+constexpr double kSliceMinFlops = 4e8;
+
 // Algorithmic work of every panel and update task, as the kernel classes
 // count it: fn(class, level, flops, elements of the factor's type, elements
 // of the tensor-core operand copy, FP32 target elements) -- diagonal block
 // and TRSM per panel (Sec. III steps 1, 2), one update per task (step 3).
+// The engine of an update task: by the source's width for the single-precision
+// tensor-core modes, by the task's multiply-adds for FP64 slices.
+enum UpdEngine { UPD_CUDA = 0, UPD_TC = 1, UPD_SLICES = 2 };
+bool on_tensor_cores(const spx::Plan &P, const spx::Task &tk, UpdEngine eng)
+{
+    if (eng == UPD_TC) return P.pw[tk.src] >= kTcMinWidth;
+    return eng == UPD_SLICES && panel_slices(P, tk.src);
+}
+
 template <typename F>
-void visit_work(const spx::Plan &P, bool tcm, F fn)
+void visit_work(const spx::Plan &P, UpdEngine eng, F fn)
 {
     const bool lu = P.method == SPX_LU;
     const double nfac = lu ? 2.0 : 1.0;
@@ -369,7 +405,7 @@ void visit_work(const spx::Plan &P, bool tcm, F fn)
             el_acc = 2.0 * (M * N + (M - N) * N);
         }
         const int lvl = P.plevel[tk.src];
-        if (tcm && P.pw[tk.src] >= kTcMinWidth) fn(SPX_K_UPDATE_TC, lvl, flops, 0.0, el_op, el_acc);
+        if (on_tensor_cores(P, tk, eng)) fn(SPX_K_UPDATE_TC, lvl, flops, 0.0, el_op, el_acc);
         else fn(SPX_K_UPDATE, lvl, flops, el_op + el_acc, 0.0, 0.0);
     }
 }
@@ -404,10 +440,21 @@ int queue_policy_level(const spx::Plan &P, int qopt, int prec)
     return queue_start_level(P, qopt == 0 ? INT32_MAX : qopt);
 }
 
+// Whether a factorization in `prec` runs its updates by slices: FP64 Cholesky
+// and LDL^T, walking the levels (no queue asked for, not the deterministic
+// rounds).
+bool slices_wanted(spx_handle h, int prec)
+{
+    const spx::Plan &P = h->plan;
+    if (prec != SPX_FP64 || P.method == SPX_LU || h->deterministic || h->queue_panels > 0) return false;
+    return h->queue_panels < 0 || P.update_flops >= kSliceMinFlops;
+}
+
 int32_t queue_level(spx_handle h, int prec)
 {
     const spx::Plan &P = h->plan;
     if (h->q_level >= P.nlevels || h->deterministic) return P.nlevels;
+    if (slices_wanted(h, prec) && h->sl_ready) return P.nlevels;
     return queue_policy_level(P, h->queue_panels, prec) >= P.nlevels ? P.nlevels : h->q_level;
 }
 
@@ -1013,6 +1060,102 @@ spx_status ensure_device(spx_handle h)
     return SPX_OK;
 }
 
+// The launch lists, operand copies and descriptors of the FP64 slices, on the
+// first FP64 factorization that wants them.  Where the copies do not fit the
+// device (1.75 times the factor's panels and the exponents), the handle stays
+// on the CUDA-core path.
+spx_status ensure_slices(spx_handle h)
+{
+    if (h->sl_ready || h->sl_failed) return SPX_OK;
+    const spx::Plan &P = h->plan;
+    const int64_t rows = std::max<int64_t>(h->op_rows, 1);
+    const int ncopy = P.method == SPX_LDLT ? 2 : 1;
+    if (rows * spx::kSliceCount >= INT32_MAX) {   // TMA row coordinates are 32-bit
+        h->sl_failed = true;
+        return SPX_OK;
+    }
+    const size_t bytes = (size_t)rows * spx::kSliceCount * h->kpad * 2;
+    const size_t nexp = (size_t)rows * (h->kpad / 64);
+    for (int k = 0; k < ncopy; ++k) {
+        if (cudaMalloc(&h->d_slop[k], bytes) != cudaSuccess ||
+            cudaMalloc((void **)&h->d_slexp[k], nexp * sizeof(int32_t)) != cudaSuccess) {
+            cudaGetLastError();
+            for (int j = 0; j < 2; ++j) {
+                cudaFree(h->d_slop[j]);
+                cudaFree(h->d_slexp[j]);
+                h->d_slop[j] = nullptr;
+                h->d_slexp[j] = nullptr;
+            }
+            h->sl_failed = true;
+            return SPX_OK;
+        }
+    }
+    for (int k = 0; k < ncopy; ++k) {
+        h->allocs.push_back(h->d_slop[k]);
+        h->allocs.push_back(h->d_slexp[k]);
+        CU(cudaMemset(h->d_slop[k], 0, bytes));
+        CU(cudaMemset(h->d_slexp[k], 0, nexp * sizeof(int32_t)));
+    }
+    if (spx::make_operand_map(h->tmap_sla, h->d_slop[0], rows * spx::kSliceCount, h->kpad, spx::OP_F16, 128) != 0 ||
+        spx::make_operand_map(h->tmap_slb, h->d_slop[ncopy - 1], rows * spx::kSliceCount, h->kpad, spx::OP_F16, 64) != 0)
+        return fail(h, SPX_ERR_CUDA, "cuTensorMapEncodeTiled failed for the FP64 slices");
+    std::vector<spx::SlTile> tiles;
+    std::vector<int32_t> small;
+    std::vector<RowChunk> chunks;
+    std::vector<int64_t> colbase((size_t)rows, 0), relbase((size_t)rows, 0);
+    std::vector<int32_t> rowlev((size_t)rows, 0);   // level of the panel a row faces
+    for (const spx::Task &tk : P.tasks)
+        for (int32_t r = tk.r0; r < tk.r1; ++r) {
+            const size_t R = (size_t)(P.prow[tk.src] + r);
+            colbase[R] = P.pval[tk.tgt] + (P.rows[R] - P.pfcol[tk.tgt]) * P.ph[tk.tgt];
+            relbase[R] = tk.relmap_off - tk.r0 - P.prow[tk.src];
+            rowlev[R] = P.plevel[tk.tgt];
+        }
+    h->sl_ptr.assign(P.nlevels + 1, 0);
+    h->small_ptr.assign(P.nlevels + 1, 0);
+    h->slc_ptr.assign(P.nlevels + 1, 0);
+    h->sl_near.assign(P.nlevels, 0);
+    h->small_near.assign(P.nlevels, 0);
+    std::vector<spx::SlTile> ft;
+    std::vector<int32_t> fs;
+    for (int32_t l = 0; l < P.nlevels; ++l) {
+        ft.clear();
+        fs.clear();
+        for (int32_t q = P.level_ptr[l]; q < P.level_ptr[l + 1]; ++q) {
+            const int32_t k = P.level_panels[q], w = P.pw[k], hk = P.ph[k];
+            for (int32_t r0 = w; r0 < hk; r0 += 64) chunks.push_back(RowChunk{k, r0});
+            if (!panel_slices(P, k)) continue;
+            for (int32_t n0 = w; n0 < hk; n0 += 64) {
+                const int32_t ncol = std::min(64, hk - n0);
+                bool near = false;   // rows ascend, not the levels of the panels that they face
+                for (int32_t c = 0; c < ncol; ++c) near = near || rowlev[(size_t)(P.prow[k] + n0 + c)] == l + 1;
+                for (int32_t m0 = w; m0 < hk; m0 += 128) {
+                    if (m0 + 128 <= n0) continue;
+                    (near ? tiles : ft)
+                        .push_back(spx::SlTile{(int32_t)(P.prow[k] + m0), (int32_t)(P.prow[k] + n0), w,
+                                               std::min(128, hk - m0), ncol, m0 - n0, {0, 0}});
+                }
+            }
+        }
+        for (int32_t t = P.level_task_ptr[l]; t < P.level_task_ptr[l + 1]; ++t)
+            if (!panel_slices(P, P.tasks[t].src)) (P.plevel[P.tasks[t].tgt] == l + 1 ? small : fs).push_back(t);
+        h->sl_near[l] = (int64_t)tiles.size();
+        h->small_near[l] = (int64_t)small.size();
+        tiles.insert(tiles.end(), ft.begin(), ft.end());
+        small.insert(small.end(), fs.begin(), fs.end());
+        h->sl_ptr[l + 1] = (int64_t)tiles.size();
+        h->small_ptr[l + 1] = (int64_t)small.size();
+        h->slc_ptr[l + 1] = (int64_t)chunks.size();
+    }
+    spx_status st;
+    if ((st = upload(h, &h->d_sl_tiles, tiles)) || (st = upload(h, &h->d_sl_small, small)) ||
+        (st = upload(h, &h->d_slc, chunks)) || (st = upload(h, &h->d_colbase, colbase)) ||
+        (st = upload(h, &h->d_relbase, relbase)))
+        return st;
+    h->sl_ready = true;
+    return SPX_OK;
+}
+
 // Enqueue the whole factorization on h->hs (captured into a graph).
 // Profiling: events recorded between kernel classes (non-graph runs only).
 struct Marks {
@@ -1043,6 +1186,12 @@ bool uses_tensor_cores(int method, int prec)
     if (method == SPX_LU) return false;
     if (method == SPX_LDLT) return prec == SPX_TF32 || prec == SPX_BF16;
     return prec == SPX_TF32 || prec == SPX_BF16 || prec == SPX_FP32;
+}
+
+UpdEngine update_engine(spx_handle h, int prec)
+{
+    if (slices_wanted(h, prec) && h->sl_ready) return UPD_SLICES;
+    return uses_tensor_cores(h->plan.method, prec) ? UPD_TC : UPD_CUDA;
 }
 
 int operand_kind(int method, int prec)
@@ -1112,6 +1261,7 @@ void enqueue_part_queue(spx_handle h, T *L, T *Dinv, T *W, void *opc, void *opc_
                                 h->tmap, h->tmap_lo, opc, opc_lo, h->kpad, op_kind, s);
 }
 
+constexpr int kFarTiles = 4;        // tiles a CTA of the far FP64 slice updates
 constexpr int kWhole = INT32_MIN;   // enqueue_factorization: the whole factorization
 
 template <typename T>
@@ -1124,6 +1274,7 @@ void enqueue_factorization(spx_handle h, bool mixed, Marks &mk, int prec, int pa
     const bool lu = P.method == SPX_LU;
     const bool ldlt = P.method == SPX_LDLT;
     const bool tc = uses_tensor_cores(P.method, prec) && sizeof(T) == 4;
+    const bool slices = sizeof(T) == 8 && part == kWhole && slices_wanted(h, prec) && h->sl_ready;
     void *opc = tc ? h->d_opc : nullptr;
     void *opc_lo = tc ? h->d_opc_lo : nullptr;
     const int op_kind = operand_kind(P.method, prec);
@@ -1239,7 +1390,14 @@ void enqueue_factorization(spx_handle h, bool mixed, Marks &mk, int prec, int pa
         };
         int64_t o;
         if (!lu) {
-            if (!link) {
+            if (slices) {
+                const int nsc = (int)(h->slc_ptr[l + 1] - h->slc_ptr[l]);
+                spx::launch_trsm_sl(h->dp, h->d_slc + h->slc_ptr[l], nsc, (const double *)Dinv, (double *)L,
+                                    (double *)W, ldlt ? 1 : 0, h->d_slop[0], h->d_slop[1], h->d_slexp[0],
+                                    h->d_slexp[1], h->op_rows, h->kpad, h->d_tcerr, s);
+                cnt += nsc > 0;
+                h->class_launches[SPX_K_TRSM] += nsc > 0;
+            } else if (!link) {
                 spx::launch_trsm<T>(h->dp, ch, nch, wmax, Dinv, L, ldlt ? spx::TRSM_LDLT : spx::TRSM_LLT, opc,
                                     opc_lo, h->kpad, op_kind, s, W);
                 cnt += nch > 0;
@@ -1254,7 +1412,15 @@ void enqueue_factorization(spx_handle h, bool mixed, Marks &mk, int prec, int pa
                                   Branches &ub, cudaStream_t one) {
                 const int na = (int)(a1 - a0), nb = (int)(b1 - b0), nc = (int)(c1 - c0);
                 auto st = [&](int k) { return one ? one : ub.pick(k); };
-                if (!tc) {
+                if (slices) {
+                    // far tiles (`one`) in short CTAs, so that the next levels' launches find free SMs
+                    spx::launch_update_sl(h->tmap_sla, h->tmap_slb, h->op_rows, h->dp, h->d_sl_tiles + c0, nc,
+                                          h->d_colbase, h->d_relbase, h->d_slexp[0], h->d_slexp[ldlt ? 1 : 0], (double *)L, h->d_tcerr,
+                                          one ? kFarTiles : 0, wmax, st(0));
+                    mk.mark(SPX_K_UPDATE_TC);
+                    spx::launch_update_small(h->dp, h->d_tasks, h->d_sl_small + a0, na, (const double *)L,
+                                             (const double *)Bop, (double *)L, st(nc > 0 ? 1 : 0));
+                } else if (!tc) {
                     spx::launch_update<T>(h->dp, h->d_tasks, h->d_tiles + a0, na, L, Bop, L, 1, 0, st(0), 0);
                     spx::launch_update<T>(h->dp, h->d_tasks, h->d_tiles + b0, nb, L, Bop, L, 1, 0,
                                           st(na > 0 ? 1 : 0), 1);
@@ -1277,7 +1443,24 @@ void enqueue_factorization(spx_handle h, bool mixed, Marks &mk, int prec, int pa
             const int64_t A0 = tc ? h->tcsmall_ptr[l] : h->tile_ptr[l], A1 = tc ? h->tcsmall_nar[l] : h->tile_nar[l];
             const int64_t B0 = A1, B1 = tc ? h->tcsmall_ptr[l + 1] : h->tile_ptr[l + 1];
             const int64_t C0 = tc ? h->tctile_ptr[l] : 0, C1 = tc ? h->tctile_ptr[l + 1] : 0;
-            if (h->deterministic) {
+            if (slices) {
+                const int64_t a0 = h->small_ptr[l], a1 = h->small_near[l], a2 = h->small_ptr[l + 1];
+                const int64_t c0 = h->sl_ptr[l], c1 = h->sl_near[l], c2 = h->sl_ptr[l + 1];
+                const bool far = lookahead && (a1 < a2 || c1 < c2);
+                if (far) cudaEventRecord(h->ev_trsm, s);
+                Branches ub{h, !mk.on};
+                launch_set(a0, lookahead ? a1 : a2, 0, 0, c0, lookahead ? c1 : c2, ub, nullptr);
+                ub.join();
+                mk.mark(SPX_K_UPDATE);
+                if (far) {
+                    cudaStream_t fs = h->fstream[l % 2];
+                    cudaStreamWaitEvent(fs, h->ev_trsm, 0);
+                    Branches none{h, false};
+                    launch_set(a1, a2, 0, 0, c1, c2, none, fs);
+                    cudaEventRecord(h->ev_far[l % 2], fs);
+                    far_pending[l % 2] = true;
+                }
+            } else if (h->deterministic) {
                 for (int r = 0; r < nround; ++r) {
                     int64_t oa, ob, oc = 0;
                     const int na = seg(sa, A0, A1, r, &oa), nb = seg(sb, B0, B1, r, &ob);
@@ -1485,7 +1668,7 @@ spx_status ensure_operand_copy(spx_handle h, int kind)
         spx_status st = dalloc(h, &p, bytes);
         if (st != SPX_OK) return st;
         CU(cudaMemset(p, 0, bytes));
-        if (spx::make_operand_map(part ? h->tmap_lo : h->tmap, p, h->op_rows, h->kpad, bf16) != 0)
+        if (spx::make_operand_map(part ? h->tmap_lo : h->tmap, p, h->op_rows, h->kpad, bf16 ? spx::OP_BF16 : spx::OP_F32) != 0)
             return fail(h, SPX_ERR_CUDA, "cuTensorMapEncodeTiled failed for the operand copy");
         (part ? h->d_opc_lo : h->d_opc) = p;
     }
@@ -1888,6 +2071,7 @@ spx_status ensure_factor_storage(spx_handle h, spx_precision precision)
             h->fgraph_prec = -1;
         }
     }
+    if (slices_wanted(h, precision) && (st = ensure_slices(h))) return st;
     if (uses_tensor_cores(P.method, precision)) {
         if ((st = ensure_operand_copy(h, operand_kind(P.method, precision)))) return st;
     }
@@ -2214,14 +2398,14 @@ spx_status spx_factorize(spx_handle h, const double *values, int values_on_devic
         }
         const double e = fp64 ? 8.0 : 4.0;
         const double nfac = (P.method == SPX_LU) ? 2.0 : 1.0;
-        const bool tcm = uses_tensor_cores(P.method, precision);
-        const double eop = precision == SPX_BF16 ? 2.0 : (precision == SPX_FP32 ? 8.0 : 4.0);
+        const UpdEngine tcm = update_engine(h, precision);
+        const double eop = tcm == UPD_SLICES ? 14.0 : precision == SPX_BF16 ? 2.0 : (precision == SPX_FP32 ? 8.0 : 4.0);
         const int32_t qlev = queue_level(h, precision);
         // (LDL^T reads its B operand from a second copy of the same size: the bytes are the same)
         visit_work(P, tcm, [&](int cls, int lvl, double flops, double el, double el_op, double el_acc) {
             const int c = lvl >= qlev ? (int)SPX_K_QUEUE : cls;
             K.flops[c] += flops;
-            K.bytes[c] += el * e + el_op * eop + el_acc * 4.0;
+            K.bytes[c] += el * e + el_op * eop + el_acc * e;
         });
         // zero fill of the factor (one write) + the scatter (value and map read, one write)
         K.bytes[SPX_K_ASSEMBLE] = (double)P.nnz_a * (16.0 + e * nfac) + (double)elems * e * nfac;
@@ -2476,16 +2660,17 @@ spx_status spx_roofline_model(spx_handle h, spx_precision precision, const doubl
     const double e = fp64 ? 8.0 : 4.0;
     const double bw = peaks[0] * 1e9, f64 = peaks[1] * 1e9, f32 = peaks[2] * 1e9, tc = peaks[3] * 1e9;
     const double simt = fp64 ? f64 : f32;
-    const bool tcm = uses_tensor_cores(P.method, precision);
-    const double eop = precision == SPX_BF16 ? 2.0 : (precision == SPX_FP32 ? 8.0 : 4.0);
-    const int qlev = P.method == SPX_LU ? P.nlevels
+    const UpdEngine tcm = slices_wanted(h, precision) ? UPD_SLICES
+                          : uses_tensor_cores(P.method, precision) ? UPD_TC : UPD_CUDA;
+    const double eop = tcm == UPD_SLICES ? 14.0 : precision == SPX_BF16 ? 2.0 : (precision == SPX_FP32 ? 8.0 : 4.0);
+    const int qlev = P.method == SPX_LU || tcm == UPD_SLICES ? P.nlevels
                      : queue_policy_level(P, h->queue_panels, precision);
     double ms[SPX_K_CLASSES] = {0, 0, 0, 0, 0, 0};
     const double nfac = lu ? 2.0 : 1.0;
     ms[SPX_K_ASSEMBLE] = ((double)P.nnz_a * (16.0 + e * nfac) + (double)P.pval[P.npanels] * e * nfac) / bw;
     visit_work(P, tcm, [&](int cls, int lvl, double flops, double el, double el_op, double el_acc) {
         const double peak = cls == SPX_K_DIAG ? f64 : (cls == SPX_K_UPDATE_TC ? tc : simt);
-        const double bytes = el * e + el_op * eop + el_acc * 4.0;
+        const double bytes = el * e + el_op * eop + el_acc * e;
         ms[lvl >= qlev ? (int)SPX_K_QUEUE : cls] += std::max(flops / peak, bytes / bw);
     });
     for (int c = 0; c < SPX_K_CLASSES; ++c) model_ms[c] = ms[c] * 1e3;

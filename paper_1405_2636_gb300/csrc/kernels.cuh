@@ -115,10 +115,34 @@ void launch_ldlt_diag(const DevPlan &p, const int32_t *panels, int count, int wm
 // operand copies (make_operand_map; tmap_lo is used for kind 2 only); err
 // receives 1 if a bounded wait expired.
 size_t tc_smem_bytes(int kind);
-int make_operand_map(void *tmap_out, void *base, int64_t rows, int kpad, int bf16);
+enum OperandType : int { OP_F32 = 0, OP_BF16 = 1, OP_F16 = 2 };
+int make_operand_map(void *tmap_out, void *base, int64_t rows, int kpad, int type, int box_rows = 128);
 void launch_update_tc(const void *tmap, const void *tmap_lo, int kind, const DevPlan &p,
                       const DevTask *tasks, const TcTile *tiles, int count, float *C, int lower,
                       int *err, cudaStream_t s);
+
+// FP64 updates and TRSM on the tensor cores by error-free slices
+// (update_sl.cu).  One tile: rows arow .. of the operand copy (nrow <= 128
+// valid) against rows brow .. (ncol <= 64) of the same panel, all k columns;
+// entry (r, c), kept when r + diff >= c, goes to C[colbase[brow + c] + relmap[relbase[brow + c] + arow + r]].
+struct __align__(16) SlTile {
+    int32_t arow, brow, k, nrow;
+    int32_t ncol, diff, pad[2];
+};
+constexpr int kSliceCount = 7;
+// oprows: rows of one slice of the operand copy; per_cta > 0: at most that
+// many tiles a CTA (a launch that others run beside), else one CTA an SM.
+// wmax: at least the width of every tile's panel.
+void launch_update_sl(const void *mapa, const void *mapb, int64_t oprows, const DevPlan &p, const SlTile *tiles,
+                      int count, const int64_t *colbase, const int64_t *relbase, const int32_t *expa, const int32_t *expb, double *C, int *err, int per_cta,
+                      int wmax, cudaStream_t s);
+// chunks: 64 rows each.  LDL^T: opa / expa hold L, opb / expb D L^T.
+void launch_trsm_sl(const DevPlan &p, const RowChunk *chunks, int count, const double *Dinv, double *X, double *Wout,
+                    int ldlt, void *opa, void *opb, int32_t *expa, int32_t *expb, int64_t oprows, int kpad, int *err,
+                    cudaStream_t s);
+// Tasks of few multiply-adds, one warp each.
+void launch_update_small(const DevPlan &p, const DevTask *tasks, const int32_t *ids, int count, const double *Aop,
+                         const double *Bop, double *C, cudaStream_t s);
 
 template <typename T>
 void launch_update(const DevPlan &p, const DevTask *tasks, const UpdTile *tiles, int count,

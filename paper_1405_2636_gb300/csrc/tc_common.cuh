@@ -128,6 +128,16 @@ __device__ __forceinline__ void mma(uint32_t tmem, uint64_t a, uint64_t b, uint3
     }
 }
 
+// One lane of a converged warp.  (A branch on elect.sync's predicate tells the
+// compiler that one thread runs it, so that descriptors stay in uniform
+// registers; a branch on the lane number does not.)
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t e;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(e));
+    return e != 0;
+}
+
 __device__ __forceinline__ void mma_commit(uint64_t *bar)
 {
     asm volatile(

@@ -369,7 +369,7 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t
 
 size_t tc_smem_bytes(int kind) { return (size_t)(kind == 2 ? 4 : 2) * kStages * kTileBytes + 1024; }
 
-int make_operand_map(void *tmap_out, void *base, int64_t rows, int kpad, int bf16)
+int make_operand_map(void *tmap_out, void *base, int64_t rows, int kpad, int type, int box_rows)
 {
     static EncodeTiledFn encode = nullptr;
     if (!encode) {
@@ -381,13 +381,16 @@ int make_operand_map(void *tmap_out, void *base, int64_t rows, int kpad, int bf1
             return -1;
         encode = (EncodeTiledFn)fn;
     }
-    const int esz = bf16 ? 2 : 4;
+    const int esz = type == OP_F32 ? 4 : 2;
     cuuint64_t dims[2] = {(cuuint64_t)kpad, (cuuint64_t)rows};
     cuuint64_t strides[1] = {(cuuint64_t)kpad * esz};
-    cuuint32_t box[2] = {(cuuint32_t)(kRowBytes / esz), (cuuint32_t)kM};
+    cuuint32_t box[2] = {(cuuint32_t)(kRowBytes / esz), (cuuint32_t)box_rows};
     cuuint32_t estr[2] = {1, 1};
     CUresult r = encode(reinterpret_cast<CUtensorMap *>(tmap_out),
-                        bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2,
+                        type == OP_BF16  ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16
+                        : type == OP_F16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16
+                                         : CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
+                        2,
                         base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                         CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
