@@ -129,10 +129,11 @@ struct spx_handle_s {
     std::vector<int64_t> tcsmall_ptr, tcsmall_nar; // per level, SIMT tiles of the narrow tasks
     // sweep work queues: item orders, chunk -> owning panels, per-panel wait
     // counts; d_qstate holds the per-sweep counters (zeroed each sweep)
+    spx::SweepItem *d_qdesc_f = nullptr, *d_qdesc_b = nullptr;
     int32_t *d_qitems_f = nullptr, *d_qitems_b = nullptr, *d_qtptr = nullptr, *d_qtgt = nullptr;
     int32_t *d_qneed_f = nullptr, *d_qneed_b = nullptr, *d_qstate = nullptr, *d_qerr = nullptr;
     int32_t *d_qmerge = nullptr;
-    int32_t q_nitems = 0, q_mat = 0, q_matb = 0, q_vec = 0;
+    int32_t q_nitems = 0, q_vec_rows = 64, q_mat = 0, q_matb = 0, q_vec = 0;
     uint32_t spin_limit = spx::kDefaultSpinLimit;   // polls before a sweep wait gives up
     int32_t *h_noalloc_err = nullptr;   // pinned: the error word of the last completed spx_solve_noalloc
     void *h_stage[2] = {nullptr, nullptr};  // pinned staging buffers for host-buffer copies
@@ -929,6 +930,7 @@ spx_status ensure_device(spx_handle h)
             if (!ok) return fail(h, SPX_ERR_STATE, "internal: sweep queue order violates a dependency");
         }
         h->q_nitems = (int32_t)itf.size();
+        h->q_vec_rows = (wmax + 63) & ~63;
         // staging sizes in elements, multiples of 4 so that the vectors
         // after the matrices stay aligned for 4-element vector accesses
         // (the backward sweep stores a w x w inverse with an odd leading
@@ -936,11 +938,38 @@ spx_status ensure_device(spx_handle h)
         h->q_mat = (wmax * std::max(wmax + ((wmax & 1) ? 2 : 1), 65) + 3) & ~3;
         h->q_matb = merge ? (65 * wmax + 3) & ~3 : 0;
         h->q_vec = 16 * std::max(wmax, 64);
-        if ((st = upload(h, &h->d_qitems_f, itf)) || (st = upload(h, &h->d_qitems_b, itb)) ||
+        auto describe = [&](const std::vector<int32_t> &order, const std::vector<int32_t> &need) {
+            std::vector<spx::SweepItem> out(order.size());
+            for (size_t k = 0; k < order.size(); ++k) {
+                const bool isp = order[k] < 0;
+                const int32_t q = isp ? -order[k] - 1 : chunks[order[k]].panel, c = isp ? pmerge[q] : order[k];
+                spx::SweepItem &it = out[k];
+                it = spx::SweepItem{};
+                it.inv = hpinv[q];
+                it.f = P.pfcol[q];
+                it.panel = q;
+                it.w = P.pw[q];
+                it.h = P.ph[q];
+                it.need = need[q];
+                it.panel_item = isp;
+                if (c >= 0) {
+                    const int32_t r0 = chunks[c].r0;
+                    it.chunk = P.pval[q] + r0;
+                    it.rows = P.prow[q] + r0;
+                    it.nr = std::min(spx::kTrsmRows, P.ph[q] - r0);
+                    it.t0 = tptr[c];
+                    it.t1 = tptr[c + 1];
+                }
+            }
+            return out;
+        };
+        if ((st = upload(h, &h->d_qdesc_f, describe(itf, needf))) ||
+            (st = upload(h, &h->d_qdesc_b, describe(itb, needb))) ||
+            (st = upload(h, &h->d_qitems_f, itf)) || (st = upload(h, &h->d_qitems_b, itb)) ||
             (st = upload(h, &h->d_qtptr, tptr)) || (st = upload(h, &h->d_qtgt, tgt)) ||
             (st = upload(h, &h->d_qneed_f, needf)) || (st = upload(h, &h->d_qneed_b, needb)) ||
             (st = upload(h, &h->d_qmerge, pmerge)) ||
-            (st = dalloc(h, &h->d_qstate, (size_t)4 * np + 2)) || (st = dalloc(h, &h->d_qerr, 1)))
+            (st = dalloc(h, &h->d_qstate, (size_t)4 * np * spx::kSweepGroups + 2)) || (st = dalloc(h, &h->d_qerr, 1)))
             return st;
         CU(cudaMemset(h->d_qerr, 0, sizeof(int32_t)));
     }
@@ -1571,39 +1600,44 @@ void enqueue_factorization(spx_handle h, bool mixed, Marks &mk, int prec, int pa
 // One forward + backward sweep in the factor's arithmetic: d_D = A^{-1} d_R.
 // Forward and backward substitution, Y (permuted right-hand sides) to Xs,
 // as one queue launch per direction (sweep.cu); Z and Tacc are work
-// vectors, `state` the 4 npanels + 2 per-sweep counters.  Returns the
+// vectors, `state` the 4 npanels groups + 2 per-sweep counters.  Returns the
 // kernels launched.
 template <typename T>
-int enqueue_queue_sweeps(spx_handle h, int nrhs, T *Y, T *Z, T *Tacc, T *Xs, int32_t *state, int32_t *err,
-                         cudaStream_t s)
+int enqueue_queue_sweeps(spx_handle h, int nrhs, T *Y, T *Z, T *Tacc, T *Xs, int32_t *state, int groups,
+                         int32_t *err, cudaStream_t s)
 {
     const spx::Plan &P = h->plan;
     const T *L = (const T *)h->d_L, *U = (const T *)h->d_U, *Dinv = (const T *)h->d_Dinv;
     const bool lu = P.method == SPX_LU;
     const int32_t np = P.npanels;
     cudaMemsetAsync(Tacc, 0, sizeof(T) * (size_t)P.n * nrhs, s);
-    cudaMemsetAsync(state, 0, sizeof(int32_t) * ((size_t)4 * np + 2), s);
+    const size_t part = (size_t)np * groups;
+    cudaMemsetAsync(state, 0, sizeof(int32_t) * (4 * part + 2), s);
     spx::SweepQueue q{};
     q.nitems = h->q_nitems;
     q.tptr = h->d_qtptr;
     q.tgt = h->d_qtgt;
+    q.merge = h->d_qmerge;
     q.err = err;
     q.spin_limit = h->spin_limit;
-    q.merge = h->d_qmerge;
+    q.vec_rows = h->q_vec_rows;
     q.mat_elems = h->q_mat;
     q.matb_elems = h->q_matb;
     q.vec_elems = h->q_vec;
+    q.groups = groups;
+    q.desc = h->d_qdesc_f;
     q.items = h->d_qitems_f;
     q.need = h->d_qneed_f;
     q.cnt = state;
-    q.flag = state + np;
-    q.head = state + 4 * np;
+    q.flag = state + part;
+    q.head = state + 4 * part;
     spx::launch_fwd_queue<T>(h->dp, q, h->d_chunks, Dinv, P.method != SPX_LLT ? 1 : 0, L, Y, Z, nrhs, s);
+    q.desc = h->d_qdesc_b;
     q.items = h->d_qitems_b;
     q.need = h->d_qneed_b;
-    q.cnt = state + 2 * np;
-    q.flag = state + 3 * np;
-    q.head = state + 4 * np + 1;
+    q.cnt = state + 2 * part;
+    q.flag = state + 3 * part;
+    q.head = state + 4 * part + 1;
     spx::launch_bwd_queue<T>(h->dp, q, h->d_chunks, Dinv, lu ? 1 : (P.method == SPX_LDLT ? 2 : 0), lu ? U : L, Z,
                              Tacc, Xs, nrhs, s);
     return 2 * (q.nitems > 0);
@@ -1617,7 +1651,8 @@ void enqueue_sweep(spx_handle h, int nrhs)
     T *Y = (T *)h->d_Y, *Z = (T *)h->d_Z, *Tacc = (T *)h->d_T, *Xs = (T *)h->d_Xs;
     int64_t k = 0;
     spx::launch_permute_in<T>(P.n, nrhs, h->d_R, P.n, h->d_perm, Y, s);
-    k += enqueue_queue_sweeps<T>(h, nrhs, Y, Z, Tacc, Xs, h->d_qstate, h->d_qerr, s);
+    k += enqueue_queue_sweeps<T>(h, nrhs, Y, Z, Tacc, Xs, h->d_qstate, spx::sweep_groups(sizeof(T) == 8, nrhs),
+                                 h->d_qerr, s);
     spx::launch_permute_out<T>(P.n, nrhs, Xs, h->d_perm, h->d_D, P.n, s);
     h->sweep_launches = k + 2;
 }
@@ -1909,7 +1944,7 @@ void enqueue_sweep_noalloc(spx_handle h, int nrhs, const double *B, int64_t ldb,
     int32_t *err = state + 4 * (size_t)P.npanels + 2;
     cudaMemsetAsync(err, 0, sizeof(int32_t), s);
     spx::launch_permute_in<T>(P.n, nrhs, B, ldb, h->d_perm, Y, s);
-    enqueue_queue_sweeps<T>(h, nrhs, Y, Z, Tacc, Xs, state, err, s);
+    enqueue_queue_sweeps<T>(h, nrhs, Y, Z, Tacc, Xs, state, 1, err, s);
     spx::launch_permute_out<T>(P.n, nrhs, Xs, h->d_perm, X, ldx, s);
     cudaMemcpyAsync(h->h_noalloc_err, err, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
 }

@@ -202,21 +202,34 @@ void launch_permute_in(int64_t n, int nrhs, const double *B, int64_t ldb, const 
 template <typename T>
 void launch_permute_out(int64_t n, int nrhs, const T *Y, const int64_t *perm, double *X,
                         int64_t ldx, cudaStream_t s);
-// Device-resident work queue of one sweep direction (sweep.cu).  items[]:
-// >= 0 a row chunk (index into the chunk list), < 0 panel -(item + 1), in
-// an order where every item's inputs come from earlier items.  cnt, flag
-// and head are zeroed before each sweep; err is set when a wait runs out.
+// One item of a sweep's work queue: a panel item (its inverse at Dinv + inv)
+// and / or 64 off-diagonal rows of the panel (nr > 0: values at L + chunk,
+// leading dimension h, row numbers at rows), whose owners are the panels
+// tgt[t0 .. t1).  need: counts a panel item waits for.
+struct __align__(16) SweepItem {
+    int64_t inv, chunk, f, rows;
+    int32_t panel, w, h, nr;
+    int32_t t0, t1, need, panel_item;
+};
+// Device-resident work queue of one sweep direction (sweep.cu): items in an
+// order where every item's inputs come from earlier items.  cnt, flag and
+// head are zeroed before each sweep; err is set when a wait runs out.
 struct SweepQueue {
-    const int32_t *items;
+    const SweepItem *desc;       // the items' descriptions, in order
+    const int32_t *items;        // the same items: >= 0 a row chunk (index into the chunk list), < 0 panel -(item + 1)
     int32_t nitems;
     const int32_t *tptr, *tgt;   // per chunk: the distinct panels owning its rows
     const int32_t *need;         // per panel: counts its panel item waits for
     const int32_t *merge;        // per panel: its first chunk when the panel item takes it along, else -1
     int32_t *cnt, *flag, *head;
     int32_t *err;
-    int32_t mat_elems, matb_elems, vec_elems;   // shared-memory staging, elements of T (matb_elems 0: no chunks taken along)
+    int32_t vec_rows;                           // rows of the widest panel, rounded up to 64
+    int32_t mat_elems, matb_elems, vec_elems;   // shared-memory staging of the 16-column kernels (matb_elems 0: no chunks taken along)
+    int32_t groups;                             // independent walks of the queue, each its column blocks; cnt and flag hold npanels counters each
     uint32_t spin_limit;                        // polls of ~256 ns before a wait gives up
 };
+constexpr int kSweepGroups = 4;   // most groups of one sweep
+int sweep_groups(bool fp64, int nrhs);
 constexpr uint32_t kDefaultSpinLimit = 1u << 22;   // about a second
 template <typename T>
 void launch_fwd_queue(const DevPlan &p, const SweepQueue &q, const RowChunk *chunks, const T *Dinv,
