@@ -257,6 +257,12 @@ struct spx_handle_s {
     bool zready = false;
     double *d_Zsel = nullptr, *d_Lh = nullptr;
     int32_t *d_row_task = nullptr;
+    // selected inversion by slices: 128-row chunks of the panels that take it,
+    // the 64-row chunks of the others, per level; L's diagonal exponents
+    std::vector<int64_t> sv128_ptr, sv64_ptr;
+    std::vector<int32_t> sv_blocks;   // most 64-column blocks of R in a slices panel of the level
+    RowChunk *d_sv128 = nullptr, *d_sv64 = nullptr;
+    int32_t *d_dexp = nullptr;
     int64_t *d_zmap = nullptr;
     double *d_scalar = nullptr;
     double *d_gtmp = nullptr, *d_lam = nullptr, *d_xg = nullptr;
@@ -364,6 +370,15 @@ bool panel_slices(const spx::Plan &P, int32_t q)
 // ... when the updates come to this many flops in all; smaller systems keep
 // the task queue (one launch).
 constexpr double kSliceMinFlops = 4e8;
+
+// Selected inversion: panels whose product Z_RR Lh has at least this many
+// multiply-adds go to the tensor cores by slices.
+constexpr double kSelinvMinMacs = 65536.0;
+bool selinv_slices(const spx::Plan &P, int32_t q)
+{
+    const double m = (double)P.ph[q] - P.pw[q];
+    return m * m * P.pw[q] >= kSelinvMinMacs;
+}
 
 // Algorithmic work of every panel and update task, as the kernel classes
 // count it: fn(class, level, flops, elements of the factor's type, elements
@@ -1089,6 +1104,25 @@ spx_status ensure_device(spx_handle h)
     return SPX_OK;
 }
 
+// Per off-diagonal row R = prow + r of a panel: where the column it faces lies
+// in the panel storage (colbase), and where in relmap the rows of that task
+// are listed (relbase + prow + r': the target row of source row r').
+spx_status ensure_colmaps(spx_handle h)
+{
+    if (h->d_colbase) return SPX_OK;
+    const spx::Plan &P = h->plan;
+    const size_t rows = (size_t)std::max<int64_t>(h->op_rows, 1);
+    std::vector<int64_t> colbase(rows, 0), relbase(rows, 0);
+    for (const spx::Task &tk : P.tasks)
+        for (int32_t r = tk.r0; r < tk.r1; ++r) {
+            const size_t R = (size_t)(P.prow[tk.src] + r);
+            colbase[R] = P.pval[tk.tgt] + (P.rows[R] - P.pfcol[tk.tgt]) * P.ph[tk.tgt];
+            relbase[R] = tk.relmap_off - tk.r0 - P.prow[tk.src];
+        }
+    spx_status st = upload(h, &h->d_relbase, relbase);
+    return st != SPX_OK ? st : upload(h, &h->d_colbase, colbase);
+}
+
 // The launch lists, operand copies and descriptors of the FP64 slices, on the
 // first FP64 factorization that wants them.  Where the copies do not fit the
 // device (1.75 times the factor's panels and the exponents), the handle stays
@@ -1131,15 +1165,9 @@ spx_status ensure_slices(spx_handle h)
     std::vector<spx::SlTile> tiles;
     std::vector<int32_t> small;
     std::vector<RowChunk> chunks;
-    std::vector<int64_t> colbase((size_t)rows, 0), relbase((size_t)rows, 0);
     std::vector<int32_t> rowlev((size_t)rows, 0);   // level of the panel a row faces
     for (const spx::Task &tk : P.tasks)
-        for (int32_t r = tk.r0; r < tk.r1; ++r) {
-            const size_t R = (size_t)(P.prow[tk.src] + r);
-            colbase[R] = P.pval[tk.tgt] + (P.rows[R] - P.pfcol[tk.tgt]) * P.ph[tk.tgt];
-            relbase[R] = tk.relmap_off - tk.r0 - P.prow[tk.src];
-            rowlev[R] = P.plevel[tk.tgt];
-        }
+        for (int32_t r = tk.r0; r < tk.r1; ++r) rowlev[(size_t)(P.prow[tk.src] + r)] = P.plevel[tk.tgt];
     h->sl_ptr.assign(P.nlevels + 1, 0);
     h->small_ptr.assign(P.nlevels + 1, 0);
     h->slc_ptr.assign(P.nlevels + 1, 0);
@@ -1178,8 +1206,7 @@ spx_status ensure_slices(spx_handle h)
     }
     spx_status st;
     if ((st = upload(h, &h->d_sl_tiles, tiles)) || (st = upload(h, &h->d_sl_small, small)) ||
-        (st = upload(h, &h->d_slc, chunks)) || (st = upload(h, &h->d_colbase, colbase)) ||
-        (st = upload(h, &h->d_relbase, relbase)))
+        (st = upload(h, &h->d_slc, chunks)) || (st = ensure_colmaps(h)))
         return st;
     h->sl_ready = true;
     return SPX_OK;
@@ -1422,7 +1449,7 @@ void enqueue_factorization(spx_handle h, bool mixed, Marks &mk, int prec, int pa
             if (slices) {
                 const int nsc = (int)(h->slc_ptr[l + 1] - h->slc_ptr[l]);
                 spx::launch_trsm_sl(h->dp, h->d_slc + h->slc_ptr[l], nsc, (const double *)Dinv, (double *)L,
-                                    (double *)W, ldlt ? 1 : 0, h->d_slop[0], h->d_slop[1], h->d_slexp[0],
+                                    (double *)W, ldlt ? spx::TRSM_LDLT : spx::TRSM_LLT, h->d_slop[0], h->d_slop[1], h->d_slexp[0],
                                     h->d_slexp[1], h->op_rows, h->kpad, h->d_tcerr, s);
                 cnt += nsc > 0;
                 h->class_launches[SPX_K_TRSM] += nsc > 0;
@@ -2862,7 +2889,7 @@ namespace {
 spx_status ensure_scalar(spx_handle h)
 {
     if (h->d_scalar) return SPX_OK;
-    return dalloc(h, &h->d_scalar, 4);
+    return dalloc(h, &h->d_scalar, (size_t)spx::logdet_workspace());
 }
 
 // grad workspace of len doubles (host-buffer calls)
@@ -2937,21 +2964,43 @@ spx_status spx_selected_inverse(spx_handle h, void *cuda_stream)
             for (int32_t r = P.pw[q]; r < P.ph[q]; ++r)
                 if (row_task[(size_t)P.prow[q] + r] < 0) return fail(h, SPX_ERR_ARG, "row without an update task");
         if ((st = upload(h, &h->d_row_task, row_task))) return st;
+        std::vector<RowChunk> c128, c64;
+        h->sv128_ptr.assign(P.nlevels + 1, 0);
+        h->sv64_ptr.assign(P.nlevels + 1, 0);
+        h->sv_blocks.assign(P.nlevels, 1);
+        for (int32_t l = 0; l < P.nlevels; ++l) {
+            for (int32_t q = P.level_ptr[l]; q < P.level_ptr[l + 1]; ++q) {
+                const int32_t k = P.level_panels[q], w = P.pw[k], hk = P.ph[k];
+                const bool sl = selinv_slices(P, k);
+                if (sl) h->sv_blocks[l] = std::max(h->sv_blocks[l], (hk - w + 63) / 64);
+                for (int32_t r0 = w; r0 < hk; r0 += sl ? 128 : 64) (sl ? c128 : c64).push_back(RowChunk{k, r0});
+            }
+            h->sv128_ptr[l + 1] = (int64_t)c128.size();
+            h->sv64_ptr[l + 1] = (int64_t)c64.size();
+        }
+        if ((st = upload(h, &h->d_sv128, c128)) || (st = upload(h, &h->d_sv64, c64)) ||
+            (st = dalloc(h, &h->d_dexp, (size_t)P.n)) || (st = ensure_colmaps(h)))
+            return st;
     }
     fence_from(h, cuda_stream);
     const int wmax = *std::max_element(h->lvl_wmax.begin(), h->lvl_wmax.end());
     if (wmax > 64) return fail(h, SPX_ERR_ARG, "the selected inverse takes panels up to 64 wide (max_width <= 64)");
     CU(cudaMemcpyAsync(h->d_Lh, h->d_L, elems * sizeof(double), cudaMemcpyDeviceToDevice, h->hs));
     CU(cudaMemsetAsync(h->d_Zsel, 0, elems * sizeof(double), h->hs));   // split-K partial sums add into it
-    spx::launch_trsm<double>(h->dp, h->d_chunks, (int)h->chunk_ptr[P.nlevels], wmax,
-                             (const double *)h->d_Dinv, h->d_Lh, spx::TRSM_RIGHT_LINV, nullptr, nullptr, 0, 0,
-                             h->hs);
+    CU(cudaMemsetAsync(h->d_tcerr, 0, sizeof(int), h->hs));
+    spx::launch_diag_exp(h->dp, (const double *)h->d_L, h->d_dexp, h->hs);
+    // (h->d_chunks: 64 rows each, as the slices TRSM takes them)
+    spx::launch_trsm_sl(h->dp, h->d_chunks, (int)h->chunk_ptr[P.nlevels], (const double *)h->d_Dinv, h->d_Lh, nullptr,
+                        spx::TRSM_RIGHT_LINV, nullptr, nullptr, nullptr, nullptr, 0, 0, h->d_tcerr, h->hs);
+    spx::launch_selinv_diag(h->dp, h->d_level_panels, P.npanels, 1, wmax, 1, (const double *)h->d_Dinv, h->d_Lh,
+                            h->d_Zsel, h->hs);
     // split-K so that a level keeps about two CTAs per SM busy near the root
     int nsm = 0;
     CU(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, h->device));
     const int want = 2 * nsm;
     for (int32_t l = P.nlevels - 1; l >= 0; --l) {
-        const int nch = (int)(h->chunk_ptr[l + 1] - h->chunk_ptr[l]);
+        const int nch = (int)(h->sv64_ptr[l + 1] - h->sv64_ptr[l]);
+        const int n128 = (int)(h->sv128_ptr[l + 1] - h->sv128_ptr[l]);
         const int npl = P.level_ptr[l + 1] - P.level_ptr[l];
         int max_rchunks = 1;   // most 16-row chunks of R in a panel of the level
         for (int32_t q = P.level_ptr[l]; q < P.level_ptr[l + 1]; ++q) {
@@ -2960,13 +3009,34 @@ spx_status spx_selected_inverse(spx_handle h, void *cuda_stream)
         }
         const int so = nch > 0 ? std::min(max_rchunks, std::max(1, (want + nch - 1) / nch)) : 1;
         const int sd = std::min((max_rchunks + 1) / 2, std::max(1, (want + npl - 1) / std::max(npl, 1)));
-        spx::launch_selinv_off(h->dp, h->d_chunks + h->chunk_ptr[l], nch, so, h->d_row_task, h->d_tasks,
-                               h->d_Lh, h->d_Zsel, h->hs);
-        spx::launch_selinv_diag(h->dp, h->d_level_panels + P.level_ptr[l], npl, sd, h->lvl_wmax[l],
-                                (const double *)h->d_Dinv, h->d_Lh, h->d_Zsel, h->hs);
+        // slices, one CTA an SM: the number of parts that makes the most loaded
+        // SM's 64-column blocks (and half a block's time to start and end a part)
+        // fewest
+        int s128 = 1;
+        double best = 1e300;
+        for (int c = 1; c <= std::min(h->sv_blocks[l], 32); ++c) {
+            const double t = std::ceil((double)n128 * c / nsm) * ((h->sv_blocks[l] + c - 1) / c + 0.5);
+            if (t < best) best = t, s128 = c;
+        }
+        spx::launch_selinv_sl(h->dp, h->d_sv128 + h->sv128_ptr[l], n128, s128, h->d_colbase, h->d_relbase, h->d_dexp,
+                              h->d_Lh, h->d_Zsel, h->d_tcerr, h->hs);
+        spx::launch_selinv_off(h->dp, h->d_sv64 + h->sv64_ptr[l], nch, so, h->d_row_task, h->d_tasks, h->d_Lh,
+                               h->d_Zsel, h->hs);
+        // the diagonal blocks by slices where a level has few panels (one CTA an SM
+        // takes as long as the FP64 unit does for 20 rows of a 64-wide panel)
+        if (npl <= nsm && h->lvl_wmax[l] > 32)
+            spx::launch_selinv_diag_sl(h->dp, h->d_level_panels + P.level_ptr[l], npl,
+                                       std::min((max_rchunks + 3) / 4, std::max(1, nsm / npl)), h->d_dexp, h->d_Lh,
+                                       h->d_Zsel, h->d_tcerr, h->hs);
+        else
+            spx::launch_selinv_diag(h->dp, h->d_level_panels + P.level_ptr[l], npl, sd, h->lvl_wmax[l], 2,
+                                    (const double *)h->d_Dinv, h->d_Lh, h->d_Zsel, h->hs);
     }
     CU(cudaGetLastError());
+    int tcerr = 0;
+    CU(cudaMemcpyAsync(&tcerr, h->d_tcerr, sizeof(int), cudaMemcpyDeviceToHost, h->hs));
     CU(cudaStreamSynchronize(h->hs));
+    if (tcerr) return fail(h, SPX_ERR_TIMEOUT, "a tensor-core tile of the selected inversion gave up waiting");
     h->zready = true;
     return SPX_OK;
 }

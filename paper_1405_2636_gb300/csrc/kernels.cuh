@@ -138,8 +138,18 @@ void launch_update_sl(const void *mapa, const void *mapb, int64_t oprows, const 
                       int wmax, cudaStream_t s);
 // chunks: 64 rows each.  LDL^T: opa / expa hold L, opb / expb D L^T.
 void launch_trsm_sl(const DevPlan &p, const RowChunk *chunks, int count, const double *Dinv, double *X, double *Wout,
-                    int ldlt, void *opa, void *opb, int32_t *expa, int32_t *expb, int64_t oprows, int kpad, int *err,
+                    int mode, void *opa, void *opb, int32_t *expa, int32_t *expb, int64_t oprows, int kpad, int *err,
                     cudaStream_t s);
+// Selected inversion's Z_RJ (update_sl.cu): chunks of 128 rows; colbase,
+// relbase: where each off-diagonal row's column lies, as in launch_update_sl;
+// dexp: leading exponents of L's diagonal by column (launch_diag_exp).
+void launch_selinv_sl(const DevPlan &p, const RowChunk *chunks, int count, int nsplit, const int64_t *colbase,
+                      const int64_t *relbase, const int32_t *dexp, const double *Lh, double *Z, int *err,
+                      cudaStream_t s);
+// Z_JJ -= Lh^T Z_RJ of a few panels (nsplit parts of R each)
+void launch_selinv_diag_sl(const DevPlan &p, const int32_t *panels, int count, int nsplit, const int32_t *dexp,
+                           const double *Lh, double *Z, int *err, cudaStream_t s);
+void launch_diag_exp(const DevPlan &p, const double *L, int32_t *dexp, cudaStream_t s);
 // Tasks of few multiply-adds, one warp each.
 void launch_update_small(const DevPlan &p, const DevTask *tasks, const int32_t *ids, int count, const double *Aop,
                          const double *Bop, double *C, cudaStream_t s);
@@ -269,8 +279,11 @@ void launch_axpy_cols(int64_t n, int nrhs, const double *D, double *X, int64_t l
 void launch_selinv_off(const DevPlan &p, const RowChunk *chunks, int count, int nsplit,
                        const int32_t *row_task, const DevTask *tasks, const double *Lh, double *Z,
                        cudaStream_t s);
-void launch_selinv_diag(const DevPlan &p, const int32_t *panels, int count, int nsplit, int wmax,
+// what: 1 Linv^T Linv (stored), 2 - Lh^T Z_RJ (added to it)
+void launch_selinv_diag(const DevPlan &p, const int32_t *panels, int count, int nsplit, int wmax, int what,
                         const double *Dinv, const double *Lh, double *Z, cudaStream_t s);
+// out: logdet_workspace() doubles, the result first
+int logdet_workspace();
 template <typename T>
 void launch_logdet(const DevPlan &p, const T *L, double *out, cudaStream_t s);
 void launch_gather(int64_t nnz, const int64_t *zmap, const double *Z, double *grad, cudaStream_t s);

@@ -126,12 +126,16 @@ __global__ void __launch_bounds__(256) selinv_off_kernel(DevPlan p, const RowChu
 
 // ---------------------------------------------------------------------------
 // Z_JJ = Linv^T Linv - Lh^T Z_RJ for one panel (w <= 64), lower pairs (a, b)
-// computed once and written to both triangles.  Split-K as above: gridDim.y
-// CTAs per panel take every gridDim.y-th chunk of 32 rows of R.
+// computed once and written to both triangles, in two launches: Linv^T Linv of
+// every panel at once before the walk down the tree (what = 1; it needs no
+// other panel, and inside the walk it took 20 us of every level), then, where
+// the slices form (update_sl.cu) does not take it, the rest per level (what =
+// 2; split-K as above: gridDim.y CTAs per panel take every gridDim.y-th chunk
+// of 32 rows of R).
 // ---------------------------------------------------------------------------
 constexpr int kSelDiagPairs = 9;   // ceil(64 * 65 / 2 / 256)
 
-__global__ void __launch_bounds__(256) selinv_diag_kernel(DevPlan p, const int32_t *__restrict__ panels,
+__global__ void __launch_bounds__(256) selinv_diag_kernel(DevPlan p, const int32_t *__restrict__ panels, int what,
                                                           const double *__restrict__ Dinv,
                                                           const double *__restrict__ Lh,
                                                           double *__restrict__ Z)
@@ -146,7 +150,8 @@ __global__ void __launch_bounds__(256) selinv_diag_kernel(DevPlan p, const int32
     const double *Mi = Dinv + p.pinv[pid];
     const int tid = threadIdx.x;
     const int sp = blockIdx.y, ns = gridDim.y;   // this CTA takes every ns-th chunk of 32 rows
-    for (int e = tid; e < w * w; e += 256) Di[e] = Mi[e];
+    if (what == 1)
+        for (int e = tid; e < w * w; e += 256) Di[e] = Mi[e];
     const int npair = w * (w + 1) / 2;
     int pa[kSelDiagPairs], pb[kSelDiagPairs];
     double acc[kSelDiagPairs];
@@ -163,14 +168,14 @@ __global__ void __launch_bounds__(256) selinv_diag_kernel(DevPlan p, const int32
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < kSelDiagPairs; ++q) {
-        if (tid + 256 * q >= npair || sp != 0) continue;
+        if (tid + 256 * q >= npair || what != 1) continue;
         const int a = pa[q], b = pb[q];   // a >= b: Linv(k, a) Linv(k, b) is nonzero for k >= a
         double s = 0.0;
 #pragma unroll 1
         for (int k = a; k < w; ++k) s = fma(Di[k + a * w], Di[k + b * w], s);
         acc[q] = s;
     }
-    for (int c0 = w + 32 * sp; c0 < h; c0 += 32 * ns) {
+    for (int c0 = what == 1 ? h : w + 32 * sp; c0 < h; c0 += 32 * ns) {
         const int m = min(32, h - c0);
         __syncthreads();
         for (int e = tid; e < 32 * w; e += 256) {
@@ -197,10 +202,10 @@ __global__ void __launch_bounds__(256) selinv_diag_kernel(DevPlan p, const int32
     for (int q = 0; q < kSelDiagPairs; ++q) {
         if (tid + 256 * q >= npair) continue;
         const int a = pa[q], b = pb[q];
-        if (ns == 1) {
+        if (what == 1) {
             Z[base + a + (int64_t)b * h] = acc[q];
             Z[base + b + (int64_t)a * h] = acc[q];
-        } else {   // partial sums over row chunks; Z starts zeroed
+        } else {
             atomicAdd(&Z[base + a + (int64_t)b * h], acc[q]);
             if (a != b) atomicAdd(&Z[base + b + (int64_t)a * h], acc[q]);
         }
@@ -215,7 +220,7 @@ void launch_selinv_off(const DevPlan &p, const RowChunk *chunks, int count, int 
     selinv_off_kernel<<<dim3(count, nsplit), 256, 0, s>>>(p, chunks, row_task, tasks, Lh, Z);
 }
 
-void launch_selinv_diag(const DevPlan &p, const int32_t *panels, int count, int nsplit, int wmax,
+void launch_selinv_diag(const DevPlan &p, const int32_t *panels, int count, int nsplit, int wmax, int what,
                         const double *Dinv, const double *Lh, double *Z, cudaStream_t s)
 {
     if (count <= 0) return;
@@ -226,14 +231,16 @@ void launch_selinv_diag(const DevPlan &p, const int32_t *panels, int count, int 
                              (int)(sizeof(double) * (64 * 64 + 64 * 64)));
         once = true;
     }
-    selinv_diag_kernel<<<dim3(count, nsplit), 256, smem, s>>>(p, panels, Dinv, Lh, Z);
+    selinv_diag_kernel<<<dim3(count, nsplit), 256, smem, s>>>(p, panels, what, Dinv, Lh, Z);
 }
 
 // ---------------------------------------------------------------------------
-// log det A = 2 sum_j log L(j, j): one block, panels by thread, FP64 sum
-// with error compensation (Knuth's two-sum on every addition, the error
-// terms summed apart), so that the result is accurate to about one unit of
-// the last place of the total rather than n of them.
+// log det A = 2 sum_j log L(j, j): panels by thread over up to 64 blocks (one
+// block's FP64 unit took 2 ms for 110,592 logarithms), FP64 sum with error
+// compensation (Knuth's two-sum on every addition, the error terms summed
+// apart), so that the result is accurate to about one unit of the last place
+// of the total rather than n of them; the blocks' pairs are added up the same
+// way by the last block to finish.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void two_sum(double a, double b, double &s, double &e)
 {
@@ -242,12 +249,31 @@ __device__ __forceinline__ void two_sum(double a, double b, double &s, double &e
     e = (a - (s - bb)) + (b - bb);
 }
 
-template <typename T>
-__global__ void __launch_bounds__(1024) logdet_kernel(DevPlan p, const T *__restrict__ L, double *out)
+// (s, c) + the pair of lane ^ o, for all o: every lane ends with the warp's sum.
+__device__ __forceinline__ void warp_pair_sum(double &s, double &c)
 {
-    __shared__ double red[64];
+    for (int o = 16; o > 0; o >>= 1) {
+        double t, e;
+        two_sum(s, __shfl_xor_sync(0xffffffffu, s, o), t, e);
+        c += e + __shfl_xor_sync(0xffffffffu, c, o);
+        s = t;
+    }
+}
+
+constexpr int kLogdetBlocks = 64, kLogdetThreads = 256;
+
+// out[0]: the result; then per block (sum, error), and a block counter (zeroed
+// beforehand) behind them.
+template <typename T>
+__global__ void __launch_bounds__(kLogdetThreads) logdet_kernel(DevPlan p, const T *__restrict__ L, double *out)
+{
+    __shared__ double red[2][kLogdetThreads / 32];
+    __shared__ bool s_last;
+    double *part = out + 1;
+    unsigned *count = reinterpret_cast<unsigned *>(part + 2 * kLogdetBlocks);
+    const int tid = threadIdx.x;
     double s = 0.0, c = 0.0;
-    for (int pid = threadIdx.x; pid < p.npanels; pid += blockDim.x) {
+    for (int pid = blockIdx.x + gridDim.x * tid; pid < p.npanels; pid += gridDim.x * kLogdetThreads) {
         const int w = p.pw[pid], h = p.ph[pid];
         const T *D = L + p.pval[pid];
         for (int k = 0; k < w; ++k) {
@@ -257,35 +283,44 @@ __global__ void __launch_bounds__(1024) logdet_kernel(DevPlan p, const T *__rest
             c += e;
         }
     }
-    for (int o = 16; o > 0; o >>= 1) {
-        double t, e;
-        two_sum(s, __shfl_xor_sync(0xffffffffu, s, o), t, e);
-        c += e + __shfl_xor_sync(0xffffffffu, c, o);
-        s = t;
-    }
-    if ((threadIdx.x & 31) == 0) {
-        red[threadIdx.x >> 5] = s;
-        red[32 + (threadIdx.x >> 5)] = c;
+    warp_pair_sum(s, c);
+    if ((tid & 31) == 0) {
+        red[0][tid >> 5] = s;
+        red[1][tid >> 5] = c;
     }
     __syncthreads();
-    if (threadIdx.x < 32) {
-        const bool has = threadIdx.x < (blockDim.x >> 5);
-        s = has ? red[threadIdx.x] : 0.0;
-        c = has ? red[32 + threadIdx.x] : 0.0;
-        for (int o = 16; o > 0; o >>= 1) {
-            double t, e;
-            two_sum(s, __shfl_xor_sync(0xffffffffu, s, o), t, e);
-            c += e + __shfl_xor_sync(0xffffffffu, c, o);
-            s = t;
+    if (tid < 32) {
+        s = tid < kLogdetThreads / 32 ? red[0][tid] : 0.0;
+        c = tid < kLogdetThreads / 32 ? red[1][tid] : 0.0;
+        warp_pair_sum(s, c);
+        if (tid == 0) {
+            part[2 * blockIdx.x] = s;
+            part[2 * blockIdx.x + 1] = c;
+            __threadfence();
+            s_last = atomicAdd(count, 1u) == gridDim.x - 1;
         }
-        if (threadIdx.x == 0) *out = 2.0 * (s + c);
     }
+    __syncthreads();
+    if (!s_last || tid >= 32) return;
+    __threadfence();
+    s = c = 0.0;
+    for (int b = tid; b < (int)gridDim.x; b += 32) {
+        double t, e;
+        two_sum(s, __ldcg(part + 2 * b), t, e);
+        s = t;
+        c += e + __ldcg(part + 2 * b + 1);
+    }
+    warp_pair_sum(s, c);
+    if (tid == 0) *out = 2.0 * (s + c);
 }
+
+int logdet_workspace() { return 2 * kLogdetBlocks + 2; }
 
 template <typename T>
 void launch_logdet(const DevPlan &p, const T *L, double *out, cudaStream_t s)
 {
-    logdet_kernel<T><<<1, 1024, 0, s>>>(p, L, out);
+    cudaMemsetAsync(out + 1 + 2 * kLogdetBlocks, 0, sizeof(double), s);
+    logdet_kernel<T><<<kLogdetBlocks, kLogdetThreads, 0, s>>>(p, L, out);
 }
 template void launch_logdet<double>(const DevPlan &, const double *, double *, cudaStream_t);
 template void launch_logdet<float>(const DevPlan &, const float *, double *, cudaStream_t);

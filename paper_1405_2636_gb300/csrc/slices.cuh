@@ -71,10 +71,12 @@ __device__ __forceinline__ long long fixed_biased(double x, int field, int scale
     const int ef = (int)((b >> 52) & 0x7FF);
     long long m = b & 0xFFFFFFFFFFFFFLL;
     if (ef > 0) m |= 0x10000000000000LL;
-    const int sh = (ef > 0 ? ef : 1) + scale - field + 4;   // <= 4 (x != 0)
-    if (sh >= 0) m <<= min(sh, 4);
-    else m = sh < -56 ? 0 : (m + (1LL << (-sh - 1))) >> -sh;
-    return (b < 0 ? -m : m) + 0x808080808080LL;
+    // m 2^(ef + scale - field + 4), at most 2^57: shifted with one bit to spare,
+    // then rounded to nearest (ties away from zero)
+    const int n = min(max(field - scale - (ef > 0 ? ef : 1), 0), 63);
+    const long long f = (long long)((((unsigned long long)m << 5) >> n) + 1) >> 1;
+    const long long sign = b >> 63;
+    return (f ^ sign) - sign + 0x808080808080LL;
 }
 
 // The seven digits of two numbers (fixed_biased), as half2 words.

@@ -276,7 +276,8 @@ __global__ void __launch_bounds__(kSlThreads, 1)
 
 // ---------------------------------------------------------------------------
 // Panel TRSM in FP64 as a product with the inverted diagonal block (the forms
-// TRSM_LLT and TRSM_LDLT of blocks.cuh), 64 rows a CTA: X's rows and the
+// TRSM_LLT, TRSM_LDLT and, for panels up to 64 wide and without the operand
+// copy, TRSM_RIGHT_LINV of blocks.cuh), 64 rows a CTA: X's rows and the
 // inverse's rows are cut into slices in shared memory, the 28 digit pairs run
 // on the tensor cores, the result is put together as in the update, written
 // back in place and written again as slices for the updates.  Each row lies
@@ -314,9 +315,33 @@ __device__ __forceinline__ void digits8(const double *x, int field, uint32_t (&w
     }
 }
 
+// One thread: all digit pairs of an A tile (slices of kABytes) and a B tile
+// (kBBytes), n columns, group g into accumulator g; done[g] completes with
+// group g, the last first.
+__device__ __forceinline__ void issue_pairs(uint32_t tmem, const unsigned char *sA, const unsigned char *sB, int n,
+                                            int ksteps, uint64_t *done)
+{
+    const uint32_t idesc = idesc_f16(n);
+    const uint64_t a0 = sw128_desc(smem_u32(sA)), b0 = sw128_desc(smem_u32(sB));
+#pragma unroll 1
+    for (int g = kGroups - 1; g >= 0; --g) {
+        const uint32_t acc = tmem + (uint32_t)(g * kBN);
+#pragma unroll 1
+        for (int s = 0; s <= g; ++s) {
+            const uint64_t da = a0 + (uint32_t)(s * (kABytes >> 4));
+            const uint64_t db = b0 + (uint32_t)((g - s) * (kBBytes >> 4));
+            mma<1>(acc, da, db, idesc, s > 0);
+            if (ksteps > 1) mma<1>(acc, da + 2, db + 2, idesc, 1);
+            if (ksteps > 2) mma<1>(acc, da + 4, db + 4, idesc, 1);
+            if (ksteps > 3) mma<1>(acc, da + 6, db + 6, idesc, 1);
+        }
+        mma_commit(&done[g]);
+    }
+}
+
 __global__ void __launch_bounds__(kTrThreads, 1)
     trsm_sl_kernel(DevPlan p, const RowChunk *__restrict__ chunks, const double *__restrict__ Dinv,
-                   double *__restrict__ X, double *__restrict__ Wout, int ldlt, __half *__restrict__ opa,
+                   double *__restrict__ X, double *__restrict__ Wout, int mode, __half *__restrict__ opa,
                    __half *__restrict__ opb, int32_t *__restrict__ expa, int32_t *__restrict__ expb, int64_t oprows,
                    int kpad, int *err)
 {
@@ -331,6 +356,7 @@ __global__ void __launch_bounds__(kTrThreads, 1)
     __shared__ int32_t s_e[2][kTrRows];
     __shared__ int s_sc[kK];
     const RowChunk ch = chunks[blockIdx.x];
+    const bool ldlt = mode == TRSM_LDLT, right = mode == TRSM_RIGHT_LINV;
     const int pid = ch.panel, w = p.pw[pid], h = p.ph[pid];
     const int nr = min(kTrRows, h - ch.r0);
     double *Xg = X + p.pval[pid] + ch.r0;
@@ -366,7 +392,7 @@ __global__ void __launch_bounds__(kTrThreads, 1)
             if (tid < kK) {
                 const int k = k0 + tid;
                 const int e = k < w ? ((__double2hiint(__ldcg(Mi + k + (int64_t)k * w)) >> 20) & 0x7FF) - 1023 : 0;
-                s_sc[tid] = (e < -1022 || e > 1023) ? 0 : (ldlt ? e >> 1 : e);
+                s_sc[tid] = (right || e < -1022 || e > 1023) ? 0 : (ldlt ? e >> 1 : e);
             }
             __syncthreads();
             // operand 0: X(rs, k0 ..), operand 1: the inverse's row c0 + rs
@@ -374,12 +400,17 @@ __global__ void __launch_bounds__(kTrThreads, 1)
 #pragma unroll 1
             for (int o = 0; o < 2; ++o) {
                 const int j = c0 + rs, k1 = k0 + kTC * ps;
-                const double *src = o == 0 ? Xg + rs + (int64_t)k1 * h : Mi + j + (int64_t)k1 * w;
-                const int64_t ld = o == 0 ? h : w;
-                const int klim = o == 0 ? (rs < nr ? w : 0) : (j < w ? j + 1 : 0);   // columns below it are read
+                const double *src = o == 0  ? Xg + rs + (int64_t)k1 * h
+                                    : right ? Mi + k1 + (int64_t)j * w    // L^{-1}: B(k, j) = Linv(k, j)
+                                            : Mi + j + (int64_t)k1 * w;
+                const int64_t ld = o == 0 ? h : (right ? 1 : w);
+                // columns read: k < klim and, for L^{-1}, k >= j
+                const int klim = o == 0 ? (rs < nr ? w : 0) : (j < w ? (right ? w : j + 1) : 0);
+                const int kmin = o == 1 && right ? j : 0;
                 double x[kTC];
 #pragma unroll
-                for (int q = 0; q < kTC; ++q) x[q] = k1 + q < klim ? __ldcg(src + q * ld) : 0.0;
+                for (int q = 0; q < kTC; ++q)
+                    x[q] = k1 + q < klim && k1 + q >= kmin ? __ldcg(src + q * ld) : 0.0;
                 if (o == 1 && ldlt) {   // unit diagonal (1/d is stored there)
 #pragma unroll
                     for (int q = 0; q < kTC; ++q)
@@ -414,24 +445,7 @@ __global__ void __launch_bounds__(kTrThreads, 1)
             __syncthreads();
             if (warp == 0) {
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                if (elect_one()) {
-                    const uint32_t idesc = idesc_f16(kBN);
-                    const uint64_t a0 = sw128_desc(smem_u32(sA)), b0 = sw128_desc(smem_u32(sB));
-#pragma unroll 1
-                    for (int g = kGroups - 1; g >= 0; --g) {
-                        const uint32_t acc = tmem + (uint32_t)(g * kBN);
-#pragma unroll 1
-                        for (int s = 0; s <= g; ++s) {
-                            const uint64_t da = a0 + (uint32_t)(s * (kABytes >> 4));
-                            const uint64_t db = b0 + (uint32_t)((g - s) * (kBBytes >> 4));
-                            mma<1>(acc, da, db, idesc, s > 0);
-                            if (ksteps > 1) mma<1>(acc, da + 2, db + 2, idesc, 1);
-                            if (ksteps > 2) mma<1>(acc, da + 4, db + 4, idesc, 1);
-                            if (ksteps > 3) mma<1>(acc, da + 6, db + 6, idesc, 1);
-                        }
-                        mma_commit(&done[g]);
-                    }
-                }
+                if (elect_one()) issue_pairs(tmem, sA, sB, kBN, ksteps, done);
                 __syncwarp();
             }
             Sum sum[kTC];
@@ -484,6 +498,7 @@ __global__ void __launch_bounds__(kTrThreads, 1)
                 else if (row_ok) dst[(int64_t)q * h] = out[q];
                 f = max(f, exp_field(out[q]));
             }
+            if (right) continue;   // no operand copy
             s_f[0][part][r] = f;
             __syncthreads();
 #pragma unroll
@@ -507,6 +522,339 @@ __global__ void __launch_bounds__(kTrThreads, 1)
     if (tid == 0 && s_fail) atomicExch(err, 1);
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kSlCols));
+}
+
+// ---------------------------------------------------------------------------
+// Selected inversion, Z_RJ = -Z_RR Lh for 128 rows i of one panel (selinv.cu
+// says what the quantities are): per 64 columns j of Z_RR the gathered 128 x 64
+// block of Z and the 64 x w block of Lh are cut into slices, multiplied, and the
+// product is added in FP64 to the running result.  Z(i, j) lies in the column
+// of the lower of the two rows: at colbase[j] + relmap[relbase[j] + i] for
+// i >= j.  Column j of Z is scaled by the leading power of two of L(j, j) and
+// row j of Lh by its inverse (see the TRSM).  The next block's entries of Z are
+// loaded before this block's sums are drained.  Split over j as in the CUDA-core
+// form (gridDim.y parts, added into a zeroed Z).
+// Bound by the integer work (about 68 instructions an entry of Z, 72 a result
+// and block); the FP64 unit would take 300,000 cycles for a block that this
+// does in about 15,000.
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(kTrThreads, 1)
+    selinv_sl_kernel(DevPlan p, const RowChunk *__restrict__ chunks, const int64_t *__restrict__ colbase,
+                     const int64_t *__restrict__ relbase, const int32_t *__restrict__ dexp,
+                     const double *__restrict__ Lh, double *__restrict__ Z, int *err)
+{
+    extern __shared__ unsigned char smraw[];
+    unsigned char *base =
+        reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~(uintptr_t)1023);
+    unsigned char *sA = base, *sB = base + kSlices * kABytes;
+    __shared__ __align__(8) uint64_t done[kSlices];
+    __shared__ uint32_t s_tmem;
+    __shared__ int s_fail;
+    __shared__ int s_f[4][kM], s_g[8][kBN];
+    __shared__ int32_t s_eb[kBN];
+    __shared__ int s_sc[2][kK];                        // this block's column scales, and the next one's
+    __shared__ int64_t s_cb[2][kK], s_rb[2][kK];
+    constexpr int kQ = kK / (kTrThreads / kM);         // 16 entries of one row of Z a thread
+    const RowChunk ch = chunks[blockIdx.x];
+    const int pid = ch.panel, w = p.pw[pid], h = p.ph[pid];
+    const int nk = (h - w + kK - 1) / kK, per = (nk + (int)gridDim.y - 1) / (int)gridDim.y;
+    const int b0 = min(nk, (int)blockIdx.y * per), b1 = min(nk, b0 + per);
+    if (b0 >= b1) return;
+    const int64_t prow = p.prow[pid];
+    const int tid = threadIdx.x, warp = tid >> 5;
+
+    if (tid == 0) {
+        for (int g = 0; g < kSlices; ++g) mbar_init(&done[g], 1);
+        s_fail = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
+                     "r"(kSlCols));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    const int r = tid & (kM - 1), part = tid / kM, i = ch.r0 + r;
+    const bool row_ok = i < h;
+    const int64_t cbi = row_ok ? colbase[prow + i] : 0, rbi = row_ok ? relbase[prow + i] + prow : 0;
+    auto columns = [&](int b) {                        // the 64 columns of block b
+        if (tid < kK) {
+            const int j = w + b * kK + tid;
+            const bool in = j < h;
+            s_cb[b & 1][tid] = in ? colbase[prow + j] : 0;
+            s_rb[b & 1][tid] = in ? relbase[prow + j] + prow : 0;
+            s_sc[b & 1][tid] = in ? dexp[p.rows[prow + j]] : 0;
+        }
+    };
+    double x[kQ];
+    auto gather = [&](int b) {
+#pragma unroll
+        for (int q = 0; q < kQ; ++q) {
+            const int k = kQ * part + q, j = w + b * kK + k;
+            double v = 0.0;
+            if (row_ok && j < h)
+                v = i >= j ? Z[s_cb[b & 1][k] + p.relmap[s_rb[b & 1][k] + i]] : Z[cbi + p.relmap[rbi + j]];
+            x[q] = v;
+        }
+    };
+    columns(b0);
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = s_tmem;
+    const uint32_t tlane = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+    gather(b0);
+    double acc[kQ];
+#pragma unroll
+    for (int q = 0; q < kQ; ++q) acc[q] = 0.0;
+    uint32_t phase = 0;
+    for (int b = b0; b < b1; ++b) {
+        const int j0 = w + b * kK, ksteps = (min(kK, h - j0) + 15) / 16;
+        int32_t ea;
+        {
+            int sc[kQ], f = kFieldZero;
+#pragma unroll
+            for (int q = 0; q < kQ; ++q) sc[q] = s_sc[b & 1][kQ * part + q];
+#pragma unroll
+            for (int q = 0; q < kQ; ++q) f = max(f, exp_field(x[q], sc[q]));
+            s_f[part][r] = f;
+            __syncthreads();
+            f = max(max(s_f[0][r], s_f[1][r]), max(s_f[2][r], s_f[3][r]));
+            ea = row_exp(f);
+            if (part < ksteps) {
+#pragma unroll 1
+                for (int q8 = 0; q8 < kQ; q8 += 8) {
+                    uint32_t wd[kSlices][4];
+                    if (q8 == 0) digits8(x, f, wd, sc);
+                    else digits8(x + 8, f, wd, sc + 8);
+                    unsigned char *t = sA + r * kRowBytes + (((kQ * part + q8) * 2) ^ ((r & 7) << 4));
+#pragma unroll
+                    for (int s = 0; s < kSlices; ++s)
+                        *reinterpret_cast<uint4 *>(t + s * kABytes) = make_uint4(wd[s][0], wd[s][1], wd[s][2], wd[s][3]);
+                }
+            }
+        }
+        {
+            const int c = tid & 63, pb = tid >> 6;     // eight entries of Lh's column c
+            double y[8];
+            int sc[8], f = kFieldZero;
+            const double *src = Lh + p.pval[pid] + (int64_t)c * h + j0 + 8 * pb;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                sc[q] = -s_sc[b & 1][8 * pb + q];
+                y[q] = c < w && j0 + 8 * pb + q < h ? src[q] : 0.0;
+            }
+#pragma unroll
+            for (int q = 0; q < 8; ++q) f = max(f, exp_field(y[q], sc[q]));
+            s_g[pb][c] = f;
+            __syncthreads();
+#pragma unroll
+            for (int q = 0; q < 8; ++q) f = max(f, s_g[q][c]);
+            if (pb == 0) s_eb[c] = row_exp(f);
+            if (8 * pb < 16 * ksteps) {
+                uint32_t wd[kSlices][4];
+                digits8(y, f, wd, sc);
+                unsigned char *t = sB + c * kRowBytes + ((16 * pb) ^ ((c & 7) << 4));
+#pragma unroll
+                for (int s = 0; s < kSlices; ++s)
+                    *reinterpret_cast<uint4 *>(t + s * kBBytes) = make_uint4(wd[s][0], wd[s][1], wd[s][2], wd[s][3]);
+            }
+        }
+        if (b + 1 < b1) columns(b + 1);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncthreads();
+        if (warp == 0) {
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            if (elect_one()) issue_pairs(tmem, sA, sB, (w + 15) & ~15, ksteps, done);
+            __syncwarp();
+        }
+        if (b + 1 < b1) gather(b + 1);
+        // eight columns at a time (registers); columns past w hold stale sums
+        if (kQ * part < w) {
+#pragma unroll
+            for (int q8 = 0; q8 < kQ; q8 += 8) {
+                Sum sum[8];
+                auto drain = [&](auto gc) {
+                    constexpr int G = decltype(gc)::value;
+                    if (!mbar_wait(&done[G], phase)) s_fail = 1;
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    uint32_t v[8];
+                    tmem_read8(tlane + (uint32_t)(G * kBN + kQ * part + q8), v);
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) add_group<G>(sum[q], __uint_as_float(v[q]));
+                };
+                drain(std::integral_constant<int, 6>());
+                drain(std::integral_constant<int, 5>());
+                drain(std::integral_constant<int, 4>());
+                drain(std::integral_constant<int, 3>());
+                drain(std::integral_constant<int, 2>());
+                drain(std::integral_constant<int, 1>());
+                drain(std::integral_constant<int, 0>());
+#pragma unroll
+                for (int q = 0; q < 8; ++q)
+                    acc[q8 + q] += finish(sum[q], ea + s_eb[kQ * part + q8 + q], true);
+            }
+        }
+        // (a warp without columns still has to see the block's last product done)
+        if (!mbar_wait(&done[0], phase)) s_fail = 1;
+        phase ^= 1u;
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncthreads();
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        if (s_fail) break;
+    }
+    if (row_ok && !s_fail) {
+        double *dst = Z + p.pval[pid] + i;
+#pragma unroll
+        for (int q = 0; q < kQ; ++q) {
+            const int c = kQ * part + q;
+            if (c >= w) continue;
+            if (gridDim.y == 1) dst[(int64_t)c * h] = acc[q];
+            else atomicAdd(dst + (int64_t)c * h, acc[q]);
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (tid == 0 && s_fail) atomicExch(err, 1);
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kSlCols));
+}
+
+// Z_JJ -= Lh^T Z_RJ over the 64-row blocks blockIdx.y, blockIdx.y + gridDim.y,
+// ... of R: both operands are columns of 64 rows cut into slices; Lh's lie
+// twice in the A tile, as X does in the TRSM.  The lower triangle is kept and
+// added to both triangles of Z_JJ, which holds Linv^T Linv.
+__global__ void __launch_bounds__(kTrThreads, 1)
+    selinv_diag_sl_kernel(DevPlan p, const int32_t *__restrict__ panels, const int32_t *__restrict__ dexp,
+                          const double *__restrict__ Lh, double *__restrict__ Z, int *err)
+{
+    extern __shared__ unsigned char smraw[];
+    unsigned char *base =
+        reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~(uintptr_t)1023);
+    unsigned char *sA = base, *sB = base + kSlices * kABytes;
+    __shared__ __align__(8) uint64_t done[kSlices];
+    __shared__ uint32_t s_tmem;
+    __shared__ int s_fail;
+    __shared__ int s_f[2][8][kTrRows];
+    __shared__ int32_t s_e[2][kTrRows];
+    const int pid = panels[blockIdx.x], w = p.pw[pid], h = p.ph[pid];
+    const int nk = (h - w + kK - 1) / kK;
+    if ((int)blockIdx.y >= nk) return;
+    const int64_t pv = p.pval[pid];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+
+    if (tid == 0) {
+        for (int g = 0; g < kSlices; ++g) mbar_init(&done[g], 1);
+        s_fail = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&s_tmem)),
+                     "r"(kSlCols));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = s_tmem;
+    const int cs = tid & (kTrRows - 1), ps = tid / kTrRows;          // staging: column and 8-row part
+    const int quad = warp & 3;
+    const int a = 32 * (quad & 1) + lane, part = 4 * (quad >> 1) + (warp >> 2);
+    double acc[kTC];
+#pragma unroll
+    for (int q = 0; q < kTC; ++q) acc[q] = 0.0;
+    uint32_t phase = 0;
+    for (int b = blockIdx.y; b < nk; b += gridDim.y) {
+        const int j0 = w + b * kK + kTC * ps, ksteps = (min(kK, h - w - b * kK) + 15) / 16;
+#pragma unroll 1
+        for (int o = 0; o < 2; ++o) {
+            const double *src = (o == 0 ? Lh : Z) + pv + (int64_t)cs * h + j0;
+            double x[kTC];
+            int sc[kTC], f = kFieldZero;
+#pragma unroll
+            for (int q = 0; q < kTC; ++q) {
+                x[q] = cs < w && j0 + q < h ? src[q] : 0.0;
+                sc[q] = j0 + q < h ? dexp[p.rows[p.prow[pid] + j0 + q]] : 0;   // row j of Lh divided, of Z times
+                if (o == 0) sc[q] = -sc[q];
+            }
+#pragma unroll
+            for (int q = 0; q < kTC; ++q) f = max(f, exp_field(x[q], sc[q]));
+            s_f[o][ps][cs] = f;
+            __syncthreads();
+#pragma unroll
+            for (int q = 0; q < 8; ++q) f = max(f, s_f[o][q][cs]);
+            if (ps == 0) s_e[o][cs] = row_exp(f);
+            if (kTC * ps < 16 * ksteps) {
+                uint32_t wd[kSlices][4];
+                digits8(x, f, wd, sc);
+                unsigned char *t = (o == 0 ? sA : sB) + cs * kRowBytes + ((16 * ps) ^ ((cs & 7) << 4));
+                const int step = o == 0 ? kABytes : kBBytes;
+#pragma unroll
+                for (int s = 0; s < kSlices; ++s) {
+                    const uint4 v = make_uint4(wd[s][0], wd[s][1], wd[s][2], wd[s][3]);
+                    *reinterpret_cast<uint4 *>(t + s * step) = v;
+                    if (o == 0) *reinterpret_cast<uint4 *>(t + s * step + kTrRows * kRowBytes) = v;
+                }
+            }
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncthreads();
+        if (warp == 0) {
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            if (elect_one()) issue_pairs(tmem, sA, sB, (w + 15) & ~15, ksteps, done);
+            __syncwarp();
+        }
+        Sum sum[kTC];
+        auto drain = [&](auto gc) {
+            constexpr int G = decltype(gc)::value;
+            if (!mbar_wait(&done[G], phase)) s_fail = 1;
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            uint32_t v[kTC];
+            tmem_read8(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(G * kBN + kTC * part), v);
+#pragma unroll
+            for (int i = 0; i < kTC; ++i) add_group<G>(sum[i], __uint_as_float(v[i]));
+        };
+        drain(std::integral_constant<int, 6>());
+        drain(std::integral_constant<int, 5>());
+        drain(std::integral_constant<int, 4>());
+        drain(std::integral_constant<int, 3>());
+        drain(std::integral_constant<int, 2>());
+        drain(std::integral_constant<int, 1>());
+        drain(std::integral_constant<int, 0>());
+        phase ^= 1u;
+        const int32_t ea = s_e[0][a];
+#pragma unroll
+        for (int q = 0; q < kTC; ++q) acc[q] += finish(sum[q], ea + s_e[1][kTC * part + q], true);
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncthreads();
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        if (s_fail) break;
+    }
+    if (!s_fail && a < w) {
+#pragma unroll
+        for (int q = 0; q < kTC; ++q) {
+            const int c = kTC * part + q;
+            if (c > a) continue;
+            atomicAdd(&Z[pv + a + (int64_t)c * h], acc[q]);
+            if (c < a) atomicAdd(&Z[pv + c + (int64_t)a * h], acc[q]);
+        }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (tid == 0 && s_fail) atomicExch(err, 1);
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kSlCols));
+}
+
+// Leading exponents of L's diagonal, by column.
+__global__ void diag_exp_kernel(DevPlan p, const double *__restrict__ L, int32_t *__restrict__ dexp)
+{
+    for (int q = blockIdx.x; q < p.npanels; q += gridDim.x) {
+        const int w = p.pw[q], h = p.ph[q];
+        for (int k = threadIdx.x; k < w; k += blockDim.x)
+            dexp[p.pfcol[q] + k] = ((__double2hiint(L[p.pval[q] + k + (int64_t)k * h]) >> 20) & 0x7FF) - 1023;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -577,7 +925,7 @@ void launch_update_sl(const void *mapa, const void *mapb, int64_t oprows, const 
 }
 
 void launch_trsm_sl(const DevPlan &p, const RowChunk *chunks, int count, const double *Dinv, double *X, double *Wout,
-                    int ldlt, void *opa, void *opb, int32_t *expa, int32_t *expb, int64_t oprows, int kpad, int *err,
+                    int mode, void *opa, void *opb, int32_t *expa, int32_t *expb, int64_t oprows, int kpad, int *err,
                     cudaStream_t s)
 {
     if (count <= 0) return;
@@ -586,8 +934,38 @@ void launch_trsm_sl(const DevPlan &p, const RowChunk *chunks, int count, const d
         cudaFuncSetAttribute(trsm_sl_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTrSmem);
         once = true;
     }
-    trsm_sl_kernel<<<count, kTrThreads, kTrSmem, s>>>(p, chunks, Dinv, X, Wout, ldlt, (__half *)opa, (__half *)opb,
+    trsm_sl_kernel<<<count, kTrThreads, kTrSmem, s>>>(p, chunks, Dinv, X, Wout, mode, (__half *)opa, (__half *)opb,
                                                       expa, expb, oprows, kpad, err);
+}
+
+void launch_selinv_sl(const DevPlan &p, const RowChunk *chunks, int count, int nsplit, const int64_t *colbase,
+                      const int64_t *relbase, const int32_t *dexp, const double *Lh, double *Z, int *err,
+                      cudaStream_t s)
+{
+    if (count <= 0) return;
+    static bool once = false;
+    if (!once) {
+        cudaFuncSetAttribute(selinv_sl_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTrSmem);
+        once = true;
+    }
+    selinv_sl_kernel<<<dim3(count, nsplit), kTrThreads, kTrSmem, s>>>(p, chunks, colbase, relbase, dexp, Lh, Z, err);
+}
+
+void launch_selinv_diag_sl(const DevPlan &p, const int32_t *panels, int count, int nsplit, const int32_t *dexp,
+                           const double *Lh, double *Z, int *err, cudaStream_t s)
+{
+    if (count <= 0) return;
+    static bool once = false;
+    if (!once) {
+        cudaFuncSetAttribute(selinv_diag_sl_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTrSmem);
+        once = true;
+    }
+    selinv_diag_sl_kernel<<<dim3(count, nsplit), kTrThreads, kTrSmem, s>>>(p, panels, dexp, Lh, Z, err);
+}
+
+void launch_diag_exp(const DevPlan &p, const double *L, int32_t *dexp, cudaStream_t s)
+{
+    if (p.npanels > 0) diag_exp_kernel<<<std::min(p.npanels, 152 * 8), 64, 0, s>>>(p, L, dexp);
 }
 
 void launch_update_small(const DevPlan &p, const DevTask *tasks, const int32_t *ids, int count, const double *Aop,
