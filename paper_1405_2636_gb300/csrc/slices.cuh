@@ -20,9 +20,9 @@
 // omitted groups come to about 2^-56 of the product of the rows' largest
 // entries (digits vary independently), an eighth of FP64's unit roundoff.
 // Measured forward errors of solutions against those with FP64 multiply-adds,
-// root mean square over 10 to 24 systems of a kind: 1.00 (20^3 diffusion),
-// 0.99 (32^3), 1.00 (LDL^T), 1.09 (graph order, 128-wide panels; 1.08 with an
-// eighth group, which costs 34 pairs instead of 28).
+// root mean square over 10 to 24 systems of a kind: 0.84 (20^3 diffusion),
+// 0.87 (32^3), 1.00 (LDL^T), 1.00 (graph order, 128-wide panels; an eighth
+// group, 34 pairs instead of 28, changed nothing).
 //
 // Integers only from the bits of the input to the bits of the result: on
 // this part a conversion to or from a double occupies the FP64 unit.
@@ -72,9 +72,12 @@ __device__ __forceinline__ long long fixed_biased(double x, int field, int scale
     long long m = b & 0xFFFFFFFFFFFFFLL;
     if (ef > 0) m |= 0x10000000000000LL;
     // m 2^(ef + scale - field + 4), at most 2^57: shifted with one bit to spare,
-    // then rounded to nearest (ties away from zero)
+    // then rounded to nearest.  A tie (every other entry that loses one bit) goes
+    // up or down by a bit from the middle of the mantissa: one way for all would
+    // make the products of L's equal-signed entries too large together.
     const int n = min(max(field - scale - (ef > 0 ? ef : 1), 0), 63);
-    const long long f = (long long)((((unsigned long long)m << 5) >> n) + 1) >> 1;
+    const long long M = (m << 5) - ((b >> 40) & 1);
+    const long long f = (long long)(((unsigned long long)M >> n) + 1) >> 1;
     const long long sign = b >> 63;
     return (f ^ sign) - sign + 0x808080808080LL;
 }
