@@ -381,9 +381,7 @@ __device__ void potrf_block(const DevPlan &p, int pid, T *__restrict__ L, T *__r
 }
 
 // Cholesky diagonal blocks wider than 64, one CTA per panel: in fixed point, or
-// where that cannot hold the block, in FP64.  128 wide: 0.54 -> 0.27 ms.
-// (Up to 64 wide the FP64 kernel below is as fast, 70 us in FP64 and 53 in
-// FP32 against 67 and 69.)
+// where that cannot hold the block, in FP64.
 template <typename T>
 __global__ void __launch_bounds__(256) potrf_wide_kernel(DevPlan p, const int32_t *__restrict__ panels,
                                                          T *__restrict__ L, T *__restrict__ Dinv,
@@ -404,6 +402,26 @@ size_t potrf_wide_smem(int wmax)
 {
     return std::max(fx::smem_bytes(std::min(wmax, fx::kMaxW)),
                     sizeof(double) * ((size_t)wmax * wmax + kDB * wmax + kDB * kDB));
+}
+
+// Cholesky diagonal blocks of 33 .. 64 columns: the same way, the block's rows
+// one a lane (64 wide: 67 -> 48 us for an FP64 factor, 51 -> 47 for FP32; up to
+// 32 columns both take the same time, 23 to 26 us, and the smaller kernel
+// stays).  What fixed
+// point cannot hold goes the FP64 way, after the time lost here.
+template <typename T>
+__global__ void __launch_bounds__(256) potrf_mid_kernel(DevPlan p, const int32_t *__restrict__ panels,
+                                                        T *__restrict__ L, T *__restrict__ Dinv,
+                                                        const double *replace_tau_p, int64_t *err_col,
+                                                        unsigned long long *nrepl)
+{
+    extern __shared__ double sm[];
+    const int pid = panels[blockIdx.x];
+    const int w = p.pw[pid], h = p.ph[pid];
+    if (fx::diag_block<T, 1>(L + p.pval[pid], Dinv + p.pinv[pid], w, h, reinterpret_cast<unsigned char *>(sm)))
+        return;
+    __syncthreads();
+    ldl_diag_block<T, 64, false>(p, pid, L, Dinv, *replace_tau_p, err_col, nrepl, nullptr, sm);
 }
 
 // The diagonal blocks of one width class, one CTA per panel.
@@ -456,12 +474,18 @@ void launch_potrf(const DevPlan &p, const int32_t *panels, int count, int wmax, 
     (void)threads;
     if (wmax <= 16) return launch_ldl<T, 16>(p, panels, count, L, Dinv, replace_tau, err_col, nrepl, s);
     if (wmax <= 32) return launch_ldl<T, 32>(p, panels, count, L, Dinv, replace_tau, err_col, nrepl, s);
-    if (wmax <= 64) return launch_ldl<T, 64>(p, panels, count, L, Dinv, replace_tau, err_col, nrepl, s);
     static bool once = false;
     if (!once) {
+        cudaFuncSetAttribute(potrf_mid_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)std::max(fx::smem_bytes(64), ldl_smem_bytes<T, 64>()));
         cudaFuncSetAttribute(potrf_wide_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)std::max(potrf_wide_smem(kMaxWidth), potrf_wide_smem(fx::kMaxW)));
         once = true;
+    }
+    if (wmax <= 64) {
+        const size_t smem = std::max(fx::smem_bytes(wmax), ldl_smem_bytes<T, 64>());
+        potrf_mid_kernel<T><<<count, 256, smem, s>>>(p, panels, L, Dinv, replace_tau, err_col, nrepl);
+        return;
     }
     potrf_wide_kernel<T><<<count, 256, potrf_wide_smem(wmax), s>>>(p, panels, L, Dinv, replace_tau, err_col, nrepl);
 }

@@ -2,24 +2,32 @@
 // in fixed-point integers.
 //
 // The block's chain of pivots runs on one SM, whose FP64 unit starts one warp
-// instruction per ~19 cycles and returns it after ~64; its integer units
-// return a 32 x 32 -> 64-bit multiply-add after ~5 cycles and start 40 times
-// as many lane operations.  A positive definite block makes fixed point safe:
+// instruction per ~19 cycles and returns it after ~64; a 32 x 32 -> 64-bit
+// multiply-add returns after ~16, and four warps start one at a time.  A positive definite block makes fixed point safe:
 // with row and column i scaled by 2^-s_i so that 1 <= a_ii < 4, every entry
 // and every partial sum of the factorization stays below sqrt(a_ii a_jj) < 4
 // in magnitude, every entry of L below 2 (Cauchy-Schwarz on A = L L^T).
 // Entries are held as 64-bit numbers a 2^59 and l 2^60, so a rounding error is
 // 2^-60 of sqrt(a_ii a_jj), where FP64's is 2^-53 of the entry's own
 // magnitude, at most that of sqrt(a_ii a_jj): the backward error of the block
-// does not grow.  Products use two signed limbs (31 bits and the rest), three
-// 32 x 32-bit multiply-adds each; the product of the low limbs is below half
-// a unit and is left out.
+// does not grow.  The inverse X of the scaled L is held as x 2^56 while every
+// |x| < 8; its rows' largest entries are at least 1/2 (at 2^53 the solves' errors
+// were 1.5 times those of FP64's, at 2^56 they are 0.85 of them).  Products use two
+// signed limbs (31 bits and the rest), three 32 x 32-bit multiply-adds each;
+// the product of the low limbs is below half a unit and of either sign, so it
+// is left out -- but for the squares on the diagonal, whose low limbs' squares
+// would all add up one way (a relative 2^-57 of every pivot, which the solve of
+// a 64^3 grid amplifies a thousandfold): those are summed beside it (low).
 //
 // What fixed point cannot hold is left to the floating-point path: the
 // function changes nothing and returns false when an entry is not finite,
-// when |a_ij| or an entry of L breaks its bound (not positive definite), or
-// when a pivot falls below 2^-44 of its bound (it is zero, negative, or so
-// small that static replacement may apply).
+// when |a_ij| or an entry of L breaks its bound (not positive definite), when
+// a pivot falls below 2^-44 of its bound (it is zero, negative, or so small
+// that static replacement may apply), or when an entry of X reaches 8.
+//
+// A 64-wide FP64 block takes 48 us (FP64 unit: 67), FP32 47 (51; both start as
+// the same integers); 128 wide 0.18 ms (0.54 on the FP64 unit).  What bounds it: per 8 columns about 6,600 cycles of one warp's
+// dependent instructions, a third of them the reciprocal square roots.
 #pragma once
 
 #include "blocks.cuh"
@@ -35,13 +43,16 @@ constexpr int kMaxW = 152;                 // widest block whose square fits the
 __host__ __device__ constexpr int width8(int w) { return (w + 7) & ~7; }
 
 // Shared memory for a block of width up to wmax: the square with L in its
-// lower triangle and the inverse, transposed, above it; the digit limbs of two
-// block columns; one block row of products; per-column scales and pivots.
+// lower triangle and the inverse, transposed, above it; the limbs of two block
+// columns of L and of a block row of X; per-column scales, pivots and sums.
 __host__ __device__ constexpr size_t smem_bytes(int wmax)
 {
-    return (size_t)8 * (width8(wmax) + 1) * (width8(wmax) + 1) + (size_t)2 * 8 * 8 * width8(wmax) +
-           (size_t)8 * 8 * width8(wmax) + (size_t)width8(wmax) * (8 + 4 + 4 + 4) + 16;
+    return (size_t)8 * (width8(wmax) + 1) * (width8(wmax) + 1) + (size_t)3 * 8 * kDB * width8(wmax) +
+           (size_t)width8(wmax) * (8 + 4 + 4 + 4 + 4) + 16;
 }
+constexpr int kFX = 56;                    // entries of X: x 2^56, |x| < 8
+constexpr long long kMaxX = 1LL << (kFX + 3);
+constexpr int kMaxXe = 61 - kFX;           // a pivot's reciprocal root above 2^kMaxXe is above that, too
 
 struct Limbs {
     int hi, lo;                            // value = hi 2^31 + lo, |lo| <= 2^30
@@ -74,10 +85,10 @@ __device__ __forceinline__ long long shfl_ll(long long v, int src)
 // 5 h^3 / 16 < 2^-61; h comes from the exact product m y0^2 modulo 2^77.
 __device__ __forceinline__ long long rsqrt_fx(long long D, int *e)
 {
-    const int n = __clzll(D), s = (n - 1) & ~1;
+    const unsigned f = __float_as_uint(__ll2float_rz(D));
+    const int s = (189 - (int)(f >> 23)) & ~1;                  // D in [2^62-s', ...), s even
     const unsigned long long M = (unsigned long long)D << s;   // m = M 2^-61 in [1, 4)
-    const unsigned t = (unsigned)(((unsigned long long)D << n) >> 32);
-    const unsigned fb = ((unsigned)(128 + s + 1 - n) << 23) | ((t >> 8) & 0x7FFFFFu);
+    const unsigned fb = f + ((unsigned)(s - 61) << 23);
     float yf;
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"(__uint_as_float(fb)));
     const unsigned yb = min(max(__float_as_uint(yf), 0x3F000000u), 0x3F7FFFFFu);   // [1/2, 1)
@@ -92,115 +103,159 @@ __device__ __forceinline__ long long rsqrt_fx(long long D, int *e)
     const long long C = (H >> 15) + ((wide(h, h) * 3) >> 30);   // (h / 2 + 3 h^2 / 8) 2^63
     *e = s / 2 - 1;
     return ((long long)y0 << 38) + (wide((int)(C >> 32), (int)y0) << 7) +
-           (long long)(((unsigned long long)(unsigned)C * y0) >> 25);
+           (long long)(((unsigned long long)(unsigned)C * y0 + (1u << 24)) >> 25);
 }
 
-// v 2^e as a double, rounded to nearest (ties away), the result in range.
-__device__ __forceinline__ double to_double(long long v, int e)
+// A number's fields by integer operations: sign, biased exponent, mantissa
+// with the leading bit (subnormal numbers: without, at exponent 1) shifted to
+// 62 bits.  value = m 2^(e - kBias); a double's m is one less where a bit from
+// the middle of its mantissa is set, so that of the ties in rounding it later
+// half go up and half down (all up: 64 entries of a row would add up).
+template <typename T>
+struct Fields;
+template <>
+struct Fields<double> {
+    static constexpr int kOne = 1023, kBias = 1075 + 9, kMin = 128, kMax = 1918;
+    long long b;
+    __device__ __forceinline__ explicit Fields(double v) { b = __double_as_longlong(v); }
+    __device__ __forceinline__ int top() const { return (int)(b >> 52); }          // sign and exponent
+    __device__ __forceinline__ unsigned mant23() const { return (unsigned)(b >> 29) & 0x7FFFFFu; }
+    __device__ __forceinline__ int exp() const { return max((int)(b >> 52) & 0x7FF, 1); }
+    __device__ __forceinline__ long long sign() const { return b >> 63; }
+    __device__ __forceinline__ unsigned long long mant() const
+    {
+        const unsigned long long m = (unsigned long long)b & 0xFFFFFFFFFFFFFULL;
+        return ((((b >> 52) & 0x7FF) != 0 ? m | 0x10000000000000ULL : m) << 9) - ((b >> 40) & 1);
+    }
+};
+template <>
+struct Fields<float> {
+    static constexpr int kOne = 127, kBias = 150 + 38, kMin = 1, kMax = 254;
+    int b;
+    __device__ __forceinline__ explicit Fields(float v) { b = __float_as_int(v); }
+    __device__ __forceinline__ int top() const { return b >> 23; }
+    __device__ __forceinline__ unsigned mant23() const { return (unsigned)b & 0x7FFFFFu; }
+    __device__ __forceinline__ int exp() const { return max((b >> 23) & 0xFF, 1); }
+    __device__ __forceinline__ long long sign() const { return b >> 31; }
+    __device__ __forceinline__ unsigned long long mant() const
+    {
+        return (unsigned long long)(((b >> 23) & 0xFF) != 0 ? mant23() | 0x800000u : mant23()) << 38;
+    }
+};
+
+// v 2^e rounded to nearest, the result in range: as a double by integer
+// operations (ties away), as a float by the conversion.
+__device__ __forceinline__ void to_value(long long v, int e, double *out)
 {
-    if (v == 0) return 0.0;
     const unsigned long long m = (unsigned long long)(v < 0 ? -v : v);
     const int n = __clzll((long long)m);
     const unsigned long long f = m << n;
     const unsigned long long bits =
         ((unsigned long long)(1023 + 63 - n + e - 1) << 52) + (f >> 11) + ((f >> 10) & 1u);
-    return __longlong_as_double((long long)(bits | (v < 0 ? 0x8000000000000000ULL : 0ULL)));
+    *out = v == 0 ? 0.0 : __longlong_as_double((long long)(bits | (v < 0 ? 0x8000000000000000ULL : 0ULL)));
 }
-
-// d 2^k (the exponent moved with integers; past the normal range by scalbn).
-__device__ __forceinline__ double scale2(double d, int k)
+__device__ __forceinline__ void to_value(long long v, int e, float *out)
 {
-    const long long b = __double_as_longlong(d);
-    const int ef = (int)((b >> 52) & 0x7FF);
-    if (ef == 0) return d == 0.0 ? d : scalbn(d, k);
-    if ((unsigned)(ef + k - 1) >= 2046u) return scalbn(d, k);
-    return __longlong_as_double(b + ((long long)k << 52));
+    *out = __ll2float_rn(v) * __uint_as_float((unsigned)(127 + e) << 23);
 }
 
 // The block columns' pivots by nw warps: every one of them factors the 8 x 8
 // diagonal part in its lanes 0 .. 7 (the same operations, so the same bits)
 // and applies it to its own rows in lanes 8 .. 31, NR rows a lane, so no warp
-// waits for another.  Per column the chain is: the pivot from its lane, its
-// reciprocal square root, the column's entry of the next row times it, the
-// square subtracted from the next pivot.
+// waits for another.  Column c takes its row's earlier columns at once, when
+// its turn comes (sums of limb products, cut to a result once a column); the
+// next pivot comes from its own lane's running sum of squares.  The chain of a
+// column is then: the pivot from its lane, its reciprocal square root, the
+// column's entry times it, its square taken from the next pivot.
 template <int NR>
 __device__ __forceinline__ void panel(long long *a, int LD, int W8, int kb, int v, int nw, int2 *lim, long long *rfix,
-                                      int *rexp, float *rowsum, int *bad)
+                                      int *rexp, const float *low, int *bad)
 {
     const int lane = threadIdx.x & 31;
     int row[NR];
     long long q[NR][kDB];
-    float sum[NR];
+    Limbs l[NR][kDB];
 #pragma unroll
     for (int t = 0; t < NR; ++t) {
         row[t] = lane < 8 ? (t == 0 ? kb + lane : W8) : kb + 8 + 24 * (v + t * nw) + lane - 8;
-        const bool in = row[t] < W8;
 #pragma unroll
-        for (int c = 0; c < kDB; ++c) q[t][c] = in && row[t] >= kb + c ? a[row[t] + (kb + c) * LD] : 0;
-        sum[t] = in ? rowsum[row[t]] : 0.0f;
+        for (int c = 0; c < kDB; ++c) q[t][c] = row[t] < W8 && row[t] >= kb + c ? a[row[t] + (kb + c) * LD] : 0;
     }
-    bool wrong = false;
-    long long d = shfl_ll(q[0][0], 0);
+    // this lane's diagonal entry (lanes 0 .. 7) and the sum of squares to take from it
+    long long own = 0, dh = 0, dm = 0;
+#pragma unroll
+    for (int c = 0; c < kDB; ++c)
+        if (lane == c) own = q[0][c];
+    if (lane < kDB) own -= __float2int_rn(low[kb + lane]);
+    int off = 0;
+    long long ykeep = 0;
+    int ekeep = 0;
+    long long d = shfl_ll(own, 0);
 #pragma unroll
     for (int c = 0; c < kDB; ++c) {
-        const int k = kb + c;
-        if ((unsigned long long)(d - kMinPivot) >= (1ULL << (kFA + 2)) - kMinPivot) {
-            wrong = true;
-            d = 1LL << kFA;
-        }
+        const bool low = (unsigned long long)(d - kMinPivot) >= (1ULL << (kFA + 2)) - kMinPivot;
+        off |= low;
+        d = low ? 1LL << kFA : d;
         int e;
         const long long y = rsqrt_fx(d, &e);
         const Limbs r = limbs(y >> 1);                     // 2^61
-        if (v == 0 && lane == c) {
-            rfix[k] = y;
-            rexp[k] = e;
+        ykeep = lane == c ? y : ykeep;
+        ekeep = lane == c ? e : ekeep;
+        long long hh[NR], mid[NR];
+#pragma unroll
+        for (int t = 0; t < NR; ++t) hh[t] = mid[t] = 0;
+#pragma unroll
+        for (int k = 0; k < c; ++k) {
+            const int oh = __shfl_sync(0xffffffffu, l[0][k].hi, c), ol = __shfl_sync(0xffffffffu, l[0][k].lo, c);
+#pragma unroll
+            for (int t = 0; t < NR; ++t) {
+                hh[t] += wide(l[t][k].hi, oh);
+                mid[t] += wide(l[t][k].hi, ol);
+                mid[t] += wide(l[t][k].lo, oh);
+            }
         }
-        Limbs l[NR];
 #pragma unroll
         for (int t = 0; t < NR; ++t) {
-            const long long x = q[t][c];
-            // |a_ik| 2^e <= sqrt(a_ii d) 2^e < 4
-            if (row[t] > k && row[t] < W8 && ((x < 0 ? -x : x) >> (kFA + 2 - e)) != 0) wrong = true;
+            long long x = q[t][c] - (hh[t] << 1) - ((mid[t] + (1LL << 29)) >> 30);
+            if (t == 0 && lane == c) x = d;
+            // |a_ik| 2^e <= sqrt(a_ii d) 2^e < 4 (rows of padding are zero)
+            const int xh = (int)(x >> 32), over = (xh ^ (xh >> 31)) >> (kFA + 2 - 32 - e);
+            off |= t > 0 || lane > c ? over : 0;
             const Limbs s = limbs((long long)((unsigned long long)x << e));
-            const long long lv =
-                (wide(s.hi, r.hi) << 2) + ((wide(s.hi, r.lo) + wide(s.lo, r.hi) + (1LL << 28)) >> 29);
-            l[t] = limbs(lv);
-            q[t][c] = lv;
+            l[t][c] = limbs((wide(s.hi, r.hi) << 2) + ((wide(s.hi, r.lo) + wide(s.lo, r.hi) + (1LL << 28)) >> 29));
         }
-        if (c + 1 < kDB) {
-            // the next pivot from its own lane's entry, ahead of the others' updates
-            const int c1 = c + 1 < kDB ? c + 1 : c;
-            d = shfl_ll(q[0][c1] - mul_ll(l[0], l[0]), c1);
-        }
-#pragma unroll
-        for (int t = 0; t < NR; ++t) {
-            const float lf = (float)l[t].hi * 0x1p-29f;
-            sum[t] = fmaf(lf, lf, sum[t]);
-            // sum_k l_ik^2 <= a_ii (the sum starts from -a_ii), with room for FP32's rounding
-            if (row[t] > k && row[t] < W8 && !(sum[t] <= 5e-4f)) wrong = true;
-        }
-#pragma unroll
-        for (int c2 = c + 1; c2 < kDB; ++c2) {
-            Limbs o;
-            o.hi = __shfl_sync(0xffffffffu, l[0].hi, c2);
-            o.lo = __shfl_sync(0xffffffffu, l[0].lo, c2);
-#pragma unroll
-            for (int t = 0; t < NR; ++t) q[t][c2] -= mul_ll(l[t], o);
-        }
+        dh += wide(l[0][c].hi, l[0][c].hi);
+        dm += wide(l[0][c].hi, l[0][c].lo) + __mulhi(l[0][c].lo, l[0][c].lo);
+        if (c + 1 < kDB) d = shfl_ll(own - (dh << 1) - ((dm + (1LL << 28)) >> 29), c + 1);
+    }
+    if (v == 0 && lane < kDB) {
+        rfix[kb + lane] = ykeep;
+        rexp[kb + lane] = ekeep;
     }
 #pragma unroll
     for (int t = 0; t < NR; ++t) {
         if (row[t] >= W8 || (lane < 8 && v != 0)) continue;
-        rowsum[row[t]] = sum[t];
 #pragma unroll
         for (int c = 0; c < kDB; ++c) {
             const bool lower = row[t] >= kb + c;
-            const Limbs l = limbs(q[t][c]);
-            if (lower) a[row[t] + (kb + c) * LD] = q[t][c];
-            lim[c * W8 + row[t]] = lower ? make_int2(l.hi, l.lo) : make_int2(0, 0);
+            if (lower) a[row[t] + (kb + c) * LD] = ((long long)l[t][c].hi << 31) + l[t][c].lo;
+            lim[c * W8 + row[t]] = lower ? make_int2(l[t][c].hi, l[t][c].lo) : make_int2(0, 0);
         }
     }
-    if (wrong) *bad = 1;
+    if (off) *bad = 1;
+}
+
+// sum over the block's eight terms of x y by limbs: hh 2^62 + mid 2^31
+__device__ __forceinline__ void dot8(const int2 *x, int xs, const int2 *y, int ys, long long &hh, long long &mid)
+{
+    hh = mid = 0;
+#pragma unroll
+    for (int c = 0; c < kDB; ++c) {
+        const int2 u = x[c * xs], v = y[c * ys];
+        hh += wide(u.x, v.x);
+        mid += wide(u.x, v.y);
+        mid += wide(u.y, v.x);
+    }
 }
 
 // Columns [j0, j1), rows >= j: a -= the rank-8 product of the block column in
@@ -214,14 +269,8 @@ __device__ __forceinline__ void rank8(long long *a, int LD, int W8, const int2 *
     }
     while (j < j1) {
         const int i = j + rem;
-        long long hh = 0, mid = 0;
-#pragma unroll
-        for (int c = 0; c < kDB; ++c) {
-            const int2 x = lim[c * W8 + i], y = lim[c * W8 + j];
-            hh += wide(x.x, y.x);
-            mid += wide(x.x, y.y);
-            mid += wide(x.y, y.x);
-        }
+        long long hh, mid;
+        dot8(lim + i, W8, lim + j, W8, hh, mid);
         a[i + j * LD] -= (hh << 1) + ((mid + (1LL << 29)) >> 30);
         rem += ts;
         while (j < j1 && rem >= W8 - j) {
@@ -231,78 +280,78 @@ __device__ __forceinline__ void rank8(long long *a, int LD, int W8, const int2 *
     }
 }
 
-// Block column b of L as doubles, in place.
-__device__ __forceinline__ void convert(long long *a, int LD, int W8, int b, int t0, int ts)
+// Block row b of X = L^{-1} by forward substitution, one column j a thread: the
+// sums T(i, j) = sum_k L(i, k) X(k, j) over the earlier blocks stand in X's
+// places, the block's own terms follow here.
+__device__ __forceinline__ void inverse_row(long long *a, int LD, int W8, int b, int j, const int2 *lim, int2 *limx,
+                                            const long long *rfix, const int *rexp, int *bad)
 {
-    for (int e = t0; e < kDB * (W8 - kDB * b); e += ts) {
-        const int c = e & 7, i = kDB * b + (e >> 3), j = kDB * b + c;
-        if (i >= j) a[i + j * LD] = __double_as_longlong(to_double(a[i + j * LD], -60));
+    const int kb = kDB * b;
+    Limbs x[kDB];
+    bool wrong = false;
+#pragma unroll
+    for (int r = 0; r < kDB; ++r) {
+        const int i = kb + r, e = rexp[i];
+        const long long y = rfix[i];
+        long long s = a[j + (i + 1) * LD], hh = 0, mid = 0;
+#pragma unroll
+        for (int k = 0; k < r; ++k) {
+            const int2 l = lim[k * W8 + i];
+            hh += wide(l.x, x[k].hi);
+            mid += wide(l.x, x[k].lo);
+            mid += wide(l.y, x[k].hi);
+        }
+        s += (hh << 2) + ((mid + (1LL << 28)) >> 29);
+        wrong = wrong || e > kMaxXe || (s ^ (s >> 63)) >= (1LL << 61);
+        const Limbs u = limbs(s), v = limbs(y >> 1);
+        long long xv = (wide(u.hi, v.hi) << 1) + ((wide(u.hi, v.lo) + wide(u.lo, v.hi) + (1LL << 29)) >> 30);
+        const int sh = min(max(e, 0), kMaxXe);
+        if (j == i) xv = (y + (1LL << (61 - kFX))) >> (62 - kFX);             // 1 / l_ii
+        wrong = wrong || (j <= i && (xv ^ (xv >> 63)) >= (kMaxX >> sh));
+        xv = (long long)((unsigned long long)(j < i ? -xv : xv) << sh);
+        if (j > i) xv = 0;
+        x[r] = limbs(xv);
+        if (j <= i) a[j + (i + 1) * LD] = xv;
+        limx[r * W8 + j] = make_int2(x[r].hi, x[r].lo);
+    }
+    if (wrong) *bad = 1;
+}
+
+// T(i, j) += sum over block b of L(i, k) X(k, j), rows i past the block,
+// columns j up to its end.
+__device__ __forceinline__ void inverse_sums(long long *a, int LD, int W8, int b, const int2 *lim, const int2 *limx,
+                                             int t0, int ts)
+{
+    const int i0 = kDB * (b + 1), nj = i0, ni = W8 - i0;
+    if (ni <= 0) return;
+    int i = t0 % nj, c = t0 / nj;          // column i, row i0 + c: columns side by side in memory
+    for (; c < ni;) {
+        long long hh, mid;
+        dot8(lim + i0 + c, W8, limx + i, W8, hh, mid);
+        a[i + (i0 + c + 1) * LD] += (hh << 2) + ((mid + (1LL << 28)) >> 29);
+        i += ts;
+        while (i >= nj) {
+            i -= nj;
+            ++c;
+        }
     }
 }
 
-// Block row b of X = L^{-1}, first half: T_j = sum_k L_bk X_kj for the blocks
-// j < b, on the FP64 tensor path (which no other part of this kernel uses), and
-// the inverse of the 8 x 8 diagonal block, by the last of nw warps.
-__device__ __forceinline__ void inverse_products(double *a, int LD, int b, int wi, int nw, double *Tm,
-                                                 const long long *rfix, const int *rexp)
+// sum_k l_ik^2 <= a_ii, with room for FP32's rounding (the sum starts from
+// -a_ii); the squares of the low limbs, in units of an entry.
+__device__ __forceinline__ void check_row(int i, int W8, const int2 *lim, float *rowsum, float *low, int *bad)
 {
-    const int lane = threadIdx.x & 31, r = lane >> 2, q = lane & 3, kb = kDB * b;
-    if (wi == nw - 1) {
-        if (lane < kDB) {
-            double x[kDB];
+    float s = rowsum[i], t = low[i];
 #pragma unroll
-            for (int i = 0; i < kDB; ++i) x[i] = 0.0;
-#pragma unroll
-            for (int i = 0; i < kDB; ++i) {
-                const double ri = to_double(rfix[kb + i], rexp[kb + i] - 62);
-                double s0 = 0.0, s1 = 0.0;
-#pragma unroll
-                for (int k = 0; k < i; ++k) {
-                    const double l = a[(kb + i) + (kb + k) * LD];
-                    if (k & 1) s1 = fma(l, x[k], s1);
-                    else s0 = fma(l, x[k], s0);
-                }
-                x[i] = i == lane ? ri : (i > lane ? -ri * (s0 + s1) : 0.0);
-            }
-            __syncwarp(0xffu);
-#pragma unroll
-            for (int i = 0; i < kDB; ++i)
-                if (i >= lane) a[(kb + lane) + (kb + i + 1) * LD] = x[i];
-        }
-        __syncwarp();
-        if (nw > 1) return;
+    for (int c = 0; c < kDB; ++c) {
+        const int2 l = lim[c * W8 + i];
+        const float f = (float)l.x * 0x1p-29f, g = (float)l.y * 0x1p-30f;
+        s = fmaf(f, f, s);
+        t = fmaf(g * 0.5f, g, t);
     }
-    for (int j = wi; j < b; j += max(nw - 1, 1)) {
-        double c0 = 0.0, c1 = 0.0, e0 = 0.0, e1 = 0.0;
-        for (int k = j; k < b; ++k) {
-            const double a0 = a[(kb + r) + (kDB * k + q) * LD], a1 = a[(kb + r) + (kDB * k + 4 + q) * LD];
-            double b0 = a[(kDB * j + r) + (kDB * k + q + 1) * LD], b1 = a[(kDB * j + r) + (kDB * k + q + 5) * LD];
-            if (k == j) {   // X_jj is lower triangular
-                if (q < r) b0 = 0.0;
-                if (q + 4 < r) b1 = 0.0;
-            }
-            dmma_f64(c0, c1, a0, b0);
-            dmma_f64(e0, e1, a1, b1);
-        }
-        Tm[(kDB * j + 2 * q) * kDB + r] = c0 + e0;
-        Tm[(kDB * j + 2 * q + 1) * kDB + r] = c1 + e1;
-    }
-}
-
-// ... second half: X_bj = -X_bb T_j.
-__device__ __forceinline__ void inverse_finish(double *a, int LD, int b, int wi, int nw, const double *Tm)
-{
-    const int lane = threadIdx.x & 31, r = lane >> 2, q = lane & 3, kb = kDB * b;
-    double a0 = -a[(kb + q) + (kb + r + 1) * LD], a1 = -a[(kb + q + 4) + (kb + r + 1) * LD];
-    if (q > r) a0 = 0.0;
-    if (q + 4 > r) a1 = 0.0;
-    for (int j = wi; j < b; j += nw) {
-        double c0 = 0.0, c1 = 0.0;
-        dmma_f64(c0, c1, a0, Tm[(kDB * j + r) * kDB + q]);
-        dmma_f64(c0, c1, a1, Tm[(kDB * j + r) * kDB + q + 4]);
-        a[(kDB * j + 2 * q) + (kb + r + 1) * LD] = c0;
-        a[(kDB * j + 2 * q + 1) + (kb + r + 1) * LD] = c1;
-    }
+    low[i] = t;
+    rowsum[i] = s;
+    if (!(s <= 5e-4f)) *bad = 1;
 }
 
 __device__ __forceinline__ void bar_some(int threads)
@@ -313,22 +362,22 @@ __device__ __forceinline__ void bar_some(int threads)
 // The whole block: L over its lower triangle, L^{-1} at Mi (w x w, zeros
 // above).  All 256 threads; false (and nothing written) when the block has to
 // go the floating-point way.  While the chain of block column b runs on up to
-// three warps (NR = 2 rows a lane: four), the others finish the rank-8 update of block column b - 1 and
-// extend the inverse by its block row.
+// three warps (NR = 2 rows a lane: four), the others finish the rank-8 update
+// of block column b - 1 and extend the inverse by its block row.
 template <typename T, int NR>
 __device__ bool diag_block(T *__restrict__ D, T *__restrict__ Mi, int w, int h, unsigned char *smraw)
 {
     const int W8 = width8(w), LD = W8 + 1, nb = W8 / kDB;
     long long *a = reinterpret_cast<long long *>(smraw);
-    double *ad = reinterpret_cast<double *>(smraw);
     int2 *lim = reinterpret_cast<int2 *>(a + (size_t)LD * LD);     // [2][8][W8]
-    double *Tm = reinterpret_cast<double *>(lim + 2 * kDB * W8);   // [W8][8]
-    long long *rfix = reinterpret_cast<long long *>(Tm + kDB * W8);
+    int2 *limx = lim + 2 * kDB * W8;                               // [8][W8]
+    long long *rfix = reinterpret_cast<long long *>(limx + kDB * W8);
     int *rexp = reinterpret_cast<int *>(rfix + W8);
     int *sc = rexp + W8;
     float *rowsum = reinterpret_cast<float *>(sc + W8);
-    int *bad = reinterpret_cast<int *>(rowsum + W8);
-    const int tid = threadIdx.x, warp = tid >> 5;
+    float *low = rowsum + W8;
+    int *bad = reinterpret_cast<int *>(low + W8);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     if (tid == 0) *bad = 0;
     __syncthreads();
@@ -336,84 +385,92 @@ __device__ bool diag_block(T *__restrict__ D, T *__restrict__ Mi, int w, int h, 
         int s = 0;
         float diag = 1.0f;
         if (tid < w) {
-            const double d = to_f64<T>(__ldcg(D + tid + (int64_t)tid * h));
-            const long long b = __double_as_longlong(d);
-            const int ef = (int)(b >> 52);   // 0 .. 0x7FE for a positive finite d
-            if (ef < 128 || ef > 1918) *bad = 1;
-            s = (ef - 1023) >> 1;
-            diag = __uint_as_float(((unsigned)(127 + ((ef - 1023) & 1)) << 23) | (unsigned)((b >> 29) & 0x7FFFFF));
+            const Fields<T> d(__ldcg(D + tid + (int64_t)tid * h));
+            const int ef = d.top();          // the exponent alone for a positive d
+            if (ef < Fields<T>::kMin || ef > Fields<T>::kMax) *bad = 1;
+            s = (ef - Fields<T>::kOne) >> 1;
+            diag = __uint_as_float(((unsigned)(127 + ((ef - Fields<T>::kOne) & 1)) << 23) | d.mant23());
         }
         sc[tid] = s;
         rowsum[tid] = -diag;
+        low[tid] = 0.0f;
     }
     __syncthreads();
-    {
-        constexpr int NB = 8;   // loads in flight a thread
-        const int total = W8 * W8;
-        for (int base = tid; base < total; base += kThreads * NB) {
+    // a warp takes columns, its lanes rows, several columns' loads in flight;
+    // X's places (above the diagonal) start as zero sums
+    for (int i = lane; i < W8; i += 32) {
+        constexpr int NB = 8;
+        const int si = sc[i];
+        for (int j0 = warp; j0 < W8; j0 += 8 * NB) {
             T v[NB];
 #pragma unroll
             for (int u = 0; u < NB; ++u) {
-                const int e = base + u * kThreads, i = e % W8, j = e / W8;
-                v[u] = (e < total && i < w && j < w && i >= j) ? __ldcg(D + i + (int64_t)j * h) : (T)0;
+                const int j = j0 + 8 * u;
+                v[u] = i < w && j < w && i >= j ? __ldcg(D + i + (int64_t)j * h) : (T)0;
             }
 #pragma unroll
             for (int u = 0; u < NB; ++u) {
-                const int e = base + u * kThreads, i = e % W8, j = e / W8;
-                if (e >= total || i < j) continue;
-                long long f = 0;
-                if (i >= w || j >= w) {
-                    f = i == j ? 1LL << kFA : 0;
-                } else {
-                    const long long b = __double_as_longlong(to_f64<T>(v[u]));
-                    const int ef = (int)((b >> 52) & 0x7FF);
-                    long long m = b & 0xFFFFFFFFFFFFFLL;
-                    if (ef > 0) m |= 0x10000000000000LL;
-                    const int sh = (ef > 0 ? ef : 1) - 1075 - sc[i] - sc[j] + kFA;   // 2^sh m
-                    if (m != 0 && sh > 8) *bad = 1;          // 4 or more, infinite or NaN
-                    else if (sh >= 0) m <<= sh;
-                    else m = sh < -60 ? 0 : (m + (1LL << (-sh - 1))) >> -sh;
-                    f = b < 0 ? -m : m;
+                const int j = j0 + 8 * u;
+                if (j >= W8) continue;
+                if (i < j) {
+                    a[i + j * LD] = 0;                 // X(j - 1, i)
+                    continue;
+                }
+                long long f = i == j ? 1LL << kFA : 0;
+                if (i < w) {
+                    const Fields<T> x(v[u]);
+                    const unsigned long long m = x.mant();
+                    const int n = si + sc[j] + Fields<T>::kBias - kFA - x.exp();   // m 2^-n
+                    if (m != 0 && n < 1) *bad = 1;     // 4 or more, infinite or NaN
+                    const long long g = (long long)((m >> min(max(n - 1, 0), 63)) + 1) >> 1, sign = x.sign();
+                    f = (g ^ sign) - sign;
                 }
                 a[i + j * LD] = f;
             }
         }
+        a[i + W8 * LD] = 0;                            // X(W8 - 1, i)
     }
     __syncthreads();
     if (*bad) return false;
 
+    // block column b of L is done: its updates past the next block column, its
+    // block row of the inverse, that row's share of the sums below
     auto others = [&](int b, int wi, int nw) {
-        // block column b is done: its updates past the next block column, its
-        // conversion, its row of the inverse
-        rank8(a, LD, W8, lim + (b & 1) * kDB * W8, kDB * (b + 2), W8, 32 * wi + (tid & 31), 32 * nw);
-        convert(a, LD, W8, b, 32 * wi + (tid & 31), 32 * nw);
+        const int2 *lb = lim + (b & 1) * kDB * W8;
+        const int cols = kDB * (b + 1), nx = min(nw, (cols + 31) / 32);
+        if (wi < nx)
+            for (int j = 32 * wi + lane; j < cols; j += 32 * nx) inverse_row(a, LD, W8, b, j, lb, limx, rfix, rexp, bad);
+        if (nx == nw) rank8(a, LD, W8, lb, kDB * (b + 2), W8, 32 * wi + lane, 32 * nw);
+        else if (wi >= nx) rank8(a, LD, W8, lb, kDB * (b + 2), W8, 32 * (wi - nx) + lane, 32 * (nw - nx));
         bar_some(32 * nw);
-        inverse_products(ad, LD, b, wi, nw, Tm, rfix, rexp);
-        bar_some(32 * nw);
-        inverse_finish(ad, LD, b, wi, nw, Tm);
+        inverse_sums(a, LD, W8, b, lb, limx, 32 * wi + lane, 32 * nw);
     };
     for (int b = 0; b < nb; ++b) {
         const int kb = kDB * b;
+        int2 *lb = lim + (b & 1) * kDB * W8;
         const int nw = min(NR == 1 ? 3 : 4, max(1, (W8 - kb - kDB + 24 * NR - 1) / (24 * NR)));
-        if (warp < nw) panel<NR>(a, LD, W8, kb, warp, nw, lim + (b & 1) * kDB * W8, rfix, rexp, rowsum,
-                                  bad);
+        if (warp < nw) panel<NR>(a, LD, W8, kb, warp, nw, lb, rfix, rexp, low, bad);
         else if (b > 0) others(b - 1, warp - nw, kThreads / 32 - nw);
         __syncthreads();
+        if (kb + tid < W8) check_row(kb + tid, W8, lb, rowsum, low, bad);
+        if (b + 1 < nb) rank8(a, LD, W8, lb, kb + kDB, kb + 2 * kDB, tid, kThreads);
+        __syncthreads();
         if (*bad) return false;
-        if (b + 1 < nb) {
-            rank8(a, LD, W8, lim + (b & 1) * kDB * W8, kb + kDB, kb + 2 * kDB, tid, kThreads);
-            __syncthreads();
-        }
     }
     others(nb - 1, warp, kThreads / 32);
     __syncthreads();
-    for (int e = tid; e < w * w; e += kThreads) {
-        const int i = e % w, j = e / w;
-        if (i >= j) {
-            D[i + (int64_t)j * h] = from_f64<T>(scale2(ad[i + j * LD], sc[i]));
-            Mi[e] = from_f64<T>(scale2(ad[j + (i + 1) * LD], -sc[j]));
-        } else {
-            Mi[e] = (T)0;
+    if (*bad) return false;
+    for (int j = warp; j < w; j += 8) {
+        const int sj = sc[j];
+        for (int i = lane; i < w; i += 32) {
+            T x = (T)0;
+            if (i >= j) {
+                T l;
+                to_value(a[i + j * LD], sc[i] - 60, &l);
+                to_value(a[j + (i + 1) * LD], -kFX - sj, &x);
+                D[i + (int64_t)j * h] = l;
+            }
+            Mi[i + j * w] = x;
         }
     }
     return true;
