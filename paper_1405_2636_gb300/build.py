@@ -25,7 +25,7 @@ CXX_FLAGS = ["-O2", "-std=c++17", "-fPIC", "-I", CSRC, "-I", INCLUDE]
 CU_SOURCES = ["api.cu", "factor.cu", "solve.cu", "update_tc.cu", "batch_api.cu", "batch_lu.cu", "selinv.cu",
               "sweep.cu", "study.cu", "fqueue_f64.cu", "fqueue_tc.cu", "fqueue_ldlt.cu", "update_sl.cu"]
 CXX_SOURCES = ["analyze.cpp"]
-HEADERS = ["kernels.cuh", "spx_plan.h", "batch_kernel.cuh", "operand.cuh", "blocks.cuh", "tc_common.cuh", "fqueue.cuh", "slices.cuh", "fxblock.cuh"]
+HEADERS = ["kernels.cuh", "spx_plan.h", "batch_kernel.cuh", "operand.cuh", "blocks.cuh", "tc_common.cuh", "fqueue.cuh", "slices.cuh", "fxblock.cuh", "lublock.cuh"]
 
 
 def _sources():

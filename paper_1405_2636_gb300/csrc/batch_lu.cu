@@ -26,6 +26,7 @@
 // and sweeps with their rows in registers and blocked pivots of the wide ones;
 // in FP64 the FP64 unit's rate for narrow panels bounds the leaves.
 #include "batch_kernel.cuh"
+#include "lublock.cuh"
 
 #include <cmath>
 
@@ -114,77 +115,6 @@ __device__ __forceinline__ int getrf_warp(T *a, int w, int ld, const Tau<T> &tau
             for (int j = k + 1; j < w; ++j) a[i + j * ld] -= lik * a[k + j * ld];
         }
         __syncwarp();
-    }
-    return nrep;
-}
-
-// The same by the whole CTA (w <= 64): the block column's 8 pivots by warp 0,
-// its rows in registers (two a lane), then the block row of U one column a
-// thread, then the rank-8 update.  64 wide in FP32: a column at a time by one
-// warp spends its time on the update's shared-memory round trips.  nrep and
-// zero_k are warp 0's.
-template <typename T>
-__device__ __forceinline__ int getrf_cta(T *a, int w, int ld, const Tau<T> &tau, int *zero_k)
-{
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    int nrep = 0;
-    for (int k0 = 0; k0 < w; k0 += 8) {
-        const int kc = min(8, w - k0), k1 = k0 + kc;
-        if (warp == 0) {
-            T v[2][8];
-#pragma unroll
-            for (int t = 0; t < 2; ++t)
-#pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    const int i = k0 + lane + 32 * t;
-                    v[t][k] = i < w && k < kc ? a[i + (k0 + k) * ld] : (T)0;
-                }
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                if (k >= kc) break;
-                const T d = tau.pivot(__shfl_sync(0xffffffffu, v[0][k], k), k0 + k, &nrep, zero_k);
-                const T r = (T)1 / d;
-                if (lane == k) v[0][k] = d;
-                else if (lane > k) v[0][k] *= r;
-                v[1][k] *= r;
-#pragma unroll
-                for (int j = k + 1; j < 8; ++j) {
-                    const T u = __shfl_sync(0xffffffffu, v[0][j], k);
-                    if (lane > k) v[0][j] -= v[0][k] * u;
-                    v[1][j] -= v[1][k] * u;
-                }
-            }
-#pragma unroll
-            for (int t = 0; t < 2; ++t)
-#pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    const int i = k0 + lane + 32 * t;
-                    if (i < w && k < kc) a[i + (k0 + k) * ld] = v[t][k];
-                }
-        }
-        __syncthreads();
-        if (k1 >= w) break;                    // kc == 8 from here on
-        if (tid < w - k1) {
-            T u[8];
-            T *col = a + k0 + (k1 + tid) * ld;
-#pragma unroll
-            for (int k = 0; k < 8; ++k) u[k] = col[k];
-#pragma unroll
-            for (int k = 0; k < 8; ++k)
-#pragma unroll
-                for (int j = k + 1; j < 8; ++j) u[j] -= a[k0 + j + (k0 + k) * ld] * u[k];
-#pragma unroll
-            for (int k = 1; k < 8; ++k) col[k] = u[k];
-        }
-        __syncthreads();
-        for (int j = k1 + warp; j < w; j += kWarps)
-            for (int i = k1 + lane; i < w; i += 32) {
-                T s = a[i + j * ld];
-#pragma unroll
-                for (int k = 0; k < 8; ++k) s -= a[i + (k0 + k) * ld] * a[k0 + k + j * ld];
-                a[i + j * ld] = s;
-            }
-        __syncthreads();
     }
     return nrep;
 }
@@ -492,7 +422,9 @@ __device__ __forceinline__ void panel_cta(const BClass &c, int p, T *Ls, T *Us, 
     for (int e = tid; e < w * w; e += kBatchThreads) lu[e % w + (e / w) * kLdC] = Lp[e % w + (e / w) * h];
     __syncthreads();
     int zk = -1;
-    const int nr = getrf_cta<T>(lu, w, kLdC, tau, &zk);
+    int nr = 0;
+    getrf_cta<T, 2>(lu, w, kLdC, [&](T d, int k) { return tau.pivot(d, k, &nr, &zk); },
+                    [](T d) { return (T)1 / d; });
     if (tid == 0) {
         if (nr) atomicAdd(nrep, nr);
         if (zk >= 0) atomicMin(zero_col, c.pfcol[p] + zk);

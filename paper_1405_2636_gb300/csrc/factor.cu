@@ -11,6 +11,7 @@
 // mixed-precision factor); the diagonal blocks are always factored in double.
 #include "blocks.cuh"
 #include "fxblock.cuh"
+#include "lublock.cuh"
 
 #include <cuda_bf16.h>
 #include <algorithm>
@@ -70,36 +71,6 @@ void launch_pack_ranges(const int64_t *ranges, int nr, T *store, T *buf, int mod
 {
     if (nr <= 0) return;
     pack_ranges_kernel<T><<<nr < 152 * 8 ? nr : 152 * 8, 256, 0, s>>>(ranges, nr, store, buf, mode);
-}
-
-// ---------------------------------------------------------------------------
-// In-place inversion of a lower-triangular w x w block held in shared memory
-// (column-major, leading dimension w), read through element (i, j) at
-// a[trans ? j + i*w : i + j*w].  Columns are taken from the right:
-//   X(j,j) = 1 / L(j,j)   (1 when unit),
-//   X(i,j) = -(sum_{k=j+1..i} X(i,k) L(k,j)) X(j,j)   for i > j,
-// using the already inverted columns k > j (from X L = I).  With trans the
-// same routine inverts U^T, i.e. writes U^{-1} in the upper triangle.  C is
-// the storage and arithmetic type; `col` is w elements of scratch.
-// ---------------------------------------------------------------------------
-template <typename C>
-__device__ void invert_lower_inplace(C *a, int w, bool trans, bool unit, C *col)
-{
-    const int tid = threadIdx.x, nt = blockDim.x;
-    for (int j = w - 1; j >= 0; --j) {
-        for (int i = j + 1 + tid; i < w; i += nt) col[i] = a[trans ? j + i * w : i + j * w];
-        __syncthreads();
-        const C xjj = unit ? (C)1 : rcp_newton(a[j + j * w]);
-        for (int i = j + 1 + tid; i < w; i += nt) {
-            const C xii = unit ? (C)1 : a[i + i * w];
-            C s = xii * col[i];
-            for (int k = j + 1; k < i; ++k) s += a[trans ? k + i * w : i + k * w] * col[k];
-            a[trans ? j + i * w : i + j * w] = -s * xjj;
-        }
-        __syncthreads();
-        if (tid == 0 && !unit) a[j + j * w] = xjj;
-        __syncthreads();
-    }
 }
 
 // Narrow the w*w doubles at sm to T in place (T = float: the floats land in
@@ -497,61 +468,65 @@ void launch_potrf(const DevPlan &p, const int32_t *panels, int count, int wmax, 
 // of the unit lower and the upper factor are stored together at Dinv (L^{-1}
 // strictly below the diagonal, U^{-1} on and above it).
 // ---------------------------------------------------------------------------
-template <typename T>
+// Bounds: the chain of a panel's pivots and barriers on one SM.  Block columns
+// of eight (lublock.cuh), FP64 pivots, the inverses in T: on a 121 x 97 grid's
+// factor in FP32 the diagonal blocks take 0.97 ms instead of 1.39 (a column, and
+// in the inverses a row of dot products, between two barriers each).
+// (The leading dimension is odd: rows and columns both free of bank conflicts.)
+constexpr size_t getrf_smem(int w) { return sizeof(double) * ((size_t)w * (w | 1) + 16 * (size_t)w); }
+
+template <typename T, int NR>
 __global__ void __launch_bounds__(256) getrf_kernel(DevPlan p, const int32_t *__restrict__ panels,
                                                     T *__restrict__ L, T *__restrict__ Dinv,
                                                     const double *tau_p, int64_t *err_col,
                                                     unsigned long long *nrepl)
 {
     extern __shared__ double sm[];
-    __shared__ double s_inv;
     const double tau = *tau_p;
     const int pid = panels[blockIdx.x];
-    const int w = p.pw[pid], h = p.ph[pid];
+    const int w = p.pw[pid], h = p.ph[pid], ld = w | 1;
     T *D = L + p.pval[pid];
-    double *col = sm + w * w;
     const int tid = threadIdx.x, nt = blockDim.x;
     for (int idx = tid; idx < w * w; idx += nt) {
         int i = idx % w, j = idx / w;
-        sm[idx] = (double)D[i + (int64_t)j * h];
+        sm[i + j * ld] = (double)D[i + (int64_t)j * h];
     }
     __syncthreads();
-    const int warp = tid >> 5, lane = tid & 31, nw = nt >> 5;
-    for (int k = 0; k < w; ++k) {
-        if (tid == 0) {
-            double d = sm[k + k * w];
-            if (tau > 0.0) {
-                if (fabs(d) < tau) {
-                    d = (d < 0.0) ? -tau : tau;
-                    atomicAdd(nrepl, 1ull);
-                }
-            } else if (d == 0.0 || d != d) {
-                atomicMin((long long *)err_col, (long long)(p.pfcol[pid] + k));
-                d = 1.0;
+    auto pivot = [&](double d, int k) {
+        if (tau > 0.0) {
+            if (fabs(d) < tau) {
+                d = (d < 0.0) ? -tau : tau;
+                if (tid == 0) atomicAdd(nrepl, 1ull);
             }
-            sm[k + k * w] = d;
-            s_inv = rcp_newton(d);
+        } else if (d == 0.0 || d != d) {
+            if (tid == 0) atomicMin((long long *)err_col, (long long)(p.pfcol[pid] + k));
+            d = 1.0;
         }
-        __syncthreads();
-        const double inv = s_inv;
-        for (int i = k + 1 + tid; i < w; i += nt) sm[i + k * w] *= inv;
-        __syncthreads();
-        for (int j = k + 1 + warp; j < w; j += nw) {
-            const double ukj = sm[k + j * w];
-            for (int i = k + 1 + lane; i < w; i += 32) sm[i + j * w] -= sm[i + k * w] * ukj;
-        }
-        __syncthreads();
-    }
+        return d;
+    };
+    getrf_cta<double, NR>(sm, w, ld, pivot, [](double d) { return rcp_newton(d); });
     for (int idx = tid; idx < w * w; idx += nt) {
         int i = idx % w, j = idx / w;
-        D[i + (int64_t)j * h] = (T)sm[idx];
+        D[i + (int64_t)j * h] = (T)sm[i + j * ld];
     }
     __syncthreads();
-    T *a = narrow_inplace<T>(sm, w * w);
-    invert_lower_inplace<T>(a, w, false, true, reinterpret_cast<T *>(col));   // unit lower L
-    invert_lower_inplace<T>(a, w, true, false, reinterpret_cast<T *>(col));   // U through U^T
+    T *a = narrow_inplace<T>(sm, w * ld);
+    invert_lu<T>(a, w, ld, reinterpret_cast<T *>(sm + (size_t)w * ld), [](T d) { return rcp_newton(d); });
     T *Mi = Dinv + p.pinv[pid];
-    for (int idx = tid; idx < w * w; idx += nt) Mi[idx] = a[idx];
+    for (int idx = tid; idx < w * w; idx += nt) Mi[idx] = a[idx % w + (idx / w) * ld];
+}
+
+template <typename T, int NR>
+void launch_getrf_nr(const DevPlan &p, const int32_t *panels, int count, int wmax, int threads, T *L, T *Dinv,
+                     const double *tau, int64_t *err_col, unsigned long long *nrepl, cudaStream_t s)
+{
+    static bool once = false;
+    if (!once) {
+        cudaFuncSetAttribute(getrf_kernel<T, NR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)getrf_smem(32 * NR < kMaxWidth ? 32 * NR : kMaxWidth));
+        once = true;
+    }
+    getrf_kernel<T, NR><<<count, threads, getrf_smem(wmax), s>>>(p, panels, L, Dinv, tau, err_col, nrepl);
 }
 
 template <typename T>
@@ -559,14 +534,9 @@ void launch_getrf(const DevPlan &p, const int32_t *panels, int count, int wmax, 
                   const double *tau, int64_t *err_col, unsigned long long *nrepl, cudaStream_t s)
 {
     if (count <= 0) return;
-    static bool once = false;
-    if (!once) {
-        cudaFuncSetAttribute(getrf_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(sizeof(double) * (kMaxWidth * kMaxWidth + kMaxWidth)));
-        once = true;
-    }
-    const size_t smem = sizeof(double) * ((size_t)wmax * wmax + wmax);
-    getrf_kernel<T><<<count, threads, smem, s>>>(p, panels, L, Dinv, tau, err_col, nrepl);
+    if (wmax <= 32) return launch_getrf_nr<T, 1>(p, panels, count, wmax, threads, L, Dinv, tau, err_col, nrepl, s);
+    if (wmax <= 64) return launch_getrf_nr<T, 2>(p, panels, count, wmax, threads, L, Dinv, tau, err_col, nrepl, s);
+    launch_getrf_nr<T, 5>(p, panels, count, wmax, threads, L, Dinv, tau, err_col, nrepl, s);
 }
 
 template <typename T>
