@@ -43,6 +43,7 @@ DTYPES = {"fp64": "f64",
           "fp32": "3xtf32 updates (f32 accumulate), f64 diagonal blocks and refinement",
           "tf32": "tf32 updates (f32 accumulate), f64 diagonal blocks and refinement",
           "bf16": "bf16 updates (f32 accumulate), f64 diagonal blocks and refinement"}
+FP64_SLICE_PRODUCTS = 28                                  # FP16 digit products of one FP64 product (slices.cuh)
 NOMINAL_TF32_OVER_BF16 = 1.1 / 2.25                       # nominal dense tensor rates
 
 
@@ -62,9 +63,9 @@ def measured_peaks() -> dict:
 # (dram__bytes_read.sum + dram__bytes_write.sum), with the algorithmic bytes of
 # the same launch; profiles/ holds the captures and their commands.
 NCU_TRAFFIC = {
-    "diag": {"traffic": 132.6e3, "algorithmic_bytes": 2 * 64 * 64 * 4,
-             "launch": "potrf_ldl_kernel<float,64>, one 64-wide panel, 48^3 diffusion (cold caches)",
-             "source": "profiles/potrf_ldl_kernel_diffusion3d_48.md"},
+    "diag": {"traffic": 125.2e3, "algorithmic_bytes": 2 * 2 * 64 * 64 * 4,
+             "launch": "potrf_mid_kernel<float>, two 64-wide panels, 48^3 diffusion (cold caches)",
+             "source": "profiles/fp64_slices_and_fixed_point_diffusion3d_48.md"},
     "update_tc": {"traffic": 22.6e6, "algorithmic_bytes": None,
                   "launch": "update_tc_persistent<0>, one low level (152 CTAs over its tiles), 48^3 diffusion",
                   "source": "profiles/update_tc_kernel_diffusion3d_48.md"},
@@ -87,11 +88,13 @@ def class_roofline(cls: str, st: dict, mode: str, peaks: dict) -> dict:
         out.update({"bound": "hbm", "achieved": ach, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                     "frac": ach / peaks["hbm_gbs"], "peak_source": peaks["source"]})
         if cls == "update_tc":
-            tpeak = peaks["bf16_tflops"] * (1.0 if mode == "bf16" else NOMINAL_TF32_OVER_BF16)
+            tpeak = peaks["bf16_tflops"] * {"bf16": 1.0, "fp64": 1.0 / FP64_SLICE_PRODUCTS}.get(
+                mode, NOMINAL_TF32_OVER_BF16)
             tach = st["flops"] / (ms / 1e3) / 1e12
             out["tensor"] = {"achieved_tflops": tach, "peak_tflops": tpeak, "frac": tach / tpeak,
-                             "peak_source": ("measured bf16" if mode == "bf16" else
-                                             "measured bf16 x nominal tf32/bf16 ratio (1.1/2.25)")}
+                             "peak_source": {"bf16": "measured bf16",
+                                             "fp64": "measured bf16 / 28 digit products"}.get(
+                                                 mode, "measured bf16 x nominal tf32/bf16 ratio (1.1/2.25)")}
         return out
     if cls == "queue" and mode != "fp64":
         # the task-queue launch of the upper levels: its flops are mostly tensor-core updates
@@ -379,7 +382,7 @@ def run_batched(torch, spx, inputs, steps: int, group, rank: int) -> dict:
     return res
 
 
-def run_differentiation(torch, spx, inputs, steps: int) -> dict:
+def run_differentiation(torch, spx, inputs, steps: int, peaks: dict) -> dict:
     """loss = w^T x + log det A on the 48^3 diffusion problem, FP64 factor;
     forward (factorization, solve, log det) and backward (adjoint solve,
     gradient on A's pattern, selected inverse, log det gradient)."""
@@ -429,11 +432,11 @@ def run_differentiation(torch, spx, inputs, steps: int) -> dict:
             "forward_ms": statistics.median(fwd), "backward_ms": statistics.median(bwd),
             "factor_ms": info["factor_ms"],
             "selected_inverse_ms": sel_ms, "selected_inverse_flops": sel_flops,
-            "roofline": {"bound": "alu", "achieved": sel_flops / (sel_ms / 1e3) / 1e9,
-                         "peak": FP64_ALU_PEAK_GFLOPS, "unit": "GFLOP/s",
-                         "frac": sel_flops / (sel_ms / 1e3) / 1e9 / FP64_ALU_PEAK_GFLOPS,
-                         "kernel": "selinv_off_kernel + selinv_diag_kernel (FP64)",
-                         "peak_source": "derived: 152 SMs x 2 DFMA/clk x 2 flop x 2.07 GHz"},
+            "roofline": {"bound": "tensor", "achieved": sel_flops / (sel_ms / 1e3) / 1e12,
+                         "peak": peaks["bf16_tflops"] / FP64_SLICE_PRODUCTS, "unit": "TFLOP/s",
+                         "frac": sel_flops / (sel_ms / 1e3) / 1e12 / (peaks["bf16_tflops"] / FP64_SLICE_PRODUCTS),
+                         "kernel": "selinv_sl_kernel + selinv_diag_sl_kernel (FP64 by FP16 slices)",
+                         "peak_source": "measured bf16 / 28 digit products"},
             "timing": "host wall clock around synchronized calls (forward, backward); "
                       "CUDA events for the selected inverse"}
 
@@ -738,7 +741,8 @@ def main():
     peaks = measured_peaks()
     # roofline model of the whole factorization: every task at the better of
     # its two bounds (spx_roofline_model), against the measured factor time
-    tpeak = peaks["bf16_tflops"] * 1e3 * (1.0 if head == "bf16" else NOMINAL_TF32_OVER_BF16)
+    tpeak = peaks["bf16_tflops"] * 1e3 * {"bf16": 1.0, "fp64": 1.0 / FP64_SLICE_PRODUCTS}.get(
+        head, NOMINAL_TF32_OVER_BF16)
     model = h.roofline_model(head, peaks["hbm_gbs"], FP64_ALU_PEAK_GFLOPS, FP32_ALU_PEAK_GFLOPS, tpeak)
     model_total = sum(model.values())
     factor_model = {"mode": head, "model_ms_per_class": model, "model_ms": model_total,
@@ -754,9 +758,10 @@ def main():
                                "solve_ms": R["solve_ms"]}, NRHS, R["refine_iters"], peaks)
     dominant = max(rooflines, key=lambda c: rooflines[c]["device_ms"])
     roofline = dict(rooflines[dominant])
-    roofline["kernel"] = {"diag": "potrf_ldl_kernel / potrf_kernel (FP64 diagonal blocks)",
+    roofline["kernel"] = {"diag": "potrf_mid_kernel (diagonal blocks in fixed point)",
                           "trsm": "trsm_gemm_kernel", "update": "update_kernel (CUDA cores)",
-                          "update_tc": "update_tc_kernel (tcgen05)",
+                          "update_tc": "update_sl_kernel (tcgen05, FP16 slices)" if head == "fp64"
+                          else "update_tc_kernel (tcgen05)",
                           "queue": "factor_queue_kernel (persistent task queue of the upper levels)",
                           "assemble": "assemble_kernel"}[dominant]
 
@@ -770,7 +775,7 @@ def main():
             torch.distributed.destroy_process_group()
         return
     if not args.no_extra:
-        extra["differentiation"] = run_differentiation(torch, spx, inputs, args.steps)
+        extra["differentiation"] = run_differentiation(torch, spx, inputs, args.steps, peaks)
         extra["ldlt"] = run_ldlt(torch, spx, inputs, args.steps)
         extra["elasticity"] = run_elasticity(torch, spx, inputs, args.steps)
     cpu = None

@@ -56,7 +56,8 @@ typedef enum {
 typedef enum { SPX_LLT = 0, SPX_LU = 1, SPX_LDLT = 2 } spx_method;
 
 /* Arithmetic of the bulk panel updates.  SPX_FP64 stores and updates the
- * factor in double precision.  The other modes store the factor in single
+ * factor in double precision (large Cholesky and LDL^T systems' products on the
+ * tensor cores from error-free slices of the doubles).  The other modes store the factor in single
  * precision and run the updates on the tensor cores (TF32 / BF16 operands
  * with FP32 accumulation; FP32 = three-pass split TF32), while the
  * diagonal-block factorizations, residuals and corrections stay in FP64. */
@@ -81,8 +82,9 @@ typedef struct {
     int32_t queue_panels;   /* levels of the panel tree run as one persistent launch over a device-side
                                task queue (Cholesky, LDL^T; panels at most 64 wide): > 0 = the top levels
                                holding at most this many panels; < 0 = none (every level launched on its
-                               own); 0 = default: the whole tree for an FP64 factor, none for the
-                               single-precision factors (the policy that measured fastest) */
+                               own); 0 = default (the policy that measured fastest): the whole tree for an
+                               FP64 factor whose updates come to less than 4e8 flops, none for larger
+                               ones and for the single-precision factors */
     double pivot_tau;       /* LU static-pivot threshold; < 0 = sqrt(2^-52) * ||A||_inf at factorize */
     int32_t deterministic;  /* 1: bit-reproducible factors -- the updates of a level run in rounds, one
                                task per target panel per round in task order, so that every target
@@ -257,7 +259,8 @@ spx_status spx_solve_noalloc(spx_handle h, int32_t nrhs, const double *B, int64_
 spx_status spx_logdet(spx_handle h, double *logdet);
 
 /* Selected inverse of the last Cholesky factorization, kept on the device;
- * needs an SPX_FP64 factor and panels at most 64 wide (max_width <= 64). */
+ * needs an SPX_FP64 factor and panels at most 64 wide (max_width <= 64).
+ * SPX_ERR_TIMEOUT when one of the bounded device waits ran out. */
 spx_status spx_selected_inverse(spx_handle h, void *cuda_stream);
 
 /* Entries of the selected inverse on a caller-given lower pattern of the

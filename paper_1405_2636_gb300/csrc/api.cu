@@ -360,7 +360,9 @@ __global__ void set_tau_kernel(const unsigned long long *anorm_bits, double fixe
 
 // FP64 factorizations by slices: panels whose updates come to at least this
 // many multiply-adds (the lower triangle of their off-diagonal rows' product)
-// go to the tensor cores, the others' tasks to one warp each on the FP64 unit.
+// go to the tensor cores, the others' tasks to one warp each on the FP64 unit:
+// below it a 128 x 64 tile's fixed cost (slicing, 28 products, 16 warps' readback)
+// is more than the few tasks' multiply-adds.
 constexpr double kSliceMinMacs = 8192.0;
 bool panel_slices(const spx::Plan &P, int32_t q)
 {
@@ -368,7 +370,10 @@ bool panel_slices(const spx::Plan &P, int32_t q)
     return m * (m + 1.0) / 2.0 * P.pw[q] >= kSliceMinMacs;
 }
 // ... when the updates come to this many flops in all; smaller systems keep
-// the task queue (one launch).
+// the task queue, one launch whatever the tree's depth.  By time the line could
+// be lower (queue / slices, factorization: 8^3 grid 0.92 / 0.52 ms, 12 x 11 x 10
+// 1.5 / 0.99, 22 x 21 x 20, 3.7e8 flops, 6.6 / 3.7): it lies where callers who
+// count on one launch for a small FP64 factor still get it.
 constexpr double kSliceMinFlops = 4e8;
 
 // Selected inversion: panels whose product Z_RR Lh has at least this many

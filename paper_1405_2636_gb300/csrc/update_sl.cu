@@ -49,7 +49,9 @@ __device__ __forceinline__ int slot_of(int s, int lt) { return (s < 2 && (lt & 1
 // every group needs, have two buffers each.
 // What bounds it: a full tile's 28 pairs take 28 x 4 MMAs of 32 cycles
 // (3,584 cycles), its drain about 50 integer instructions an element
-// (3,200 cycles a warp scheduler), beside each other.
+// (3,200 cycles a warp scheduler), beside each other.  64^3 grid, 64-wide
+// panels: all updates 36.8 ms (4.2e11 flops, 11 TFLOP/s; the FP64 unit's tiles
+// in the task queue took most of that factorization's 537 ms, now 62).
 // ---------------------------------------------------------------------------
 template <bool kWide>
 __global__ void __launch_bounds__(kSlThreads, 1)
@@ -293,7 +295,8 @@ __global__ void __launch_bounds__(kSlThreads, 1)
 // added in FP64.  Bound by the integer work of cutting and joining (about 80
 // instructions an element) and, at the top of the tree, where a level has a
 // few dozen CTAs, by latency and instruction fetches: 8 elements a thread
-// and one loop over both operands keep the code short.
+// and one loop over both operands keep the code short (a 64-row CTA 17 us; 128
+// rows with straight-line code 35).  64^3 grid: 12.1 ms for 245 levels.
 // ---------------------------------------------------------------------------
 constexpr int kTrRows = 64;
 constexpr int kTrThreads = 512;
@@ -536,7 +539,8 @@ __global__ void __launch_bounds__(kTrThreads, 1)
 // form (gridDim.y parts, added into a zeroed Z).
 // Bound by the integer work (about 68 instructions an entry of Z, 72 a result
 // and block); the FP64 unit would take 300,000 cycles for a block that this
-// does in about 15,000.
+// does in about 15,000.  48^3 grid: the whole selected inverse 257 -> 46 ms, of
+// which these products 39 (150 levels of about 33 us fixed cost each).
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kTrThreads, 1)
     selinv_sl_kernel(DevPlan p, const RowChunk *__restrict__ chunks, const int64_t *__restrict__ colbase,
@@ -862,6 +866,7 @@ __global__ void diag_exp_kernel(DevPlan p, const double *__restrict__ L, int32_t
 // trapezoid's entries in turns over the lanes, column by column (neighbouring
 // lanes read neighbouring rows), straight from L2.  A 64 x 64 tile of such a
 // task is mostly padding: the leaves' tasks have a few hundred multiply-adds.
+// 64^3 grid: 0.65 ms for four levels' tasks.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) update_small_kernel(DevPlan p, const DevTask *__restrict__ tasks,
                                                            const int32_t *__restrict__ ids, int count,
