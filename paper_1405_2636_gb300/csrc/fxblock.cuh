@@ -48,7 +48,7 @@ __host__ __device__ constexpr int width8(int w) { return (w + 7) & ~7; }
 __host__ __device__ constexpr size_t smem_bytes(int wmax)
 {
     return (size_t)8 * (width8(wmax) + 1) * (width8(wmax) + 1) + (size_t)3 * 8 * kDB * width8(wmax) +
-           (size_t)width8(wmax) * (8 + 4 + 4 + 4 + 4) + 16;
+           (size_t)width8(wmax) * (8 + 4 + 4 + 4 + 4);
 }
 constexpr int kFX = 56;                    // entries of X: x 2^56, |x| < 8
 constexpr long long kMaxX = 1LL << (kFX + 3);
@@ -167,9 +167,10 @@ __device__ __forceinline__ void to_value(long long v, int e, float *out)
 // next pivot comes from its own lane's running sum of squares.  The chain of a
 // column is then: the pivot from its lane, its reciprocal square root, the
 // column's entry times it, its square taken from the next pivot.
+// True when this thread saw what fixed point cannot hold.
 template <int NR>
-__device__ __forceinline__ void panel(long long *a, int LD, int W8, int kb, int v, int nw, int2 *lim, long long *rfix,
-                                      int *rexp, const float *low, int *bad)
+__device__ __forceinline__ bool panel(long long *a, int LD, int W8, int kb, int v, int nw, int2 *lim, long long *rfix,
+                                      int *rexp, const float *low)
 {
     const int lane = threadIdx.x & 31;
     int row[NR];
@@ -242,7 +243,7 @@ __device__ __forceinline__ void panel(long long *a, int LD, int W8, int kb, int 
             lim[c * W8 + row[t]] = lower ? make_int2(l[t][c].hi, l[t][c].lo) : make_int2(0, 0);
         }
     }
-    if (off) *bad = 1;
+    return off != 0;
 }
 
 // sum over the block's eight terms of x y by limbs: hh 2^62 + mid 2^31
@@ -282,9 +283,9 @@ __device__ __forceinline__ void rank8(long long *a, int LD, int W8, const int2 *
 
 // Block row b of X = L^{-1} by forward substitution, one column j a thread: the
 // sums T(i, j) = sum_k L(i, k) X(k, j) over the earlier blocks stand in X's
-// places, the block's own terms follow here.
-__device__ __forceinline__ void inverse_row(long long *a, int LD, int W8, int b, int j, const int2 *lim, int2 *limx,
-                                            const long long *rfix, const int *rexp, int *bad)
+// places, the block's own terms follow here.  True when an entry breaks its bound.
+__device__ __forceinline__ bool inverse_row(long long *a, int LD, int W8, int b, int j, const int2 *lim, int2 *limx,
+                                            const long long *rfix, const int *rexp)
 {
     const int kb = kDB * b;
     Limbs x[kDB];
@@ -314,7 +315,7 @@ __device__ __forceinline__ void inverse_row(long long *a, int LD, int W8, int b,
         if (j <= i) a[j + (i + 1) * LD] = xv;
         limx[r * W8 + j] = make_int2(x[r].hi, x[r].lo);
     }
-    if (wrong) *bad = 1;
+    return wrong;
 }
 
 // T(i, j) += sum over block b of L(i, k) X(k, j), rows i past the block,
@@ -338,8 +339,8 @@ __device__ __forceinline__ void inverse_sums(long long *a, int LD, int W8, int b
 }
 
 // sum_k l_ik^2 <= a_ii, with room for FP32's rounding (the sum starts from
-// -a_ii); the squares of the low limbs, in units of an entry.
-__device__ __forceinline__ void check_row(int i, int W8, const int2 *lim, float *rowsum, float *low, int *bad)
+// -a_ii), or true; the squares of the low limbs, in units of an entry.
+__device__ __forceinline__ bool check_row(int i, int W8, const int2 *lim, float *rowsum, float *low)
 {
     float s = rowsum[i], t = low[i];
 #pragma unroll
@@ -351,7 +352,7 @@ __device__ __forceinline__ void check_row(int i, int W8, const int2 *lim, float 
     }
     low[i] = t;
     rowsum[i] = s;
-    if (!(s <= 5e-4f)) *bad = 1;
+    return !(s <= 5e-4f);
 }
 
 __device__ __forceinline__ void bar_some(int threads)
@@ -363,7 +364,10 @@ __device__ __forceinline__ void bar_some(int threads)
 // above).  All 256 threads; false (and nothing written) when the block has to
 // go the floating-point way.  While the chain of block column b runs on up to
 // three warps (NR = 2 rows a lane: four), the others finish the rank-8 update
-// of block column b - 1 and extend the inverse by its block row.
+// of block column b - 1 and extend the inverse by its block row.  What a thread
+// finds wrong stays its own (bad) until a barrier joins all threads' flags, so
+// that all leave at the same barrier: a shared flag, read behind one barrier,
+// could already hold what a faster warp finds before the next.
 template <typename T, int NR>
 __device__ bool diag_block(T *__restrict__ D, T *__restrict__ Mi, int w, int h, unsigned char *smraw)
 {
@@ -376,18 +380,16 @@ __device__ bool diag_block(T *__restrict__ D, T *__restrict__ Mi, int w, int h, 
     int *sc = rexp + W8;
     float *rowsum = reinterpret_cast<float *>(sc + W8);
     float *low = rowsum + W8;
-    int *bad = reinterpret_cast<int *>(low + W8);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    bool bad = false;
 
-    if (tid == 0) *bad = 0;
-    __syncthreads();
     if (tid < W8) {
         int s = 0;
         float diag = 1.0f;
         if (tid < w) {
             const Fields<T> d(__ldcg(D + tid + (int64_t)tid * h));
             const int ef = d.top();          // the exponent alone for a positive d
-            if (ef < Fields<T>::kMin || ef > Fields<T>::kMax) *bad = 1;
+            bad = ef < Fields<T>::kMin || ef > Fields<T>::kMax;
             s = (ef - Fields<T>::kOne) >> 1;
             diag = __uint_as_float(((unsigned)(127 + ((ef - Fields<T>::kOne) & 1)) << 23) | d.mant23());
         }
@@ -421,7 +423,7 @@ __device__ bool diag_block(T *__restrict__ D, T *__restrict__ Mi, int w, int h, 
                     const Fields<T> x(v[u]);
                     const unsigned long long m = x.mant();
                     const int n = si + sc[j] + Fields<T>::kBias - kFA - x.exp();   // m 2^-n
-                    if (m != 0 && n < 1) *bad = 1;     // 4 or more, infinite or NaN
+                    bad = bad || (m != 0 && n < 1);    // 4 or more, infinite or NaN
                     const long long g = (long long)((m >> min(max(n - 1, 0), 63)) + 1) >> 1, sign = x.sign();
                     f = (g ^ sign) - sign;
                 }
@@ -430,8 +432,7 @@ __device__ bool diag_block(T *__restrict__ D, T *__restrict__ Mi, int w, int h, 
         }
         a[i + W8 * LD] = 0;                            // X(W8 - 1, i)
     }
-    __syncthreads();
-    if (*bad) return false;
+    if (__syncthreads_or(bad)) return false;
 
     // block column b of L is done: its updates past the next block column, its
     // block row of the inverse, that row's share of the sums below
@@ -439,7 +440,7 @@ __device__ bool diag_block(T *__restrict__ D, T *__restrict__ Mi, int w, int h, 
         const int2 *lb = lim + (b & 1) * kDB * W8;
         const int cols = kDB * (b + 1), nx = min(nw, (cols + 31) / 32);
         if (wi < nx)
-            for (int j = 32 * wi + lane; j < cols; j += 32 * nx) inverse_row(a, LD, W8, b, j, lb, limx, rfix, rexp, bad);
+            for (int j = 32 * wi + lane; j < cols; j += 32 * nx) bad |= inverse_row(a, LD, W8, b, j, lb, limx, rfix, rexp);
         if (nx == nw) rank8(a, LD, W8, lb, kDB * (b + 2), W8, 32 * wi + lane, 32 * nw);
         else if (wi >= nx) rank8(a, LD, W8, lb, kDB * (b + 2), W8, 32 * (wi - nx) + lane, 32 * (nw - nx));
         bar_some(32 * nw);
@@ -449,17 +450,15 @@ __device__ bool diag_block(T *__restrict__ D, T *__restrict__ Mi, int w, int h, 
         const int kb = kDB * b;
         int2 *lb = lim + (b & 1) * kDB * W8;
         const int nw = min(NR == 1 ? 3 : 4, max(1, (W8 - kb - kDB + 24 * NR - 1) / (24 * NR)));
-        if (warp < nw) panel<NR>(a, LD, W8, kb, warp, nw, lb, rfix, rexp, low, bad);
+        if (warp < nw) bad |= panel<NR>(a, LD, W8, kb, warp, nw, lb, rfix, rexp, low);
         else if (b > 0) others(b - 1, warp - nw, kThreads / 32 - nw);
         __syncthreads();
-        if (kb + tid < W8) check_row(kb + tid, W8, lb, rowsum, low, bad);
+        if (kb + tid < W8) bad |= check_row(kb + tid, W8, lb, rowsum, low);
         if (b + 1 < nb) rank8(a, LD, W8, lb, kb + kDB, kb + 2 * kDB, tid, kThreads);
-        __syncthreads();
-        if (*bad) return false;
+        if (__syncthreads_or(bad)) return false;
     }
     others(nb - 1, warp, kThreads / 32);
-    __syncthreads();
-    if (*bad) return false;
+    if (__syncthreads_or(bad)) return false;
     for (int j = warp; j < w; j += 8) {
         const int sj = sc[j];
         for (int i = lane; i < w; i += 32) {

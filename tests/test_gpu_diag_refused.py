@@ -1,0 +1,66 @@
+"""Diagonal blocks that the fixed-point kernel (csrc/fxblock.cuh) refuses, found
+out at every one of their columns, beside blocks that it takes, all in one
+launch: each block's decision is its own, and the result is the factor either
+way.  A refusal has to be taken by all threads of a block at the same barrier;
+block columns here break the bounds of L, of the pivots and of the inverse one
+after another, so that a thread that left early would meet the wrong barrier.
+
+L L^T is compared with the matrix: every entry of it is a sum of at most w products
+of L's entries and one rounding each, to the factor's precision.
+"""
+import numpy as np
+import pytest
+import scipy.sparse as sp
+
+import oracle
+from paper_1405_2636_gb300 import inputs, spx
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    import torch
+    import __graft_entry__
+
+    __graft_entry__.build()
+    assert torch.cuda.is_available()
+
+
+def _block(w, g, small=None, pivot=1.0):
+    """w x w block L L^T, L's rows of norm about one; pivot `small` set to `pivot`."""
+    L = np.tril(g.uniform(-1.0, 1.0, (w, w)), -1) / np.sqrt(w)
+    np.fill_diagonal(L, g.uniform(0.7, 1.0, w))
+    if small is not None:
+        L[small, small] = pivot
+    A = np.tril(L @ L.T)
+    return A + np.tril(A, -1).T
+
+
+@pytest.mark.parametrize("width", [40, 64, 96, 128])
+@pytest.mark.parametrize("pivot", [0.05, 2.0 ** -21, 2.0 ** -24])
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_refused_at_every_column(width, pivot, prec):
+    if prec == "fp32" and pivot < 0.01:
+        pivot = 2.0 ** -9                  # an FP32 factor knows its entries to 2^-24
+    g = np.random.default_rng([width, 7])
+    blocks = []
+    for col in range(0, width, 1 if width <= 64 else 3):
+        blocks += [_block(width, g, col, pivot), _block(width, g)]
+    A = sp.csc_matrix(sp.block_diag(blocks))
+    cp, ri, vals = inputs.csc_arrays(A)
+    h = spx.analyze(cp, ri, "llt", ordering=spx.SPX_ORDER_NATURAL, max_width=width, queue_panels=-1)
+    assert h.info()["npanels"] == len(blocks)
+    p = h.perm()
+    F = oracle.cholesky(A, p)
+    for _ in range(3):
+        h.factorize(vals, prec)
+        Lx = h.factor_on_pattern(F.sym.Lp, F.sym.Li)
+        M = sp.csc_matrix((Lx, F.sym.Li, F.sym.Lp))
+        eps = 2.0 ** -53 if prec == "fp64" else 2.0 ** -24
+        # backward error of w multiply-adds
+        assert abs(M @ M.T - A[p][:, p]).max() <= 2 * (width + 2) * eps * np.max(A.diagonal())
+    n = A.shape[0]
+    X, _ = h.solve(inputs.rhs(n, 2, 1))
+    assert oracle.backward_error(A, X, inputs.rhs(n, 2, 1)) <= (1e-13 if prec == "fp64" else 1e-12)
+    h.free()
