@@ -289,7 +289,12 @@ __global__ void __launch_bounds__(kSlThreads, 1)
 // leading one of 1 / l_kk (LDL^T: of 1 / sqrt(d_k)) and the inverse's by the
 // opposite, which the products do not see: X(i, k) grows with the scale of
 // unknown k and Linv(j, k) falls with it, and without this one large entry of
-// each row, at different k, would set the rows' exponents.
+// each row, at different k, would set the rows' exponents.  LDL^T's two operand
+// copies for the update are cut with such scales, too: L(i, k) falls and
+// (D L^T)(j, k) grows with the scale of unknown k, so L's column k is taken
+// times about sqrt(|d_k|) and D L^T's divided by it (unscaled, the update's
+// error was that of FP64 multiply-adds times the ratio of the largest to the
+// smallest scale in the panel).  Cholesky's L has no such factor.
 // Panels wider than 64 go by 64-column blocks, the last one first (block c
 // needs the old X of blocks <= c), the partial sums of their digit blocks
 // added in FP64.  Bound by the integer work of cutting and joining (about 80
@@ -494,12 +499,14 @@ __global__ void __launch_bounds__(kTrThreads, 1)
                     if (j0 + q < w) out[q] *= __ldcg(Mi + (j0 + q) + (int64_t)(j0 + q) * w);
             }
             double *dst = (o == 1 ? Wout + p.pval[pid] + ch.r0 : Xg) + r + (int64_t)j0 * h;
-            int f = 1;
+            int sc[kTC], f = kFieldZero;
 #pragma unroll
             for (int q = 0; q < kTC; ++q) {
+                // (s_sc: this block's columns, the last that the products took)
+                sc[q] = ldlt ? (o == 1 ? s_sc[kTC * part + q] : -s_sc[kTC * part + q]) : 0;
                 if (j0 + q >= w) out[q] = 0.0;
                 else if (row_ok) dst[(int64_t)q * h] = out[q];
-                f = max(f, exp_field(out[q]));
+                f = max(f, exp_field(out[q], sc[q]));
             }
             if (right) continue;   // no operand copy
             s_f[0][part][r] = f;
@@ -511,7 +518,7 @@ __global__ void __launch_bounds__(kTrThreads, 1)
                 const int64_t orow = p.prow[pid] + ch.r0 + r;
                 if (part == 0) (o == 1 ? expb : expa)[(int64_t)(c0 / kK) * oprows + orow] = row_exp(f);
                 uint32_t wd[kSlices][4];
-                digits8(out, f, wd);
+                digits8(out, f, wd, sc);
                 __half *op = (o == 1 ? opb : opa) + orow * kpad + j0;
 #pragma unroll
                 for (int s = 0; s < kSlices; ++s)
