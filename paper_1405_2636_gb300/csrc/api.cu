@@ -216,6 +216,7 @@ struct spx_handle_s {
     int64_t *d_colbase = nullptr, *d_relbase = nullptr;   // per operand row: where its column goes
     void *d_slop[2] = {nullptr, nullptr};
     int32_t *d_slexp[2] = {nullptr, nullptr};
+    int32_t *d_rowexp = nullptr;   // per column, the exponent of its unknown's scale (launch_potrf)
     alignas(64) unsigned char tmap_sla[128];
     alignas(64) unsigned char tmap_slb[128];
     int *d_tcerr = nullptr;
@@ -1211,7 +1212,7 @@ spx_status ensure_slices(spx_handle h)
     }
     spx_status st;
     if ((st = upload(h, &h->d_sl_tiles, tiles)) || (st = upload(h, &h->d_sl_small, small)) ||
-        (st = upload(h, &h->d_slc, chunks)) || (st = ensure_colmaps(h)))
+        (st = upload(h, &h->d_slc, chunks)) || (st = dalloc(h, &h->d_rowexp, (size_t)P.n)) || (st = ensure_colmaps(h)))
         return st;
     h->sl_ready = true;
     return SPX_OK;
@@ -1410,10 +1411,10 @@ void enqueue_factorization(spx_handle h, bool mixed, Marks &mk, int prec, int pa
             const cudaStream_t sc = br.pick(nlaunch++);
             if (ldlt)
                 spx::launch_ldlt_diag<T>(h->dp, h->d_level_panels + a, b - a, cw, L, Dinv, h->d_tau, h->d_err,
-                                         h->d_nrepl, h->d_nneg, sc);
+                                         h->d_nrepl, h->d_nneg, slices ? h->d_rowexp : nullptr, sc);
             else if (!lu)
                 spx::launch_potrf<T>(h->dp, h->d_level_panels + a, b - a, cw, kClassThreads[c], L,
-                                     Dinv, h->d_tau, h->d_err, h->d_nrepl, sc);
+                                     Dinv, h->d_tau, h->d_err, h->d_nrepl, slices ? h->d_rowexp : nullptr, sc);
             else
                 spx::launch_getrf<T>(h->dp, h->d_level_panels + a, b - a, cw, kClassThreads[c], L,
                                      Dinv, h->d_tau, h->d_err, h->d_nrepl, sc);
@@ -1454,7 +1455,7 @@ void enqueue_factorization(spx_handle h, bool mixed, Marks &mk, int prec, int pa
             if (slices) {
                 const int nsc = (int)(h->slc_ptr[l + 1] - h->slc_ptr[l]);
                 spx::launch_trsm_sl(h->dp, h->d_slc + h->slc_ptr[l], nsc, (const double *)Dinv, (double *)L,
-                                    (double *)W, ldlt ? spx::TRSM_LDLT : spx::TRSM_LLT, h->d_slop[0], h->d_slop[1], h->d_slexp[0],
+                                    (double *)W, ldlt ? spx::TRSM_LDLT : spx::TRSM_LLT, h->d_rowexp, h->d_slop[0], h->d_slop[1], h->d_slexp[0],
                                     h->d_slexp[1], h->op_rows, h->kpad, h->d_tcerr, s);
                 cnt += nsc > 0;
                 h->class_launches[SPX_K_TRSM] += nsc > 0;
@@ -2996,7 +2997,7 @@ spx_status spx_selected_inverse(spx_handle h, void *cuda_stream)
     spx::launch_diag_exp(h->dp, (const double *)h->d_L, h->d_dexp, h->hs);
     // (h->d_chunks: 64 rows each, as the slices TRSM takes them)
     spx::launch_trsm_sl(h->dp, h->d_chunks, (int)h->chunk_ptr[P.nlevels], (const double *)h->d_Dinv, h->d_Lh, nullptr,
-                        spx::TRSM_RIGHT_LINV, nullptr, nullptr, nullptr, nullptr, 0, 0, h->d_tcerr, h->hs);
+                        spx::TRSM_RIGHT_LINV, nullptr, nullptr, nullptr, nullptr, nullptr, 0, 0, h->d_tcerr, h->hs);
     spx::launch_selinv_diag(h->dp, h->d_level_panels, P.npanels, 1, wmax, 1, (const double *)h->d_Dinv, h->d_Lh,
                             h->d_Zsel, h->hs);
     // split-K so that a level keeps about two CTAs per SM busy near the root

@@ -156,6 +156,16 @@ __device__ __forceinline__ void dmma_f64(double &d0, double &d1, double a, doubl
                  : "d"(a), "d"(b));
 }
 
+// Leading exponent of |x| from its high word (|x| < 2^(e + 1)); far below every
+// other for zero and the smallest subnormal numbers, far above for infinities and NaN.
+constexpr int kNoExp = 1 << 13;
+__device__ __forceinline__ int lead_exp(int hi)
+{
+    hi &= 0x7FFFFFFF;
+    return hi == 0 ? -kNoExp : hi >= 0x7FF00000 ? kNoExp : (hi >> 20) - 1023;
+}
+__device__ __forceinline__ int high_word(const double *x) { return __ldcg(reinterpret_cast<const int *>(x) + 1); }
+
 constexpr int kDB = 8;
 constexpr long kDiagSpin = 1l << 22;   // polls of the hand-off counter before a diagonal block gives up
 
@@ -189,8 +199,10 @@ __device__ __forceinline__ double shfl_d(double v, int src)
 template <typename T, int W, bool ldlt>
 __device__ __forceinline__ void ldl_diag_block(const DevPlan &p, int pid, T *__restrict__ L,
                                                T *__restrict__ Dinv, double replace_tau, int64_t *err_col,
-                                               unsigned long long *nrepl, unsigned long long *nneg, double *sm)
+                                               unsigned long long *nrepl, unsigned long long *nneg, double *sm,
+                                               int32_t *rowexp = nullptr)
 {
+    constexpr bool kExps = std::is_same<T, double>::value;   // rowexp: the columns' scales for the TRSM by slices
     constexpr int LD = W + 1;
     constexpr int NT = 256;
     double *a = sm;                          // W x LD, FP64 working block
@@ -201,6 +213,7 @@ __device__ __forceinline__ void ldl_diag_block(const DevPlan &p, int pid, T *__r
     volatile int *hflag = reinterpret_cast<volatile int *>(hand + 9 * kDB);   // columns handed to warp 1
     T *x = reinterpret_cast<T *>(hand + 9 * kDB + 8);   // W x LD inverse workspace
     T *tmp = x + W * LD;                     // (W/2)^2, the FP64 factors' inverse
+    int *rmax = reinterpret_cast<int *>(hand);          // after the factorization, LDL^T: rows' largest exponents
     T *dvf = tmp + (W / 2) * (W / 2);        // pivots (Cholesky: their square roots) in T
     T *rvf = dvf + W;                        // and their reciprocals
     const int w = p.pw[pid], h = p.ph[pid];
@@ -225,6 +238,8 @@ __device__ __forceinline__ void ldl_diag_block(const DevPlan &p, int pid, T *__r
             if (idx >= W * W) continue;
             const int i = idx % W, j = idx / W;
             a[i + j * LD] = (i < w && j < w) ? to_f64<T>(vv[q]) : (i == j ? 1.0 : 0.0);
+            if constexpr (kExps && !ldlt)
+                if (rowexp && i == j && i < w) rowexp[col0 + i] = lead_exp(__double2hiint(vv[q])) >> 1;
         }
         if (tid == 0) *hflag = 0;
     }
@@ -409,16 +424,22 @@ __device__ __forceinline__ void ldl_diag_block(const DevPlan &p, int pid, T *__r
         }
         dvf[tid] = from_f64<T>(dv[tid]);
         rvf[tid] = from_f64<T>(rsv[tid]);
+        if constexpr (kExps && ldlt) rmax[tid] = lead_exp(__double2hiint(dv[tid])) >> 1;
     }
     __syncthreads();
     for (int idx = tid; idx < W * W; idx += NT) {
         const int i = idx % W, j = idx / W;
         const T l = i > j ? from_f64<T>(a[i + j * LD]) : (T)0;
+        if constexpr (kExps && ldlt)
+            if (rowexp && i > j)
+                atomicMax(&rmax[i], lead_exp(__double2hiint(l)) + (lead_exp(__double2hiint(dv[j])) >> 1));
         if (i < w && j < w && i >= j)
             D[i + (int64_t)j * h] = i == j ? dvf[j] : (ldlt ? l : l * dvf[j]);
         x[i + j * LD] = i > j ? l : (i == j ? (T)1 : (T)0);
     }
     __syncthreads();
+    if constexpr (kExps && ldlt)
+        if (rowexp && tid < w) rowexp[col0 + tid] = rmax[tid];
 
     T *Mi = Dinv + p.pinv[pid];
     if constexpr (std::is_same<T, float>::value) {

@@ -328,7 +328,7 @@ __device__ void invert_lower_blocked(C *a, int w, C *tmp)
 // ---------------------------------------------------------------------------
 template <typename T>
 __device__ void potrf_block(const DevPlan &p, int pid, T *__restrict__ L, T *__restrict__ Dinv, double replace_tau,
-                            int64_t *err_col, unsigned long long *nrepl, double *sm)
+                            int64_t *err_col, unsigned long long *nrepl, double *sm, int32_t *rowexp)
 {
     const int w = p.pw[pid], h = p.ph[pid];
     T *D = L + p.pval[pid];
@@ -336,6 +336,7 @@ __device__ void potrf_block(const DevPlan &p, int pid, T *__restrict__ L, T *__r
     for (int idx = tid; idx < w * w; idx += nt) {
         int i = idx % w, j = idx / w;
         sm[idx] = (i >= j) ? (double)D[i + (int64_t)j * h] : 0.0;
+        if (rowexp && i == j) rowexp[p.pfcol[pid] + i] = lead_exp(__double2hiint(sm[idx])) >> 1;
     }
     __syncthreads();
     if (w <= 64) chol_reg64(sm, w, w, replace_tau, p.pfcol[pid], err_col, nrepl);
@@ -357,16 +358,17 @@ template <typename T>
 __global__ void __launch_bounds__(256) potrf_wide_kernel(DevPlan p, const int32_t *__restrict__ panels,
                                                          T *__restrict__ L, T *__restrict__ Dinv,
                                                          const double *replace_tau_p, int64_t *err_col,
-                                                         unsigned long long *nrepl)
+                                                         unsigned long long *nrepl, int32_t *rowexp)
 {
     extern __shared__ double sm[];
     const int pid = panels[blockIdx.x];
     const int w = p.pw[pid], h = p.ph[pid];
     if (w <= fx::kMaxW && fx::diag_block<T, 2>(L + p.pval[pid], Dinv + p.pinv[pid], w, h,
-                                               reinterpret_cast<unsigned char *>(sm)))
+                                               reinterpret_cast<unsigned char *>(sm),
+                                               rowexp ? rowexp + p.pfcol[pid] : nullptr))
         return;
     __syncthreads();
-    potrf_block<T>(p, pid, L, Dinv, *replace_tau_p, err_col, nrepl, sm);
+    potrf_block<T>(p, pid, L, Dinv, *replace_tau_p, err_col, nrepl, sm, rowexp);
 }
 
 size_t potrf_wide_smem(int wmax)
@@ -384,15 +386,16 @@ template <typename T>
 __global__ void __launch_bounds__(256) potrf_mid_kernel(DevPlan p, const int32_t *__restrict__ panels,
                                                         T *__restrict__ L, T *__restrict__ Dinv,
                                                         const double *replace_tau_p, int64_t *err_col,
-                                                        unsigned long long *nrepl)
+                                                        unsigned long long *nrepl, int32_t *rowexp)
 {
     extern __shared__ double sm[];
     const int pid = panels[blockIdx.x];
     const int w = p.pw[pid], h = p.ph[pid];
-    if (fx::diag_block<T, 1>(L + p.pval[pid], Dinv + p.pinv[pid], w, h, reinterpret_cast<unsigned char *>(sm)))
+    if (fx::diag_block<T, 1>(L + p.pval[pid], Dinv + p.pinv[pid], w, h, reinterpret_cast<unsigned char *>(sm),
+                             rowexp ? rowexp + p.pfcol[pid] : nullptr))
         return;
     __syncthreads();
-    ldl_diag_block<T, 64, false>(p, pid, L, Dinv, *replace_tau_p, err_col, nrepl, nullptr, sm);
+    ldl_diag_block<T, 64, false>(p, pid, L, Dinv, *replace_tau_p, err_col, nrepl, nullptr, sm, rowexp);
 }
 
 // The diagonal blocks of one width class, one CTA per panel.
@@ -401,16 +404,16 @@ __global__ void __launch_bounds__(256) potrf_ldl_kernel(DevPlan p, const int32_t
                                                         T *__restrict__ L, T *__restrict__ Dinv,
                                                         const double *replace_tau_p,
                                                         int64_t *err_col, unsigned long long *nrepl,
-                                                        unsigned long long *nneg)
+                                                        unsigned long long *nneg, int32_t *rowexp)
 {
     extern __shared__ double sm[];
-    ldl_diag_block<T, W, ldlt>(p, panels[blockIdx.x], L, Dinv, *replace_tau_p, err_col, nrepl, nneg, sm);
+    ldl_diag_block<T, W, ldlt>(p, panels[blockIdx.x], L, Dinv, *replace_tau_p, err_col, nrepl, nneg, sm, rowexp);
 }
 
 template <typename T, int W, bool ldlt = false>
 void launch_ldl(const DevPlan &p, const int32_t *panels, int count, T *L, T *Dinv,
-                const double *replace_tau, int64_t *err_col, unsigned long long *nrepl, cudaStream_t s,
-                unsigned long long *nneg = nullptr)
+                const double *replace_tau, int64_t *err_col, unsigned long long *nrepl, int32_t *rowexp,
+                cudaStream_t s, unsigned long long *nneg = nullptr)
 {
     static bool once = false;
     const size_t smem = ldl_smem_bytes<T, W>();
@@ -419,7 +422,8 @@ void launch_ldl(const DevPlan &p, const int32_t *panels, int count, T *L, T *Din
                              (int)smem);
         once = true;
     }
-    potrf_ldl_kernel<T, W, ldlt><<<count, 256, smem, s>>>(p, panels, L, Dinv, replace_tau, err_col, nrepl, nneg);
+    potrf_ldl_kernel<T, W, ldlt><<<count, 256, smem, s>>>(p, panels, L, Dinv, replace_tau, err_col, nrepl, nneg,
+                                                         rowexp);
 }
 
 // LDL^T diagonal blocks (panels at most 64 wide): l with d on the diagonal,
@@ -428,23 +432,23 @@ void launch_ldl(const DevPlan &p, const int32_t *panels, int count, T *L, T *Din
 template <typename T>
 void launch_ldlt_diag(const DevPlan &p, const int32_t *panels, int count, int wmax, T *L, T *Dinv,
                       const double *tau, int64_t *err_col, unsigned long long *nrepl,
-                      unsigned long long *nneg, cudaStream_t s)
+                      unsigned long long *nneg, int32_t *rowexp, cudaStream_t s)
 {
     if (count <= 0) return;
-    if (wmax <= 16) return launch_ldl<T, 16, true>(p, panels, count, L, Dinv, tau, err_col, nrepl, s, nneg);
-    if (wmax <= 32) return launch_ldl<T, 32, true>(p, panels, count, L, Dinv, tau, err_col, nrepl, s, nneg);
-    launch_ldl<T, 64, true>(p, panels, count, L, Dinv, tau, err_col, nrepl, s, nneg);
+    if (wmax <= 16) return launch_ldl<T, 16, true>(p, panels, count, L, Dinv, tau, err_col, nrepl, rowexp, s, nneg);
+    if (wmax <= 32) return launch_ldl<T, 32, true>(p, panels, count, L, Dinv, tau, err_col, nrepl, rowexp, s, nneg);
+    launch_ldl<T, 64, true>(p, panels, count, L, Dinv, tau, err_col, nrepl, rowexp, s, nneg);
 }
 
 template <typename T>
 void launch_potrf(const DevPlan &p, const int32_t *panels, int count, int wmax, int threads, T *L, T *Dinv,
-                  const double *replace_tau, int64_t *err_col, unsigned long long *nrepl,
+                  const double *replace_tau, int64_t *err_col, unsigned long long *nrepl, int32_t *rowexp,
                   cudaStream_t s)
 {
     if (count <= 0) return;
     (void)threads;
-    if (wmax <= 16) return launch_ldl<T, 16>(p, panels, count, L, Dinv, replace_tau, err_col, nrepl, s);
-    if (wmax <= 32) return launch_ldl<T, 32>(p, panels, count, L, Dinv, replace_tau, err_col, nrepl, s);
+    if (wmax <= 16) return launch_ldl<T, 16>(p, panels, count, L, Dinv, replace_tau, err_col, nrepl, rowexp, s);
+    if (wmax <= 32) return launch_ldl<T, 32>(p, panels, count, L, Dinv, replace_tau, err_col, nrepl, rowexp, s);
     static bool once = false;
     if (!once) {
         cudaFuncSetAttribute(potrf_mid_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -455,10 +459,11 @@ void launch_potrf(const DevPlan &p, const int32_t *panels, int count, int wmax, 
     }
     if (wmax <= 64) {
         const size_t smem = std::max(fx::smem_bytes(wmax), ldl_smem_bytes<T, 64>());
-        potrf_mid_kernel<T><<<count, 256, smem, s>>>(p, panels, L, Dinv, replace_tau, err_col, nrepl);
+        potrf_mid_kernel<T><<<count, 256, smem, s>>>(p, panels, L, Dinv, replace_tau, err_col, nrepl, rowexp);
         return;
     }
-    potrf_wide_kernel<T><<<count, 256, potrf_wide_smem(wmax), s>>>(p, panels, L, Dinv, replace_tau, err_col, nrepl);
+    potrf_wide_kernel<T><<<count, 256, potrf_wide_smem(wmax), s>>>(p, panels, L, Dinv, replace_tau, err_col, nrepl,
+                                                                   rowexp);
 }
 
 // ---------------------------------------------------------------------------
@@ -625,15 +630,15 @@ template void launch_pack_ranges<double>(const int64_t *, int, double *, double 
 template void launch_pack_ranges<float>(const int64_t *, int, float *, float *, int, cudaStream_t);
 template void launch_assemble<double>(int64_t, const double *, const int64_t *, double *, double *, cudaStream_t);
 template void launch_assemble<float>(int64_t, const double *, const int64_t *, float *, float *, cudaStream_t);
-template void launch_potrf<double>(const DevPlan &, const int32_t *, int, int, int, double *, double *, const double *, int64_t *, unsigned long long *, cudaStream_t);
-template void launch_potrf<float>(const DevPlan &, const int32_t *, int, int, int, float *, float *, const double *, int64_t *, unsigned long long *, cudaStream_t);
+template void launch_potrf<double>(const DevPlan &, const int32_t *, int, int, int, double *, double *, const double *, int64_t *, unsigned long long *, int32_t *, cudaStream_t);
+template void launch_potrf<float>(const DevPlan &, const int32_t *, int, int, int, float *, float *, const double *, int64_t *, unsigned long long *, int32_t *, cudaStream_t);
 template void launch_getrf<double>(const DevPlan &, const int32_t *, int, int, int, double *, double *, const double *, int64_t *, unsigned long long *, cudaStream_t);
 template void launch_getrf<float>(const DevPlan &, const int32_t *, int, int, int, float *, float *, const double *, int64_t *, unsigned long long *, cudaStream_t);
 template void launch_trsm<double>(const DevPlan &, const RowChunk *, int, int, const double *, double *, int, void *, void *, int, int, cudaStream_t, double *);
 template void launch_lead<float>(const DevPlan &, RowChunk, const DevTask *, int32_t, const float *, float *, void *, void *, int, int, cudaStream_t);
-template void launch_ldlt_diag<double>(const DevPlan &, const int32_t *, int, int, double *, double *, const double *, int64_t *, unsigned long long *, unsigned long long *, cudaStream_t);
+template void launch_ldlt_diag<double>(const DevPlan &, const int32_t *, int, int, double *, double *, const double *, int64_t *, unsigned long long *, unsigned long long *, int32_t *, cudaStream_t);
 template void launch_trsm<float>(const DevPlan &, const RowChunk *, int, int, const float *, float *, int, void *, void *, int, int, cudaStream_t, float *);
-template void launch_ldlt_diag<float>(const DevPlan &, const int32_t *, int, int, float *, float *, const double *, int64_t *, unsigned long long *, unsigned long long *, cudaStream_t);
+template void launch_ldlt_diag<float>(const DevPlan &, const int32_t *, int, int, float *, float *, const double *, int64_t *, unsigned long long *, unsigned long long *, int32_t *, cudaStream_t);
 template void launch_update<double>(const DevPlan &, const DevTask *, const UpdTile *, int, const double *, const double *, double *, int, int, cudaStream_t, int);
 template void launch_update<float>(const DevPlan &, const DevTask *, const UpdTile *, int, const float *, const float *, float *, int, int, cudaStream_t, int);
 

@@ -368,8 +368,9 @@ __device__ __forceinline__ void bar_some(int threads)
 // finds wrong stays its own (bad) until a barrier joins all threads' flags, so
 // that all leave at the same barrier: a shared flag, read behind one barrier,
 // could already hold what a faster warp finds before the next.
+// rowexp (or null): the exponents of about sqrt(a_ii).
 template <typename T, int NR>
-__device__ bool diag_block(T *__restrict__ D, T *__restrict__ Mi, int w, int h, unsigned char *smraw)
+__device__ bool diag_block(T *__restrict__ D, T *__restrict__ Mi, int w, int h, unsigned char *smraw, int32_t *rowexp)
 {
     const int W8 = width8(w), LD = W8 + 1, nb = W8 / kDB;
     long long *a = reinterpret_cast<long long *>(smraw);
@@ -391,6 +392,7 @@ __device__ bool diag_block(T *__restrict__ D, T *__restrict__ Mi, int w, int h, 
             const int ef = d.top();          // the exponent alone for a positive d
             bad = ef < Fields<T>::kMin || ef > Fields<T>::kMax;
             s = (ef - Fields<T>::kOne) >> 1;
+            if (rowexp) rowexp[tid] = s;
             diag = __uint_as_float(((unsigned)(127 + ((ef - Fields<T>::kOne) & 1)) << 23) | d.mant23());
         }
         sc[tid] = s;

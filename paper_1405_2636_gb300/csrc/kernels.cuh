@@ -77,9 +77,11 @@ void launch_assemble(int64_t nnz, const double *vals, const int64_t *amap, T *L,
 template <typename T>
 void launch_pack_ranges(const int64_t *ranges, int nr, T *store, T *buf, int mode, cudaStream_t s);
 
+// rowexp (FP64 factors, or null): per column k the exponent of about sqrt(a_kk), the
+// entry as it stood before the block's elimination, for launch_trsm_sl.
 template <typename T>
 void launch_potrf(const DevPlan &p, const int32_t *panels, int count, int wmax, int threads, T *L, T *Dinv,
-                  const double *replace_tau, int64_t *err_col, unsigned long long *nrepl,
+                  const double *replace_tau, int64_t *err_col, unsigned long long *nrepl, int32_t *rowexp,
                   cudaStream_t s);
 
 template <typename T>
@@ -105,11 +107,12 @@ void launch_lead(const DevPlan &p, RowChunk ch, const DevTask *tasks, int32_t ta
 
 // LDL^T diagonal blocks, panels at most 64 wide (factor.cu): l with d on the
 // diagonal, l^{-1} with 1/d on its diagonal at Dinv; static pivoting with
-// threshold *tau; negative pivots counted in *nneg.
+// threshold *tau; negative pivots counted in *nneg; rowexp as in launch_potrf, of
+// the largest l(k, m) sqrt(|d_m|) of row k.
 template <typename T>
 void launch_ldlt_diag(const DevPlan &p, const int32_t *panels, int count, int wmax, T *L, T *Dinv,
                       const double *tau, int64_t *err_col, unsigned long long *nrepl,
-                      unsigned long long *nneg, cudaStream_t s);
+                      unsigned long long *nneg, int32_t *rowexp, cudaStream_t s);
 
 // Tensor-core update (update_tc.cu).  tmap / tmap_lo: CUtensorMaps over the
 // operand copies (make_operand_map; tmap_lo is used for kind 2 only); err
@@ -136,9 +139,10 @@ constexpr int kSliceCount = 7;
 void launch_update_sl(const void *mapa, const void *mapb, int64_t oprows, const DevPlan &p, const SlTile *tiles,
                       int count, const int64_t *colbase, const int64_t *relbase, const int32_t *expa, const int32_t *expb, double *C, int *err, int per_cta,
                       int wmax, cudaStream_t s);
-// chunks: 64 rows each.  LDL^T: opa / expa hold L, opb / expb D L^T.
+// chunks: 64 rows each.  LDL^T: opa / expa hold L, opb / expb D L^T.  rowexp: the
+// columns' scales (launch_potrf; TRSM_RIGHT_LINV needs none).
 void launch_trsm_sl(const DevPlan &p, const RowChunk *chunks, int count, const double *Dinv, double *X, double *Wout,
-                    int mode, void *opa, void *opb, int32_t *expa, int32_t *expb, int64_t oprows, int kpad, int *err,
+                    int mode, const int32_t *rowexp, void *opa, void *opb, int32_t *expa, int32_t *expb, int64_t oprows, int kpad, int *err,
                     cudaStream_t s);
 // Selected inversion's Z_RJ (update_sl.cu): chunks of 128 rows; colbase,
 // relbase: where each off-diagonal row's column lies, as in launch_update_sl;

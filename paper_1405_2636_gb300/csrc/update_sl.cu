@@ -7,6 +7,7 @@
 // each (row, block) has its own exponent at exp[block * rows + prow[p] + r].
 // The TRSM writes it; the update loads 128-row (A) and 64-row (B) boxes of it
 // by TMA with the 128-byte swizzle.
+#include "blocks.cuh"
 #include "slices.cuh"
 
 #include <algorithm>
@@ -286,10 +287,14 @@ __global__ void __launch_bounds__(kSlThreads, 1)
 // twice in the 128-row A tile, so that all four TMEM lane quadrants hold
 // results: quadrants 0 and 1 drain columns 0 .. 31, 2 and 3 the rest.
 // Both operands' columns k are scaled by powers of two first, X's by the
-// leading one of 1 / l_kk (LDL^T: of 1 / sqrt(d_k)) and the inverse's by the
-// opposite, which the products do not see: X(i, k) grows with the scale of
+// inverse of about sqrt(a_kk) (LDL^T: of the largest l(k, m) sqrt(|d_m|)), whose
+// exponents the diagonal block's kernel leaves in rowexp, and the inverse's by
+// the opposite, which the products do not see: X(i, k) grows with the scale of
 // unknown k and Linv(j, k) falls with it, and without this one large entry of
-// each row, at different k, would set the rows' exponents.  LDL^T's two operand
+// each row, at different k, would set the rows' exponents.  (Not by the pivot
+// l_kk, which elimination inside the block may leave far below sqrt(a_kk): on
+// smooth covariance matrices of 256 points and a nugget of 1e-8 that left the
+// entries of L L^T 2.9e-12 off, where FP64 multiply-adds leave 4.9e-14.)  LDL^T's two operand
 // copies for the update are cut with such scales, too: L(i, k) falls and
 // (D L^T)(j, k) grows with the scale of unknown k, so L's column k is taken
 // times about sqrt(|d_k|) and D L^T's divided by it (unscaled, the update's
@@ -349,7 +354,8 @@ __device__ __forceinline__ void issue_pairs(uint32_t tmem, const unsigned char *
 
 __global__ void __launch_bounds__(kTrThreads, 1)
     trsm_sl_kernel(DevPlan p, const RowChunk *__restrict__ chunks, const double *__restrict__ Dinv,
-                   double *__restrict__ X, double *__restrict__ Wout, int mode, __half *__restrict__ opa,
+                   double *__restrict__ X, double *__restrict__ Wout, int mode, const int32_t *__restrict__ rowexp,
+                   __half *__restrict__ opa,
                    __half *__restrict__ opb, int32_t *__restrict__ expa, int32_t *__restrict__ expb, int64_t oprows,
                    int kpad, int *err)
 {
@@ -362,7 +368,8 @@ __global__ void __launch_bounds__(kTrThreads, 1)
     __shared__ int s_fail;
     __shared__ int s_f[2][8][kTrRows];                // exponent fields, parts of a row: X's, the inverse's
     __shared__ int32_t s_e[2][kTrRows];
-    __shared__ int s_sc[kK];
+    __shared__ int s_sc[kMaxWidth + kK];              // scales of the products' columns (up to whole digit blocks),
+    __shared__ int s_sd[kK];                          // and LDL^T's of the operand copies'
     const RowChunk ch = chunks[blockIdx.x];
     const bool ldlt = mode == TRSM_LDLT, right = mode == TRSM_RIGHT_LINV;
     const int pid = ch.panel, w = p.pw[pid], h = p.ph[pid];
@@ -381,12 +388,21 @@ __global__ void __launch_bounds__(kTrThreads, 1)
                      "r"(kSlCols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
+    if (const int k = tid - 32; k >= 0 && k < kMaxWidth + kK) {      // (warp 0 allocates the accumulators)
+        // column k of X times 2^s_sc, column k of the inverse divided by it
+        const int e = k < w && !right ? rowexp[p.pfcol[pid] + k] : 0;
+        s_sc[k] = e < -kNoExp / 4 || e > kNoExp / 4 ? 0 : -e;        // (rows of zeros, infinities, NaN)
+        if (k < kK) {
+            const int d = ldlt && k < w ? lead_exp(high_word(X + p.pval[pid] + k + (int64_t)k * h)) : 0;
+            s_sd[k] = d < -kNoExp / 2 || d > kNoExp / 2 ? 0 : d >> 1;
+        }
+    }
+    const int rs = tid & (kTrRows - 1), ps = tid / kTrRows;          // staging: row and 8-column part
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = s_tmem;
 
-    const int rs = tid & (kTrRows - 1), ps = tid / kTrRows;          // staging: row and 8-column part
     const int quad = warp & 3;
     const int r = 32 * (quad & 1) + lane, part = 4 * (quad >> 1) + (warp >> 2);   // results: row and part
     const bool row_ok = r < nr;
@@ -396,13 +412,6 @@ __global__ void __launch_bounds__(kTrThreads, 1)
         double out[kTC];
         for (int k0 = 0; k0 <= c0; k0 += kK) {
             const int ksteps = (min(kK, w - k0) + 15) / 16;
-            // column k of X times 2^s_sc, column k of the inverse divided by it
-            if (tid < kK) {
-                const int k = k0 + tid;
-                const int e = k < w ? ((__double2hiint(__ldcg(Mi + k + (int64_t)k * w)) >> 20) & 0x7FF) - 1023 : 0;
-                s_sc[tid] = (right || e < -1022 || e > 1023) ? 0 : (ldlt ? e >> 1 : e);
-            }
-            __syncthreads();
             // operand 0: X(rs, k0 ..), operand 1: the inverse's row c0 + rs
             // (B(k, j) = Linv(j, k)); eight columns of one row a thread
 #pragma unroll 1
@@ -426,7 +435,7 @@ __global__ void __launch_bounds__(kTrThreads, 1)
                 }
                 int sc[kTC];
 #pragma unroll
-                for (int q = 0; q < kTC; ++q) sc[q] = o == 0 ? s_sc[k1 - k0 + q] : -s_sc[k1 - k0 + q];
+                for (int q = 0; q < kTC; ++q) sc[q] = o == 0 ? s_sc[k1 + q] : -s_sc[k1 + q];
                 int f = kFieldZero;
 #pragma unroll
                 for (int q = 0; q < kTC; ++q) f = max(f, exp_field(x[q], sc[q]));
@@ -502,8 +511,7 @@ __global__ void __launch_bounds__(kTrThreads, 1)
             int sc[kTC], f = kFieldZero;
 #pragma unroll
             for (int q = 0; q < kTC; ++q) {
-                // (s_sc: this block's columns, the last that the products took)
-                sc[q] = ldlt ? (o == 1 ? s_sc[kTC * part + q] : -s_sc[kTC * part + q]) : 0;
+                sc[q] = ldlt ? (o == 1 ? -s_sd[kTC * part + q] : s_sd[kTC * part + q]) : 0;   // (at most 64 wide)
                 if (j0 + q >= w) out[q] = 0.0;
                 else if (row_ok) dst[(int64_t)q * h] = out[q];
                 f = max(f, exp_field(out[q], sc[q]));
@@ -937,7 +945,7 @@ void launch_update_sl(const void *mapa, const void *mapb, int64_t oprows, const 
 }
 
 void launch_trsm_sl(const DevPlan &p, const RowChunk *chunks, int count, const double *Dinv, double *X, double *Wout,
-                    int mode, void *opa, void *opb, int32_t *expa, int32_t *expb, int64_t oprows, int kpad, int *err,
+                    int mode, const int32_t *rowexp, void *opa, void *opb, int32_t *expa, int32_t *expb, int64_t oprows, int kpad, int *err,
                     cudaStream_t s)
 {
     if (count <= 0) return;
@@ -946,7 +954,7 @@ void launch_trsm_sl(const DevPlan &p, const RowChunk *chunks, int count, const d
         cudaFuncSetAttribute(trsm_sl_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTrSmem);
         once = true;
     }
-    trsm_sl_kernel<<<count, kTrThreads, kTrSmem, s>>>(p, chunks, Dinv, X, Wout, mode, (__half *)opa, (__half *)opb,
+    trsm_sl_kernel<<<count, kTrThreads, kTrSmem, s>>>(p, chunks, Dinv, X, Wout, mode, rowexp, (__half *)opa, (__half *)opb,
                                                       expa, expb, oprows, kpad, err);
 }
 
