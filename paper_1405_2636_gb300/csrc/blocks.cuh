@@ -175,6 +175,133 @@ __device__ __forceinline__ double shfl_d(double v, int src)
 }
 
 // ---------------------------------------------------------------------------
+// Inverse of a factored diagonal block, by 256 threads: Mi (w x w) from the
+// unit-lower l at x (leading dimension W + 1, padded with the identity to W) and
+// rvf, the reciprocals of the pivots (Cholesky: of their square roots).  FP32
+// factors invert l by forward substitution in registers (warp v owns columns
+// v, v + 8, ...); FP64 factors by blocks (8 x 8 diagonal blocks by single lanes,
+// then pairs of blocks merged with X21 = -C^{-1} (B A^{-1})), which does a sixth
+// of the multiply-adds.  tmp: (W / 2)^2 elements.
+// ---------------------------------------------------------------------------
+template <typename T, int W, bool ldlt>
+__device__ __forceinline__ void invert_unit(T *x, T *tmp, const T *rvf, T *__restrict__ Mi, int w)
+{
+    constexpr int LD = W + 1, NT = 256;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if constexpr (std::is_same<T, float>::value) {
+        // forward substitution in registers: warp v owns columns v, v + 8, ...
+        // of X = l^{-1}, W / 32 rows per lane; at step k the lane holding row
+        // k broadcasts x_k and every lane subtracts l(i, k) x_k.  The k loop
+        // is split at the row-group boundary so that the broadcast reads a
+        // fixed register.
+        constexpr int CPW = W / 8;
+        constexpr int RG = (W + 31) / 32;
+        T xr[CPW][RG];
+#pragma unroll
+        for (int t = 0; t < CPW; ++t)
+#pragma unroll
+            for (int g = 0; g < RG; ++g) xr[t][g] = (32 * g + lane == warp + 8 * t) ? (T)1 : (T)0;
+        auto step = [&](int k, auto gk) {
+            constexpr int G = decltype(gk)::value;
+            T lk[RG];
+#pragma unroll
+            for (int g = 0; g < RG; ++g) {
+                const int i = 32 * g + lane;
+                const T v = x[min(i, W - 1) + k * LD];
+                lk[g] = (i > k && i < W) ? v : (T)0;
+            }
+#pragma unroll
+            for (int t = 0; t < CPW; ++t) {
+                const T xk = __shfl_sync(0xffffffffu, xr[t][G], k & 31);
+#pragma unroll
+                for (int g = 0; g < RG; ++g) xr[t][g] = fmaf(-lk[g], xk, xr[t][g]);
+            }
+        };
+        const int kmid = W < 32 ? W - 1 : 32;
+        for (int k = warp; k < kmid; ++k) step(k, std::integral_constant<int, 0>());
+        if constexpr (RG > 1)
+            for (int k = 32; k < W - 1; ++k) step(k, std::integral_constant<int, RG - 1>());
+        // Cholesky: L^{-1} = diag(1/sqrt(d)) l^{-1}.  LDL^T: l^{-1} below the
+        // diagonal (unit), 1/d on it.
+#pragma unroll
+        for (int t = 0; t < CPW; ++t) {
+            const int j = warp + 8 * t;
+#pragma unroll
+            for (int g = 0; g < RG; ++g) {
+                const int i = 32 * g + lane;
+                if (i < w && j < w) {
+                    T v;
+                    if constexpr (ldlt) v = i > j ? xr[t][g] : (i == j ? rvf[i] : (T)0);
+                    else v = i >= j ? xr[t][g] * rvf[i] : (T)0;
+                    Mi[i + j * w] = v;
+                }
+            }
+        }
+    } else {
+        // unit-lower inverse: 8 x 8 diagonal blocks first, four a warp (one a warp:
+        // as many FP64 instructions a warp, all on one unit)
+        if (tid < W) {
+            const int o = tid & ~(kDB - 1), jj = tid & (kDB - 1);
+            T xr[kDB];
+#pragma unroll
+            for (int q = 0; q < kDB; ++q) xr[q] = q == jj ? (T)1 : (T)0;
+#pragma unroll
+            for (int kk = 0; kk < kDB; ++kk) {
+                if (kk >= jj) {
+#pragma unroll
+                    for (int ii = kk + 1; ii < kDB; ++ii) xr[ii] -= x[(o + ii) + (o + kk) * LD] * xr[kk];
+                }
+            }
+            __syncwarp(W < 32 ? (1u << W) - 1u : 0xffffffffu);
+#pragma unroll
+            for (int ii = 0; ii < kDB; ++ii)
+                if (ii > jj) x[(o + ii) + (o + jj) * LD] = xr[ii];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int sz = kDB; sz < W; sz *= 2) {
+            const int npair = W / (2 * sz);
+            for (int e = tid; e < npair * sz * sz; e += NT) {
+                const int pr = e / (sz * sz), rem = e % (sz * sz), i = rem % sz, j = rem / sz;
+                const int o = pr * 2 * sz;
+                T acc = (T)0;
+                for (int k = j; k < sz; ++k) acc += x[(o + sz + i) + (o + k) * LD] * x[(o + k) + (o + j) * LD];
+                tmp[pr * sz * sz + i + j * sz] = acc;
+            }
+            __syncthreads();
+            // rows i and sz - 1 - i of a column by one thread, one after the other:
+            // sz - 1 products whatever i is, so that the lanes end together (a row a
+            // thread, a warp's loop was sz - 1 steps long for half as many of work;
+            // with the 8 x 8 blocks four a warp, 24 -> 20 us for a 64-wide inverse)
+            for (int e = tid; e < npair * sz * sz / 2; e += NT) {
+                const int pr = e / (sz * sz / 2), rem = e % (sz * sz / 2), i = rem % (sz / 2), j = rem / (sz / 2);
+                const int o = pr * 2 * sz, i2 = sz - 1 - i;
+                const T *t = tmp + pr * sz * sz + j * sz, *c = x + (o + sz) * (LD + 1);
+                T acc = t[i];                             // C^{-1} has a unit diagonal
+                for (int k = 0; k < sz - 1; ++k) {
+                    if (k == i) {
+                        x[(o + sz + i) + (o + j) * LD] = -acc;
+                        acc = t[i2];
+                    }
+                    const int kk = k < i ? k : k - i;
+                    acc += c[(k < i ? i : i2) + kk * LD] * t[kk];
+                }
+                x[(o + sz + i2) + (o + j) * LD] = -acc;
+            }
+            __syncthreads();
+        }
+        // Cholesky: L^{-1} = diag(1/sqrt(d)) l^{-1}.  LDL^T: l^{-1} below the
+        // diagonal (unit), 1/d on it.
+        for (int idx = tid; idx < w * w; idx += NT) {
+            const int i = idx % w, j = idx / w;
+            T v = (T)0;
+            if (i >= j) v = ldlt ? (i > j ? x[i + j * LD] : rvf[i]) : x[i + j * LD] * rvf[i];
+            Mi[idx] = v;
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
 // Diagonal block of width <= W (W = 16, 32, 64; the block is padded with the
 // identity to W).  On this part a warp issues one FP64 instruction per ~64
 // cycles and the SM as a whole one per ~19 (conversions included), so the
@@ -190,11 +317,7 @@ __device__ __forceinline__ double shfl_d(double v, int src)
 //    path for W = 64, where nothing else runs);
 //  * pivot tests and FP64 <-> FP32 conversions on the bit patterns;
 //  * L = l diag(sqrt(d)) is formed afterwards, all columns in parallel;
-//  * L^{-1} = diag(1/sqrt(d)) l^{-1}: FP32 factors invert the unit-lower l
-//    by forward substitution in registers (warp v owns columns v, v + 8, ...);
-//    FP64 factors by blocks (8 x 8 diagonal blocks by single lanes, then
-//    pairs of blocks merged with X21 = -C^{-1} (B A^{-1})), which does a
-//    sixth of the multiply-adds.
+//  * L^{-1} = diag(1/sqrt(d)) l^{-1} by invert_unit.
 // ---------------------------------------------------------------------------
 template <typename T, int W, bool ldlt>
 __device__ __forceinline__ void ldl_diag_block(const DevPlan &p, int pid, T *__restrict__ L,
@@ -441,104 +564,7 @@ __device__ __forceinline__ void ldl_diag_block(const DevPlan &p, int pid, T *__r
     if constexpr (kExps && ldlt)
         if (rowexp && tid < w) rowexp[col0 + tid] = rmax[tid];
 
-    T *Mi = Dinv + p.pinv[pid];
-    if constexpr (std::is_same<T, float>::value) {
-        // forward substitution in registers: warp v owns columns v, v + 8, ...
-        // of X = l^{-1}, W / 32 rows per lane; at step k the lane holding row
-        // k broadcasts x_k and every lane subtracts l(i, k) x_k.  The k loop
-        // is split at the row-group boundary so that the broadcast reads a
-        // fixed register.
-        constexpr int CPW = W / 8;
-        constexpr int RG = (W + 31) / 32;
-        T xr[CPW][RG];
-#pragma unroll
-        for (int t = 0; t < CPW; ++t)
-#pragma unroll
-            for (int g = 0; g < RG; ++g) xr[t][g] = (32 * g + lane == warp + 8 * t) ? (T)1 : (T)0;
-        auto step = [&](int k, auto gk) {
-            constexpr int G = decltype(gk)::value;
-            T lk[RG];
-#pragma unroll
-            for (int g = 0; g < RG; ++g) {
-                const int i = 32 * g + lane;
-                const T v = x[min(i, W - 1) + k * LD];
-                lk[g] = (i > k && i < W) ? v : (T)0;
-            }
-#pragma unroll
-            for (int t = 0; t < CPW; ++t) {
-                const T xk = __shfl_sync(0xffffffffu, xr[t][G], k & 31);
-#pragma unroll
-                for (int g = 0; g < RG; ++g) xr[t][g] = fmaf(-lk[g], xk, xr[t][g]);
-            }
-        };
-        const int kmid = W < 32 ? W - 1 : 32;
-        for (int k = warp; k < kmid; ++k) step(k, std::integral_constant<int, 0>());
-        if constexpr (RG > 1)
-            for (int k = 32; k < W - 1; ++k) step(k, std::integral_constant<int, RG - 1>());
-        // Cholesky: L^{-1} = diag(1/sqrt(d)) l^{-1}.  LDL^T: l^{-1} below the
-        // diagonal (unit), 1/d on it.
-#pragma unroll
-        for (int t = 0; t < CPW; ++t) {
-            const int j = warp + 8 * t;
-#pragma unroll
-            for (int g = 0; g < RG; ++g) {
-                const int i = 32 * g + lane;
-                if (i < w && j < w) {
-                    T v;
-                    if constexpr (ldlt) v = i > j ? xr[t][g] : (i == j ? rvf[i] : (T)0);
-                    else v = i >= j ? xr[t][g] * rvf[i] : (T)0;
-                    Mi[i + j * w] = v;
-                }
-            }
-        }
-    } else {
-        // unit-lower inverse: 8 x 8 diagonal blocks first
-        if (warp < W / kDB && lane < kDB) {
-            const int o = warp * kDB, jj = lane;
-            T xr[kDB];
-#pragma unroll
-            for (int q = 0; q < kDB; ++q) xr[q] = q == jj ? (T)1 : (T)0;
-#pragma unroll
-            for (int kk = 0; kk < kDB; ++kk) {
-                if (kk >= jj) {
-#pragma unroll
-                    for (int ii = kk + 1; ii < kDB; ++ii) xr[ii] -= x[(o + ii) + (o + kk) * LD] * xr[kk];
-                }
-            }
-            __syncwarp(0xffu);
-#pragma unroll
-            for (int ii = 0; ii < kDB; ++ii)
-                if (ii > jj) x[(o + ii) + (o + jj) * LD] = xr[ii];
-        }
-        __syncthreads();
-#pragma unroll
-        for (int sz = kDB; sz < W; sz *= 2) {
-            const int npair = W / (2 * sz);
-            for (int e = tid; e < npair * sz * sz; e += NT) {
-                const int pr = e / (sz * sz), rem = e % (sz * sz), i = rem % sz, j = rem / sz;
-                const int o = pr * 2 * sz;
-                T acc = (T)0;
-                for (int k = j; k < sz; ++k) acc += x[(o + sz + i) + (o + k) * LD] * x[(o + k) + (o + j) * LD];
-                tmp[pr * sz * sz + i + j * sz] = acc;
-            }
-            __syncthreads();
-            for (int e = tid; e < npair * sz * sz; e += NT) {
-                const int pr = e / (sz * sz), rem = e % (sz * sz), i = rem % sz, j = rem / sz;
-                const int o = pr * 2 * sz;
-                T acc = tmp[pr * sz * sz + i + j * sz];   // C^{-1} has a unit diagonal
-                for (int k = 0; k < i; ++k) acc += x[(o + sz + i) + (o + sz + k) * LD] * tmp[pr * sz * sz + k + j * sz];
-                x[(o + sz + i) + (o + j) * LD] = -acc;
-            }
-            __syncthreads();
-        }
-        // Cholesky: L^{-1} = diag(1/sqrt(d)) l^{-1}.  LDL^T: l^{-1} below the
-        // diagonal (unit), 1/d on it.
-        for (int idx = tid; idx < w * w; idx += NT) {
-            const int i = idx % w, j = idx / w;
-            if constexpr (ldlt) Mi[idx] = i > j ? x[i + j * LD] : (i == j ? rvf[i] : (T)0);
-            else Mi[idx] = i >= j ? x[i + j * LD] * rvf[i] : (T)0;
-        }
-    }
+    invert_unit<T, W, ldlt>(x, tmp, rvf, Dinv + p.pinv[pid], w);
 }
 
 template <typename T, int W>

@@ -352,8 +352,9 @@ __device__ void potrf_block(const DevPlan &p, int pid, T *__restrict__ L, T *__r
     for (int idx = tid; idx < w * w; idx += nt) Mi[idx] = a[idx];
 }
 
-// Cholesky diagonal blocks wider than 64, one CTA per panel: in fixed point, or
-// where that cannot hold the block, in FP64.
+// Cholesky diagonal blocks wider than 64, one CTA per panel: in fixed point (the
+// inverse from the stored factor where fixed point cannot hold it), or where that
+// cannot hold the block, in FP64.
 template <typename T>
 __global__ void __launch_bounds__(256) potrf_wide_kernel(DevPlan p, const int32_t *__restrict__ panels,
                                                          T *__restrict__ L, T *__restrict__ Dinv,
@@ -363,11 +364,26 @@ __global__ void __launch_bounds__(256) potrf_wide_kernel(DevPlan p, const int32_
     extern __shared__ double sm[];
     const int pid = panels[blockIdx.x];
     const int w = p.pw[pid], h = p.ph[pid];
-    if (w <= fx::kMaxW && fx::diag_block<T, 2>(L + p.pval[pid], Dinv + p.pinv[pid], w, h,
-                                               reinterpret_cast<unsigned char *>(sm),
-                                               rowexp ? rowexp + p.pfcol[pid] : nullptr))
-        return;
-    __syncthreads();
+    if (w <= fx::kMaxW) {
+        const T *D = L + p.pval[pid];
+        T *Mi = Dinv + p.pinv[pid];
+        const fx::Outcome r = fx::diag_block<T, 2>(L + p.pval[pid], Mi, w, h, reinterpret_cast<unsigned char *>(sm),
+                                                   rowexp ? rowexp + p.pfcol[pid] : nullptr);
+        if (r == fx::kDone) return;
+        __syncthreads();
+        if (r == fx::kNoInverse) {
+            T *a = reinterpret_cast<T *>(sm);
+            const int tid = threadIdx.x, nt = blockDim.x;
+            for (int idx = tid; idx < w * w; idx += nt) {
+                const int i = idx % w, j = idx / w;
+                a[idx] = i >= j ? __ldcg(D + i + (int64_t)j * h) : (T)0;
+            }
+            __syncthreads();
+            invert_lower_blocked<T>(a, w, a + (size_t)w * w);
+            for (int idx = tid; idx < w * w; idx += nt) Mi[idx] = a[idx];
+            return;
+        }
+    }
     potrf_block<T>(p, pid, L, Dinv, *replace_tau_p, err_col, nrepl, sm, rowexp);
 }
 
@@ -380,8 +396,9 @@ size_t potrf_wide_smem(int wmax)
 // Cholesky diagonal blocks of 33 .. 64 columns: the same way, the block's rows
 // one a lane (64 wide: 67 -> 48 us for an FP64 factor, 51 -> 47 for FP32; up to
 // 32 columns both take the same time, 23 to 26 us, and the smaller kernel
-// stays).  What fixed
-// point cannot hold goes the FP64 way, after the time lost here.
+// stays).  A block whose inverse fixed point cannot hold has it formed from the
+// stored factor (in all 68 us for FP64, 49 for FP32); one whose factor it cannot
+// hold goes the FP64 way, after the time lost here.
 template <typename T>
 __global__ void __launch_bounds__(256) potrf_mid_kernel(DevPlan p, const int32_t *__restrict__ panels,
                                                         T *__restrict__ L, T *__restrict__ Dinv,
@@ -391,10 +408,34 @@ __global__ void __launch_bounds__(256) potrf_mid_kernel(DevPlan p, const int32_t
     extern __shared__ double sm[];
     const int pid = panels[blockIdx.x];
     const int w = p.pw[pid], h = p.ph[pid];
-    if (fx::diag_block<T, 1>(L + p.pval[pid], Dinv + p.pinv[pid], w, h, reinterpret_cast<unsigned char *>(sm),
-                             rowexp ? rowexp + p.pfcol[pid] : nullptr))
-        return;
+    const T *D = L + p.pval[pid];
+    T *Mi = Dinv + p.pinv[pid];
+    const fx::Outcome r = fx::diag_block<T, 1>(L + p.pval[pid], Mi, w, h, reinterpret_cast<unsigned char *>(sm),
+                                               rowexp ? rowexp + p.pfcol[pid] : nullptr);
+    if (r == fx::kDone) return;
     __syncthreads();
+    if (r == fx::kNoInverse) {
+        // the factor's unit-lower part and its diagonal's reciprocals, as ldl_diag_block leaves them
+        constexpr int W = 64, LD = W + 1;
+        T *x = reinterpret_cast<T *>(sm), *tmp = x + W * LD, *rvf = tmp + (W / 2) * (W / 2);
+        const int tid = threadIdx.x, i = tid % W, j0 = tid / W;
+        T v[W / 4];
+#pragma unroll
+        for (int q = 0; q < W / 4; ++q) {
+            const int j = j0 + 4 * q;
+            v[q] = i > j && i < w ? __ldcg(D + i + (int64_t)j * h) : (i == j ? (T)1 : (T)0);
+        }
+        if (tid < W) rvf[tid] = tid < w ? rcp_newton(__ldcg(D + tid + (int64_t)tid * h)) : (T)1;
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < W / 4; ++q) {
+            const int j = j0 + 4 * q;
+            x[i + j * LD] = i > j ? v[q] * rvf[j] : v[q];
+        }
+        __syncthreads();
+        invert_unit<T, W, false>(x, tmp, rvf, Mi, w);
+        return;
+    }
     ldl_diag_block<T, 64, false>(p, pid, L, Dinv, *replace_tau_p, err_col, nrepl, nullptr, sm, rowexp);
 }
 

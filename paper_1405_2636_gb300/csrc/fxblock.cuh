@@ -20,13 +20,18 @@
 // a 64^3 grid amplifies a thousandfold): those are summed beside it (low).
 //
 // What fixed point cannot hold is left to the floating-point path: the
-// function changes nothing and returns false when an entry is not finite,
-// when |a_ij| or an entry of L breaks its bound (not positive definite), when
+// function changes nothing and returns kRefused when an entry is not finite,
+// when |a_ij| or an entry of L breaks its bound (not positive definite), or when
 // a pivot falls below 2^-44 of its bound (it is zero, negative, or so small
-// that static replacement may apply), or when an entry of X reaches 8.
+// that static replacement may apply).  When an entry of X reaches 8, which
+// ordinary blocks do (12 on a plate's separator, 48 with coefficients spread over
+// e^4), L is as good as ever: it is stored, the caller forms the inverse alone in
+// floating point, and kNoInverse says so.
 //
-// A 64-wide FP64 block takes 48 us (FP64 unit: 67), FP32 47 (51; both start as
-// the same integers); 128 wide 0.18 ms (0.54 on the FP64 unit).  What bounds it: per 8 columns about 6,600 cycles of one warp's
+// A 64-wide FP64 block takes 49 us (FP64 unit: 69), FP32 47 (53; both start as
+// the same integers); 128 wide 0.18 ms (0.58 on the FP64 unit).  With the inverse
+// in floating point 68 us and 49, 0.40 ms and 0.25 (the whole block a second time
+// on the FP64 unit: 111 and 92, 0.74 and 0.60).  What bounds it: per 8 columns about 6,600 cycles of one warp's
 // dependent instructions, a third of them the reciprocal square roots.
 #pragma once
 
@@ -48,7 +53,7 @@ __host__ __device__ constexpr int width8(int w) { return (w + 7) & ~7; }
 __host__ __device__ constexpr size_t smem_bytes(int wmax)
 {
     return (size_t)8 * (width8(wmax) + 1) * (width8(wmax) + 1) + (size_t)3 * 8 * kDB * width8(wmax) +
-           (size_t)width8(wmax) * (8 + 4 + 4 + 4 + 4);
+           (size_t)width8(wmax) * (8 + 4 + 4 + 4 + 4) + 16;
 }
 constexpr int kFX = 56;                    // entries of X: x 2^56, |x| < 8
 constexpr long long kMaxX = 1LL << (kFX + 3);
@@ -361,16 +366,19 @@ __device__ __forceinline__ void bar_some(int threads)
 }
 
 // The whole block: L over its lower triangle, L^{-1} at Mi (w x w, zeros
-// above).  All 256 threads; false (and nothing written) when the block has to
-// go the floating-point way.  While the chain of block column b runs on up to
+// above).  All 256 threads.  While the chain of block column b runs on up to
 // three warps (NR = 2 rows a lane: four), the others finish the rank-8 update
 // of block column b - 1 and extend the inverse by its block row.  What a thread
-// finds wrong stays its own (bad) until a barrier joins all threads' flags, so
-// that all leave at the same barrier: a shared flag, read behind one barrier,
-// could already hold what a faster warp finds before the next.
+// finds stays its own until a barrier joins all threads' words, so that all leave
+// at the same barrier: a shared flag, read behind one barrier, could already hold
+// what a faster warp finds before the next.  (leave_out is such a flag and decides
+// nothing: it saves work on an inverse that is not used, between barriers that
+// every thread passes.)
 // rowexp (or null): the exponents of about sqrt(a_ii).
+enum Outcome { kRefused, kNoInverse, kDone };
+enum Found : int { kBad = 1, kWideInv = 2 };
 template <typename T, int NR>
-__device__ bool diag_block(T *__restrict__ D, T *__restrict__ Mi, int w, int h, unsigned char *smraw, int32_t *rowexp)
+__device__ Outcome diag_block(T *__restrict__ D, T *__restrict__ Mi, int w, int h, unsigned char *smraw, int32_t *rowexp)
 {
     const int W8 = width8(w), LD = W8 + 1, nb = W8 / kDB;
     long long *a = reinterpret_cast<long long *>(smraw);
@@ -382,17 +390,19 @@ __device__ bool diag_block(T *__restrict__ D, T *__restrict__ Mi, int w, int h, 
     float *rowsum = reinterpret_cast<float *>(sc + W8);
     float *low = rowsum + W8;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    bool bad = false;
+    volatile int *leave_out = reinterpret_cast<int *>(low + W8);   // a thread saw kWideInv: no more of the inverse
+    int found = 0;
 
+    if (tid == 0) *leave_out = 0;
     if (tid < W8) {
         int s = 0;
         float diag = 1.0f;
         if (tid < w) {
             const Fields<T> d(__ldcg(D + tid + (int64_t)tid * h));
             const int ef = d.top();          // the exponent alone for a positive d
-            bad = ef < Fields<T>::kMin || ef > Fields<T>::kMax;
+            found = ef < Fields<T>::kMin || ef > Fields<T>::kMax ? kBad : 0;
             s = (ef - Fields<T>::kOne) >> 1;
-            if (rowexp) rowexp[tid] = s;
+            if (sizeof(T) == 8 && rowexp) rowexp[tid] = s;   // (FP64 factors only)
             diag = __uint_as_float(((unsigned)(127 + ((ef - Fields<T>::kOne) & 1)) << 23) | d.mant23());
         }
         sc[tid] = s;
@@ -425,7 +435,7 @@ __device__ bool diag_block(T *__restrict__ D, T *__restrict__ Mi, int w, int h, 
                     const Fields<T> x(v[u]);
                     const unsigned long long m = x.mant();
                     const int n = si + sc[j] + Fields<T>::kBias - kFA - x.exp();   // m 2^-n
-                    bad = bad || (m != 0 && n < 1);    // 4 or more, infinite or NaN
+                    found |= m != 0 && n < 1 ? kBad : 0;   // 4 or more, infinite or NaN
                     const long long g = (long long)((m >> min(max(n - 1, 0), 63)) + 1) >> 1, sign = x.sign();
                     f = (g ^ sign) - sign;
                 }
@@ -434,33 +444,41 @@ __device__ bool diag_block(T *__restrict__ D, T *__restrict__ Mi, int w, int h, 
         }
         a[i + W8 * LD] = 0;                            // X(W8 - 1, i)
     }
-    if (__syncthreads_or(bad)) return false;
+    if (__syncthreads_or(found)) return kRefused;
 
     // block column b of L is done: its updates past the next block column, its
     // block row of the inverse, that row's share of the sums below
     auto others = [&](int b, int wi, int nw) {
         const int2 *lb = lim + (b & 1) * kDB * W8;
         const int cols = kDB * (b + 1), nx = min(nw, (cols + 31) / 32);
-        if (wi < nx)
-            for (int j = 32 * wi + lane; j < cols; j += 32 * nx) bad |= inverse_row(a, LD, W8, b, j, lb, limx, rfix, rexp);
+        if (wi < nx && !*leave_out)
+            for (int j = 32 * wi + lane; j < cols; j += 32 * nx)
+                if (inverse_row(a, LD, W8, b, j, lb, limx, rfix, rexp)) {
+                    found |= kWideInv;
+                    *leave_out = 1;
+                }
         if (nx == nw) rank8(a, LD, W8, lb, kDB * (b + 2), W8, 32 * wi + lane, 32 * nw);
         else if (wi >= nx) rank8(a, LD, W8, lb, kDB * (b + 2), W8, 32 * (wi - nx) + lane, 32 * (nw - nx));
         bar_some(32 * nw);
-        inverse_sums(a, LD, W8, b, lb, limx, 32 * wi + lane, 32 * nw);
+        if (!*leave_out) inverse_sums(a, LD, W8, b, lb, limx, 32 * wi + lane, 32 * nw);
     };
     for (int b = 0; b < nb; ++b) {
         const int kb = kDB * b;
         int2 *lb = lim + (b & 1) * kDB * W8;
         const int nw = min(NR == 1 ? 3 : 4, max(1, (W8 - kb - kDB + 24 * NR - 1) / (24 * NR)));
-        if (warp < nw) bad |= panel<NR>(a, LD, W8, kb, warp, nw, lb, rfix, rexp, low);
+        if (warp < nw) found |= panel<NR>(a, LD, W8, kb, warp, nw, lb, rfix, rexp, low) ? kBad : 0;
         else if (b > 0) others(b - 1, warp - nw, kThreads / 32 - nw);
         __syncthreads();
-        if (kb + tid < W8) bad |= check_row(kb + tid, W8, lb, rowsum, low);
+        if (kb + tid < W8) found |= check_row(kb + tid, W8, lb, rowsum, low) ? kBad : 0;
         if (b + 1 < nb) rank8(a, LD, W8, lb, kb + kDB, kb + 2 * kDB, tid, kThreads);
-        if (__syncthreads_or(bad)) return false;
+        if (__syncthreads_or(found & kBad)) return kRefused;
     }
     others(nb - 1, warp, kThreads / 32);
-    if (__syncthreads_or(bad)) return false;
+    if (__syncthreads_or(found & kWideInv)) {
+        for (int j = warp; j < w; j += 8)
+            for (int i = j + lane; i < w; i += 32) to_value(a[i + j * LD], sc[i] - 60, D + i + (int64_t)j * h);
+        return kNoInverse;
+    }
     for (int j = warp; j < w; j += 8) {
         const int sj = sc[j];
         for (int i = lane; i < w; i += 32) {
@@ -474,7 +492,7 @@ __device__ bool diag_block(T *__restrict__ D, T *__restrict__ Mi, int w, int h, 
             Mi[i + j * w] = x;
         }
     }
-    return true;
+    return kDone;
 }
 
 }  // namespace fx

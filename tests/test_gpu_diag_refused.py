@@ -64,3 +64,24 @@ def test_refused_at_every_column(width, pivot, prec):
     X, _ = h.solve(inputs.rhs(n, 2, 1))
     assert oracle.backward_error(A, X, inputs.rhs(n, 2, 1)) <= (1e-13 if prec == "fp64" else 1e-12)
     h.free()
+
+
+@pytest.mark.parametrize("width", [40, 64])
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_wide_inverse_costs_no_second_factorization(width, prec):
+    """A block whose inverse breaks the fixed-point bound takes no longer than the
+    floating-point kernel, which LDL^T runs on the same block: at most a quarter
+    more (timing noise; a second factorization took 1.4 to 1.7 times as long)."""
+    A = sp.csc_matrix(_block(width, np.random.default_rng(width), width * 3 // 4, 0.02))
+    cp, ri, vals = inputs.csc_arrays(A)
+    ms = {}
+    for method in ("llt", "ldlt"):
+        h = spx.analyze(cp, ri, method, ordering=spx.SPX_ORDER_NATURAL, max_width=width, queue_panels=-1)
+        h.set_profiling(True)
+        t = []
+        for _ in range(40):
+            h.factorize(vals, prec)
+            t.append(h.kernel_stats()["diag"]["ms"])
+        ms[method] = np.median(t)
+        h.free()
+    assert ms["llt"] <= 1.25 * ms["ldlt"], ms
