@@ -213,6 +213,8 @@ struct spx_handle_s {
     spx::SlTile *d_sl_tiles = nullptr;
     int32_t *d_sl_small = nullptr;
     RowChunk *d_slc = nullptr;
+    spx::SlPlace *d_slplace = nullptr;   // per TRSM chunk: where its digits go
+    int64_t sl_rows = 0;                 // rows of one slice of the operand copies
     int64_t *d_colbase = nullptr, *d_relbase = nullptr;   // per operand row: where its column goes
     void *d_slop[2] = {nullptr, nullptr};
     int32_t *d_slexp[2] = {nullptr, nullptr};
@@ -1130,20 +1132,62 @@ spx_status ensure_colmaps(spx_handle h)
 }
 
 // The launch lists, operand copies and descriptors of the FP64 slices, on the
-// first FP64 factorization that wants them.  Where the copies do not fit the
-// device (1.75 times the factor's panels and the exponents), the handle stays
-// on the CUDA-core path.
+// first FP64 factorization that wants them.  The copies hold the off-diagonal
+// rows of the panels that panel_slices sends to the tensor cores, 14 bytes an
+// element of the panel's width rounded up to 16, 32 or 64 (or 64-column blocks):
+// 1.9 times the factor's panels on the 64^3 grid, LDL^T with its two copies 3.7
+// times on 32^3 x 2.  Where they do not fit the device, the handle stays on the
+// CUDA-core path.
 spx_status ensure_slices(spx_handle h)
 {
     if (h->sl_ready || h->sl_failed) return SPX_OK;
     const spx::Plan &P = h->plan;
     const int64_t rows = std::max<int64_t>(h->op_rows, 1);
     const int ncopy = P.method == SPX_LDLT ? 2 : 1;
-    if (rows * spx::kSliceCount >= INT32_MAX) {   // TMA row coordinates are 32-bit
+    // blocks of 128 rows side by side, each in the column of its class (four of 16
+    // elements, two of 32, one of 64) that is filled least
+    struct Column {
+        int64_t top;
+        int32_t chunk;
+    };
+    std::vector<Column> cls[3] = {{{0, 0}, {0, 1}, {0, 2}, {0, 3}}, {{0, 0}, {0, 2}}, {{0, 0}}};
+    auto class_of = [&](int32_t q) { return P.pw[q] <= 16 ? 0 : P.pw[q] <= 32 ? 1 : 2; };
+    struct Block {
+        int64_t row;
+        int32_t chunk, height;
+    };
+    std::vector<Block> blocks;
+    std::vector<int64_t> first(P.npanels, -1);   // a panel's first block
+    for (int32_t q = 0; q < P.npanels; ++q) {
+        if (!panel_slices(P, q)) continue;
+        first[q] = (int64_t)blocks.size();
+        std::vector<Column> &c = cls[class_of(q)];
+        for (int32_t r0 = P.pw[q]; r0 < P.ph[q]; r0 += 128) {
+            const int32_t height = std::min(128, P.ph[q] - r0);
+            Column &to = *std::min_element(c.begin(), c.end(), [](const Column &x, const Column &y) { return x.top < y.top; });
+            blocks.push_back(Block{to.top, to.chunk, height});
+            to.top += (int64_t)height * ((P.pw[q] + 63) / 64);
+        }
+    }
+    int64_t base[3], total = 0;
+    for (int k = 0; k < 3; ++k) {
+        base[k] = total;
+        int64_t most = 0;
+        for (const Column &c : cls[k]) most = std::max(most, c.top);
+        total += most;
+    }
+    total = std::max<int64_t>(total, 1);
+    if (total * spx::kSliceCount >= INT32_MAX) {   // TMA row coordinates are 32-bit
         h->sl_failed = true;
         return SPX_OK;
     }
-    const size_t bytes = (size_t)rows * spx::kSliceCount * h->kpad * 2;
+    h->sl_rows = total;
+    // rows r0 .. of panel q: the block they lie in, and their row in the copy
+    auto block_of = [&](int32_t q, int32_t r0) -> const Block & { return blocks[first[q] + (r0 - P.pw[q]) / 128]; };
+    auto row_of = [&](int32_t q, int32_t r0) {
+        return (int32_t)(base[class_of(q)] + block_of(q, r0).row + (r0 - P.pw[q]) % 128);
+    };
+    const size_t bytes = (size_t)total * spx::kSliceCount * 64 * 2;
     const size_t nexp = (size_t)rows * (h->kpad / 64);
     for (int k = 0; k < ncopy; ++k) {
         if (cudaMalloc(&h->d_slop[k], bytes) != cudaSuccess ||
@@ -1165,12 +1209,13 @@ spx_status ensure_slices(spx_handle h)
         CU(cudaMemset(h->d_slop[k], 0, bytes));
         CU(cudaMemset(h->d_slexp[k], 0, nexp * sizeof(int32_t)));
     }
-    if (spx::make_operand_map(h->tmap_sla, h->d_slop[0], rows * spx::kSliceCount, h->kpad, spx::OP_F16, 128) != 0 ||
-        spx::make_operand_map(h->tmap_slb, h->d_slop[ncopy - 1], rows * spx::kSliceCount, h->kpad, spx::OP_F16, 64) != 0)
+    if (spx::make_operand_map(h->tmap_sla, h->d_slop[0], total * spx::kSliceCount, 64, spx::OP_F16, 128) != 0 ||
+        spx::make_operand_map(h->tmap_slb, h->d_slop[ncopy - 1], total * spx::kSliceCount, 64, spx::OP_F16, 64) != 0)
         return fail(h, SPX_ERR_CUDA, "cuTensorMapEncodeTiled failed for the FP64 slices");
     std::vector<spx::SlTile> tiles;
     std::vector<int32_t> small;
     std::vector<RowChunk> chunks;
+    std::vector<spx::SlPlace> places;
     std::vector<int32_t> rowlev((size_t)rows, 0);   // level of the panel a row faces
     for (const spx::Task &tk : P.tasks)
         for (int32_t r = tk.r0; r < tk.r1; ++r) rowlev[(size_t)(P.prow[tk.src] + r)] = P.plevel[tk.tgt];
@@ -1186,8 +1231,14 @@ spx_status ensure_slices(spx_handle h)
         fs.clear();
         for (int32_t q = P.level_ptr[l]; q < P.level_ptr[l + 1]; ++q) {
             const int32_t k = P.level_panels[q], w = P.pw[k], hk = P.ph[k];
-            for (int32_t r0 = w; r0 < hk; r0 += 64) chunks.push_back(RowChunk{k, r0});
-            if (!panel_slices(P, k)) continue;
+            const bool sl = first[k] >= 0;
+            for (int32_t r0 = w; r0 < hk; r0 += 64) {
+                chunks.push_back(RowChunk{k, r0});
+                places.push_back(sl ? spx::SlPlace{row_of(k, r0), block_of(k, r0).chunk, block_of(k, r0).height,
+                                                   16 << class_of(k)}
+                                    : spx::SlPlace{-1, 0, 0, 0});
+            }
+            if (!sl) continue;
             for (int32_t n0 = w; n0 < hk; n0 += 64) {
                 const int32_t ncol = std::min(64, hk - n0);
                 bool near = false;   // rows ascend, not the levels of the panels that they face
@@ -1196,7 +1247,8 @@ spx_status ensure_slices(spx_handle h)
                     if (m0 + 128 <= n0) continue;
                     (near ? tiles : ft)
                         .push_back(spx::SlTile{(int32_t)(P.prow[k] + m0), (int32_t)(P.prow[k] + n0), w,
-                                               std::min(128, hk - m0), ncol, m0 - n0, {0, 0}});
+                                               std::min(128, hk - m0), ncol, m0 - n0, row_of(k, m0), row_of(k, n0),
+                                               block_of(k, m0).chunk, block_of(k, n0).chunk, block_of(k, n0).height, 0});
                 }
             }
         }
@@ -1212,7 +1264,8 @@ spx_status ensure_slices(spx_handle h)
     }
     spx_status st;
     if ((st = upload(h, &h->d_sl_tiles, tiles)) || (st = upload(h, &h->d_sl_small, small)) ||
-        (st = upload(h, &h->d_slc, chunks)) || (st = dalloc(h, &h->d_rowexp, (size_t)P.n)) || (st = ensure_colmaps(h)))
+        (st = upload(h, &h->d_slc, chunks)) || (st = upload(h, &h->d_slplace, places)) ||
+        (st = dalloc(h, &h->d_rowexp, (size_t)P.n)) || (st = ensure_colmaps(h)))
         return st;
     h->sl_ready = true;
     return SPX_OK;
@@ -1456,7 +1509,7 @@ void enqueue_factorization(spx_handle h, bool mixed, Marks &mk, int prec, int pa
                 const int nsc = (int)(h->slc_ptr[l + 1] - h->slc_ptr[l]);
                 spx::launch_trsm_sl(h->dp, h->d_slc + h->slc_ptr[l], nsc, (const double *)Dinv, (double *)L,
                                     (double *)W, ldlt ? spx::TRSM_LDLT : spx::TRSM_LLT, h->d_rowexp, h->d_slop[0], h->d_slop[1], h->d_slexp[0],
-                                    h->d_slexp[1], h->op_rows, h->kpad, h->d_tcerr, s);
+                                    h->d_slexp[1], h->d_slplace + h->slc_ptr[l], h->sl_rows, h->op_rows, h->d_tcerr, s);
                 cnt += nsc > 0;
                 h->class_launches[SPX_K_TRSM] += nsc > 0;
             } else if (!link) {
@@ -1476,7 +1529,7 @@ void enqueue_factorization(spx_handle h, bool mixed, Marks &mk, int prec, int pa
                 auto st = [&](int k) { return one ? one : ub.pick(k); };
                 if (slices) {
                     // far tiles (`one`) in short CTAs, so that the next levels' launches find free SMs
-                    spx::launch_update_sl(h->tmap_sla, h->tmap_slb, h->op_rows, h->dp, h->d_sl_tiles + c0, nc,
+                    spx::launch_update_sl(h->tmap_sla, h->tmap_slb, h->sl_rows, h->op_rows, h->dp, h->d_sl_tiles + c0, nc,
                                           h->d_colbase, h->d_relbase, h->d_slexp[0], h->d_slexp[ldlt ? 1 : 0], (double *)L, h->d_tcerr,
                                           one ? kFarTiles : 0, wmax, st(0));
                     mk.mark(SPX_K_UPDATE_TC);
@@ -2997,7 +3050,7 @@ spx_status spx_selected_inverse(spx_handle h, void *cuda_stream)
     spx::launch_diag_exp(h->dp, (const double *)h->d_L, h->d_dexp, h->hs);
     // (h->d_chunks: 64 rows each, as the slices TRSM takes them)
     spx::launch_trsm_sl(h->dp, h->d_chunks, (int)h->chunk_ptr[P.nlevels], (const double *)h->d_Dinv, h->d_Lh, nullptr,
-                        spx::TRSM_RIGHT_LINV, nullptr, nullptr, nullptr, nullptr, nullptr, 0, 0, h->d_tcerr, h->hs);
+                        spx::TRSM_RIGHT_LINV, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, 0, 0, h->d_tcerr, h->hs);
     spx::launch_selinv_diag(h->dp, h->d_level_panels, P.npanels, 1, wmax, 1, (const double *)h->d_Dinv, h->d_Lh,
                             h->d_Zsel, h->hs);
     // split-K so that a level keeps about two CTAs per SM busy near the root

@@ -125,25 +125,34 @@ void launch_update_tc(const void *tmap, const void *tmap_lo, int kind, const Dev
                       int *err, cudaStream_t s);
 
 // FP64 updates and TRSM on the tensor cores by error-free slices
-// (update_sl.cu).  One tile: rows arow .. of the operand copy (nrow <= 128
-// valid) against rows brow .. (ncol <= 64) of the same panel, all k columns;
-// entry (r, c), kept when r + diff >= c, goes to C[colbase[brow + c] + relmap[relbase[brow + c] + arow + r]].
+// (update_sl.cu).  One tile: rows arow .. of one panel (nrow <= 128; numbered over
+// all panels, as prow does) against rows brow .. (ncol <= 64) of the same panel,
+// all k columns; entry (r, c), kept when r + diff >= c, goes to
+// C[colbase[brow + c] + relmap[relbase[brow + c] + arow + r]].  In the operand copy
+// the rows lie from row aop / bop on, columns from 16 achunk / 16 bchunk; further
+// digit blocks (panels wider than 64) nrow / bstep rows on each.
 struct __align__(16) SlTile {
     int32_t arow, brow, k, nrow;
-    int32_t ncol, diff, pad[2];
+    int32_t ncol, diff, aop, bop;
+    int32_t achunk, bchunk, bstep, pad;
+};
+// Where 64 rows of a panel lie in the operand copy: row -1: nowhere; cols: columns
+// that are kept (16, 32 or 64), step: rows between digit blocks.
+struct __align__(16) SlPlace {
+    int32_t row, chunk, step, cols;
 };
 constexpr int kSliceCount = 7;
-// oprows: rows of one slice of the operand copy; per_cta > 0: at most that
+// oprows: rows of one slice of the operand copy; exprows: of the exponents; per_cta > 0: at most that
 // many tiles a CTA (a launch that others run beside), else one CTA an SM.
 // wmax: at least the width of every tile's panel.
-void launch_update_sl(const void *mapa, const void *mapb, int64_t oprows, const DevPlan &p, const SlTile *tiles,
-                      int count, const int64_t *colbase, const int64_t *relbase, const int32_t *expa, const int32_t *expb, double *C, int *err, int per_cta,
+void launch_update_sl(const void *mapa, const void *mapb, int64_t oprows, int64_t exprows, const DevPlan &p,
+                      const SlTile *tiles, int count, const int64_t *colbase, const int64_t *relbase, const int32_t *expa, const int32_t *expb, double *C, int *err, int per_cta,
                       int wmax, cudaStream_t s);
-// chunks: 64 rows each.  LDL^T: opa / expa hold L, opb / expb D L^T.  rowexp: the
+// chunks: 64 rows each, places: theirs.  LDL^T: opa / expa hold L, opb / expb D L^T.  rowexp: the
 // columns' scales (launch_potrf; TRSM_RIGHT_LINV needs none).
 void launch_trsm_sl(const DevPlan &p, const RowChunk *chunks, int count, const double *Dinv, double *X, double *Wout,
-                    int mode, const int32_t *rowexp, void *opa, void *opb, int32_t *expa, int32_t *expb, int64_t oprows, int kpad, int *err,
-                    cudaStream_t s);
+                    int mode, const int32_t *rowexp, void *opa, void *opb, int32_t *expa, int32_t *expb,
+                    const SlPlace *places, int64_t oprows, int64_t exprows, int *err, cudaStream_t s);
 // Selected inversion's Z_RJ (update_sl.cu): chunks of 128 rows; colbase,
 // relbase: where each off-diagonal row's column lies, as in launch_update_sl;
 // dexp: leading exponents of L's diagonal by column (launch_diag_exp).

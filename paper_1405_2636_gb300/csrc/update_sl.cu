@@ -2,11 +2,15 @@
 // and 3, Sec. V-B) on the FP16 tensor cores by error-free slices
 // (slices.cuh), for Cholesky and LDL^T factors in FP64.
 //
-// Operand copy: slice s of row r of panel p is a K-major FP16 row at operand
-// row s * rows + prow[p] + r, kpad elements, in digit blocks of 64 columns;
-// each (row, block) has its own exponent at exp[block * rows + prow[p] + r].
-// The TRSM writes it; the update loads 128-row (A) and 64-row (B) boxes of it
-// by TMA with the 128-byte swizzle.
+// Operand copy, of the off-diagonal rows of the panels whose updates run here,
+// in blocks of 128 rows by 64 columns (digit blocks): an array of K-major FP16
+// rows of 64 elements (128 bytes), slice s of it from row s * oprows on.  A block
+// of a panel at most 32 or 16 columns wide takes half or a quarter of the row
+// (columns 16 * chunk on), beside other blocks: SlPlace says where.  Each (row,
+// digit block) has its own exponent at exp[block * exprows + prow[p] + r].  The
+// TRSM writes the copy; the update loads 128-row (A) and 64-row (B) boxes of it by
+// TMA with the 128-byte swizzle, whole rows whatever the width, and its MMAs start
+// at the chunk.
 #include "blocks.cuh"
 #include "slices.cuh"
 
@@ -57,7 +61,7 @@ __device__ __forceinline__ int slot_of(int s, int lt) { return (s < 2 && (lt & 1
 template <bool kWide>
 __global__ void __launch_bounds__(kSlThreads, 1)
     update_sl_kernel(const __grid_constant__ CUtensorMap mapa, const __grid_constant__ CUtensorMap mapb,
-                     int64_t oprows, const SlTile *__restrict__ tiles, int count, const int64_t *__restrict__ colbase,
+                     int64_t oprows, int64_t exprows, const SlTile *__restrict__ tiles, int count, const int64_t *__restrict__ colbase,
                      const int64_t *__restrict__ relbase, const int32_t *__restrict__ relmap,
                      const int32_t *__restrict__ expa, const int32_t *__restrict__ expb, double *__restrict__ C,
                      int *err)
@@ -112,8 +116,10 @@ __global__ void __launch_bounds__(kSlThreads, 1)
                         }
                         unsigned char *dst = base + slot * kSlotBytes;
                         mbar_expect_tx(&full[slot], kSlotBytes);
-                        tma_load_2d(dst, &mapa, &full[slot], kx, (int)(s * oprows) + tl.arow);
-                        tma_load_2d(dst + kABytes, &mapb, &full[slot], kx, (int)(s * oprows) + tl.brow);
+                        const int ra = tl.aop + (kWide ? kx / kK * tl.nrow : 0);
+                        const int rb = tl.bop + (kWide ? kx / kK * tl.bstep : 0);
+                        tma_load_2d(dst, &mapa, &full[slot], 0, (int)(s * oprows) + ra);
+                        tma_load_2d(dst + kABytes, &mapb, &full[slot], 0, (int)(s * oprows) + rb);
                     }
                 }
             }
@@ -130,6 +136,7 @@ __global__ void __launch_bounds__(kSlThreads, 1)
                 for (int kx = 0; kx == 0 || (kWide && kx < tl.k && ok); kx += kK, ++lt) {
                     const uint32_t idesc = idesc_f16((tl.ncol + 15) & ~15);
                     const int ksteps = (min(kK, tl.k - kx) + 15) / 16;
+                    const uint64_t da0 = desc0 + (uint32_t)(2 * tl.achunk), db0 = desc0 + (uint32_t)(2 * tl.bchunk);
                     auto arrived = [&](int s) {
                         return mbar_wait_or(&full[slot_of(s, lt)], (uint32_t)(s < 2 ? lt >> 1 : lt) & 1u, &s_fail);
                     };
@@ -144,8 +151,8 @@ __global__ void __launch_bounds__(kSlThreads, 1)
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                         uint32_t more = 0;
                         auto pair = [&](int s, int u) {
-                            const uint64_t da = desc0 + (uint32_t)(slot_of(s, lt) * (kSlotBytes >> 4));
-                            const uint64_t db = desc0 + (uint32_t)(slot_of(u, lt) * (kSlotBytes >> 4) + (kABytes >> 4));
+                            const uint64_t da = da0 + (uint32_t)(slot_of(s, lt) * (kSlotBytes >> 4));
+                            const uint64_t db = db0 + (uint32_t)(slot_of(u, lt) * (kSlotBytes >> 4) + (kABytes >> 4));
                             mma<1>(acc, da, db, idesc, more);
                             if (ksteps > 1) mma<1>(acc, da + 2, db + 2, idesc, 1);
                             if (ksteps > 2) mma<1>(acc, da + 4, db + 4, idesc, 1);
@@ -219,7 +226,7 @@ __global__ void __launch_bounds__(kSlThreads, 1)
                 ++ng;
             };
             for (int kx = 0; kx == 0 || (kWide && kx < cur.k); kx += kK) {
-                const int64_t blk = kWide ? (int64_t)(kx / kK) * oprows : 0;
+                const int64_t blk = kWide ? (int64_t)(kx / kK) * exprows : 0;
                 if (lane < kEC) s_eb[warp][lane] = expb[blk + cur.brow + min(kEC * part + lane, cur.ncol - 1)];
                 const int32_t ea = row_ok ? expa[blk + cur.arow + r] : 0;
                 __syncwarp();
@@ -356,8 +363,8 @@ __global__ void __launch_bounds__(kTrThreads, 1)
     trsm_sl_kernel(DevPlan p, const RowChunk *__restrict__ chunks, const double *__restrict__ Dinv,
                    double *__restrict__ X, double *__restrict__ Wout, int mode, const int32_t *__restrict__ rowexp,
                    __half *__restrict__ opa,
-                   __half *__restrict__ opb, int32_t *__restrict__ expa, int32_t *__restrict__ expb, int64_t oprows,
-                   int kpad, int *err)
+                   __half *__restrict__ opb, int32_t *__restrict__ expa, int32_t *__restrict__ expb,
+                   const SlPlace *__restrict__ places, int64_t oprows, int64_t exprows, int *err)
 {
     extern __shared__ unsigned char smraw[];
     unsigned char *base =
@@ -372,6 +379,7 @@ __global__ void __launch_bounds__(kTrThreads, 1)
     __shared__ int s_sd[kK];                          // and LDL^T's of the operand copies'
     const RowChunk ch = chunks[blockIdx.x];
     const bool ldlt = mode == TRSM_LDLT, right = mode == TRSM_RIGHT_LINV;
+    const SlPlace at = right ? SlPlace{-1, 0, 0, 0} : places[blockIdx.x];
     const int pid = ch.panel, w = p.pw[pid], h = p.ph[pid];
     const int nr = min(kTrRows, h - ch.r0);
     double *Xg = X + p.pval[pid] + ch.r0;
@@ -516,7 +524,7 @@ __global__ void __launch_bounds__(kTrThreads, 1)
                 else if (row_ok) dst[(int64_t)q * h] = out[q];
                 f = max(f, exp_field(out[q], sc[q]));
             }
-            if (right) continue;   // no operand copy
+            if (at.row < 0) continue;   // no operand copy
             s_f[0][part][r] = f;
             __syncthreads();
 #pragma unroll
@@ -524,13 +532,15 @@ __global__ void __launch_bounds__(kTrThreads, 1)
             __syncthreads();
             if (row_ok) {
                 const int64_t orow = p.prow[pid] + ch.r0 + r;
-                if (part == 0) (o == 1 ? expb : expa)[(int64_t)(c0 / kK) * oprows + orow] = row_exp(f);
+                if (part == 0) (o == 1 ? expb : expa)[(int64_t)(c0 / kK) * exprows + orow] = row_exp(f);
+                if (kTC * part >= at.cols) continue;
                 uint32_t wd[kSlices][4];
                 digits8(out, f, wd, sc);
-                __half *op = (o == 1 ? opb : opa) + orow * kpad + j0;
+                __half *op = (o == 1 ? opb : opa) + ((int64_t)at.row + r + c0 / kK * at.step) * kK + 16 * at.chunk +
+                             kTC * part;
 #pragma unroll
                 for (int s = 0; s < kSlices; ++s)
-                    *reinterpret_cast<uint4 *>(op + (int64_t)s * oprows * kpad) =
+                    *reinterpret_cast<uint4 *>(op + (int64_t)s * oprows * kK) =
                         make_uint4(wd[s][0], wd[s][1], wd[s][2], wd[s][3]);
             }
         }
@@ -918,8 +928,8 @@ __global__ void __launch_bounds__(256) update_small_kernel(DevPlan p, const DevT
 
 }  // namespace
 
-void launch_update_sl(const void *mapa, const void *mapb, int64_t oprows, const DevPlan &p, const SlTile *tiles,
-                      int count, const int64_t *colbase, const int64_t *relbase, const int32_t *expa,
+void launch_update_sl(const void *mapa, const void *mapb, int64_t oprows, int64_t exprows, const DevPlan &p,
+                      const SlTile *tiles, int count, const int64_t *colbase, const int64_t *relbase, const int32_t *expa,
                       const int32_t *expb, double *C, int *err, int per_cta, int wmax, cudaStream_t s)
 {
     if (count <= 0) return;
@@ -937,16 +947,16 @@ void launch_update_sl(const void *mapa, const void *mapb, int64_t oprows, const 
     const CUtensorMap &ma = *reinterpret_cast<const CUtensorMap *>(mapa);
     const CUtensorMap &mb = *reinterpret_cast<const CUtensorMap *>(mapb);
     if (wmax > kK)
-        update_sl_kernel<true><<<grid, kSlThreads, kSlSmem, s>>>(ma, mb, oprows, tiles, count, colbase, relbase,
+        update_sl_kernel<true><<<grid, kSlThreads, kSlSmem, s>>>(ma, mb, oprows, exprows, tiles, count, colbase, relbase,
                                                                  p.relmap, expa, expb, C, err);
     else
-        update_sl_kernel<false><<<grid, kSlThreads, kSlSmem, s>>>(ma, mb, oprows, tiles, count, colbase, relbase,
+        update_sl_kernel<false><<<grid, kSlThreads, kSlSmem, s>>>(ma, mb, oprows, exprows, tiles, count, colbase, relbase,
                                                                   p.relmap, expa, expb, C, err);
 }
 
 void launch_trsm_sl(const DevPlan &p, const RowChunk *chunks, int count, const double *Dinv, double *X, double *Wout,
-                    int mode, const int32_t *rowexp, void *opa, void *opb, int32_t *expa, int32_t *expb, int64_t oprows, int kpad, int *err,
-                    cudaStream_t s)
+                    int mode, const int32_t *rowexp, void *opa, void *opb, int32_t *expa, int32_t *expb,
+                    const SlPlace *places, int64_t oprows, int64_t exprows, int *err, cudaStream_t s)
 {
     if (count <= 0) return;
     static bool once = false;
@@ -955,7 +965,7 @@ void launch_trsm_sl(const DevPlan &p, const RowChunk *chunks, int count, const d
         once = true;
     }
     trsm_sl_kernel<<<count, kTrThreads, kTrSmem, s>>>(p, chunks, Dinv, X, Wout, mode, rowexp, (__half *)opa, (__half *)opb,
-                                                      expa, expb, oprows, kpad, err);
+                                                      expa, expb, places, oprows, exprows, err);
 }
 
 void launch_selinv_sl(const DevPlan &p, const RowChunk *chunks, int count, int nsplit, const int64_t *colbase,
