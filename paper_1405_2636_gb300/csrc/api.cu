@@ -313,12 +313,46 @@ spx_status fail(spx_handle h, spx_status st, const std::string &msg)
             return fail(h, SPX_ERR_CUDA, std::string(#call) + ": " + cudaGetErrorString(e_)); \
     } while (0)
 
+void dfree(spx_handle h, void *p)
+{
+    if (!p) return;
+    cudaFree(p);
+    auto it = std::find(h->allocs.begin(), h->allocs.end(), p);
+    if (it != h->allocs.end()) h->allocs.erase(it);
+}
+
+// Gives back the operand copies of the FP64 slices (ensure_slices): a
+// factorization writes them and only it reads them, so between factorizations
+// they are memory that may be lent.
+bool drop_slices(spx_handle h)
+{
+    if (!h->sl_ready) return false;
+    cudaStreamSynchronize(h->hs);
+    if (h->fgraph && h->fgraph_prec == SPX_FP64) {   // it holds their addresses
+        cudaGraphExecDestroy(h->fgraph);
+        h->fgraph = nullptr;
+        h->fgraph_prec = -1;
+    }
+    for (int k = 0; k < 2; ++k) {
+        dfree(h, h->d_slop[k]);
+        dfree(h, h->d_slexp[k]);
+        h->d_slop[k] = nullptr;
+        h->d_slexp[k] = nullptr;
+    }
+    h->sl_ready = false;
+    return true;
+}
+
 template <typename T>
 spx_status dalloc(spx_handle h, T **p, size_t count)
 {
     *p = nullptr;
     if (count == 0) count = 1;
     cudaError_t e = cudaMalloc((void **)p, count * sizeof(T));
+    if (e == cudaErrorMemoryAllocation && drop_slices(h)) {
+        cudaGetLastError();
+        e = cudaMalloc((void **)p, count * sizeof(T));
+    }
     if (e != cudaSuccess) {
         *p = nullptr;
         return fail(h, SPX_ERR_ALLOC, std::string("cudaMalloc: ") + cudaGetErrorString(e));
@@ -334,14 +368,6 @@ spx_status upload(spx_handle h, T **p, const std::vector<T> &v)
     if (st != SPX_OK) return st;
     if (!v.empty()) CU(cudaMemcpy(*p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice));
     return SPX_OK;
-}
-
-void dfree(spx_handle h, void *p)
-{
-    if (!p) return;
-    cudaFree(p);
-    auto it = std::find(h->allocs.begin(), h->allocs.end(), p);
-    if (it != h->allocs.end()) h->allocs.erase(it);
 }
 
 // --- small device helpers ---------------------------------------------------
@@ -1136,14 +1162,12 @@ spx_status ensure_colmaps(spx_handle h)
 // rows of the panels that panel_slices sends to the tensor cores, 14 bytes an
 // element of the panel's width rounded up to 16, 32 or 64 (or 64-column blocks):
 // 1.9 times the factor's panels on the 64^3 grid, LDL^T with its two copies 3.7
-// times on 32^3 x 2.  Where they do not fit the device, the handle stays on the
-// CUDA-core path.
-spx_status ensure_slices(spx_handle h)
+// times on 32^3 x 2.
+spx_status build_slices(spx_handle h)
 {
-    if (h->sl_ready || h->sl_failed) return SPX_OK;
+    if (h->sl_rows > 0) return SPX_OK;
     const spx::Plan &P = h->plan;
     const int64_t rows = std::max<int64_t>(h->op_rows, 1);
-    const int ncopy = P.method == SPX_LDLT ? 2 : 1;
     // blocks of 128 rows side by side, each in the column of its class (four of 16
     // elements, two of 32, one of 64) that is filled least
     struct Column {
@@ -1181,37 +1205,11 @@ spx_status ensure_slices(spx_handle h)
         h->sl_failed = true;
         return SPX_OK;
     }
-    h->sl_rows = total;
     // rows r0 .. of panel q: the block they lie in, and their row in the copy
     auto block_of = [&](int32_t q, int32_t r0) -> const Block & { return blocks[first[q] + (r0 - P.pw[q]) / 128]; };
     auto row_of = [&](int32_t q, int32_t r0) {
         return (int32_t)(base[class_of(q)] + block_of(q, r0).row + (r0 - P.pw[q]) % 128);
     };
-    const size_t bytes = (size_t)total * spx::kSliceCount * 64 * 2;
-    const size_t nexp = (size_t)rows * (h->kpad / 64);
-    for (int k = 0; k < ncopy; ++k) {
-        if (cudaMalloc(&h->d_slop[k], bytes) != cudaSuccess ||
-            cudaMalloc((void **)&h->d_slexp[k], nexp * sizeof(int32_t)) != cudaSuccess) {
-            cudaGetLastError();
-            for (int j = 0; j < 2; ++j) {
-                cudaFree(h->d_slop[j]);
-                cudaFree(h->d_slexp[j]);
-                h->d_slop[j] = nullptr;
-                h->d_slexp[j] = nullptr;
-            }
-            h->sl_failed = true;
-            return SPX_OK;
-        }
-    }
-    for (int k = 0; k < ncopy; ++k) {
-        h->allocs.push_back(h->d_slop[k]);
-        h->allocs.push_back(h->d_slexp[k]);
-        CU(cudaMemset(h->d_slop[k], 0, bytes));
-        CU(cudaMemset(h->d_slexp[k], 0, nexp * sizeof(int32_t)));
-    }
-    if (spx::make_operand_map(h->tmap_sla, h->d_slop[0], total * spx::kSliceCount, 64, spx::OP_F16, 128) != 0 ||
-        spx::make_operand_map(h->tmap_slb, h->d_slop[ncopy - 1], total * spx::kSliceCount, 64, spx::OP_F16, 64) != 0)
-        return fail(h, SPX_ERR_CUDA, "cuTensorMapEncodeTiled failed for the FP64 slices");
     std::vector<spx::SlTile> tiles;
     std::vector<int32_t> small;
     std::vector<RowChunk> chunks;
@@ -1267,7 +1265,65 @@ spx_status ensure_slices(spx_handle h)
         (st = upload(h, &h->d_slc, chunks)) || (st = upload(h, &h->d_slplace, places)) ||
         (st = dalloc(h, &h->d_rowexp, (size_t)P.n)) || (st = ensure_colmaps(h)))
         return st;
-    h->sl_ready = true;
+    h->sl_rows = total;
+    return SPX_OK;
+}
+
+// Lists and copies, on the first FP64 factorization that wants them and again
+// after they were given back (drop_slices: another allocation of the handle did
+// not fit, or the factor's precision changed).  They are only made where the
+// selected inverse and a solve's vectors for 16 right-hand sides still fit beside
+// them; elsewhere the factorization stays on the CUDA-core path.
+spx_status ensure_slices(spx_handle h)
+{
+    if (h->sl_ready || h->sl_failed) return SPX_OK;
+    const spx::Plan &P = h->plan;
+    spx_status st = build_slices(h);
+    if (st == SPX_ERR_ALLOC) {   // not even the lists
+        cudaGetLastError();
+        h->err.clear();
+        void *lists[] = {h->d_sl_tiles, h->d_sl_small, h->d_slc, h->d_slplace, h->d_rowexp};
+        for (void *p : lists) dfree(h, p);
+        h->sl_failed = true;
+        return SPX_OK;
+    }
+    if (st != SPX_OK || h->sl_failed) return st;
+    const int ncopy = P.method == SPX_LDLT ? 2 : 1;
+    const size_t bytes = (size_t)h->sl_rows * spx::kSliceCount * 64 * 2;
+    const size_t nexp = (size_t)std::max<int64_t>(h->op_rows, 1) * (h->kpad / 64);
+    const size_t later = (P.method == SPX_LLT && !h->d_Zsel ? (size_t)2 * P.pval[P.npanels] * sizeof(double) : 0) +
+                         (h->ws_nrhs < 16 ? (size_t)8 * 16 * P.n * sizeof(double) : 0);
+    size_t free_bytes = 0, total_bytes = 0;
+    CU(cudaMemGetInfo(&free_bytes, &total_bytes));
+    if (free_bytes < ncopy * (bytes + nexp * sizeof(int32_t)) + later) return SPX_OK;
+    h->sl_ready = true;   // (drop_slices frees what there is)
+    for (int k = 0; k < ncopy; ++k) {
+        char *p = nullptr;
+        if (cudaMalloc((void **)&p, bytes) == cudaSuccess) {
+            h->allocs.push_back(p);
+            h->d_slop[k] = p;
+        }
+        if (p && cudaMalloc((void **)&h->d_slexp[k], nexp * sizeof(int32_t)) == cudaSuccess)
+            h->allocs.push_back(h->d_slexp[k]);
+        if (!h->d_slop[k] || !h->d_slexp[k]) {
+            cudaGetLastError();
+            drop_slices(h);
+            return SPX_OK;
+        }
+        CU(cudaMemset(h->d_slop[k], 0, bytes));
+        CU(cudaMemset(h->d_slexp[k], 0, nexp * sizeof(int32_t)));
+    }
+    const int64_t rows = h->sl_rows * spx::kSliceCount;
+    if (spx::make_operand_map(h->tmap_sla, h->d_slop[0], rows, 64, spx::OP_F16, 128) != 0 ||
+        spx::make_operand_map(h->tmap_slb, h->d_slop[ncopy - 1], rows, 64, spx::OP_F16, 64) != 0) {
+        drop_slices(h);
+        return fail(h, SPX_ERR_CUDA, "cuTensorMapEncodeTiled failed for the FP64 slices");
+    }
+    if (h->fgraph && h->fgraph_prec == SPX_FP64) {   // captured on the other path
+        cudaGraphExecDestroy(h->fgraph);
+        h->fgraph = nullptr;
+        h->fgraph_prec = -1;
+    }
     return SPX_OK;
 }
 
@@ -2163,6 +2219,7 @@ spx_status ensure_factor_storage(spx_handle h, spx_precision precision)
     const size_t esz = fp64 ? sizeof(double) : sizeof(float);
     spx_status st;
     if (h->factor_prec_alloc != (fp64 ? 1 : 0)) {
+        drop_slices(h);
         dfree(h, h->d_L);
         dfree(h, h->d_U);
         dfree(h, h->d_Dinv);
