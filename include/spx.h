@@ -221,7 +221,8 @@ spx_status spx_get_panels(spx_handle h, int64_t *first_col, int32_t *width, int3
  *   needs 4 * n * nrhs elements of the factor's type (8 bytes for an FP64
  *   factor, 4 otherwise) plus 4 * npanels + 3 32-bit words (the sweep
  *   counters and the error word), and returns SPX_ERR_ARG when that exceeds
- *   16 MiB.
+ *   16 MiB.  What is left of the buffer holds further sets of counters, with
+ *   which the columns of an FP64 factor run in up to four groups at once.
  *   The sweeps wait on device-side counters with a bounded wait
  *   (spx_set_wait_limit); the call's own error word, kept in the same
  *   buffer and zeroed at the start of each call, is copied to host memory
