@@ -1582,28 +1582,30 @@ void enqueue_factorization(spx_handle h, bool mixed, Marks &mk, int prec, int pa
             auto launch_set = [&](int64_t a0, int64_t a1, int64_t b0, int64_t b1, int64_t c0, int64_t c1,
                                   Branches &ub, cudaStream_t one) {
                 const int na = (int)(a1 - a0), nb = (int)(b1 - b0), nc = (int)(c1 - c0);
-                auto st = [&](int k) { return one ? one : ub.pick(k); };
+                // a stream is only forked for a launch: one that gets none would hand every
+                // level's nodes on to all later ones of a captured graph
+                auto st = [&](int n, int k) { return one ? one : ub.pick(n > 0 ? k : 0); };
                 if (slices) {
                     // far tiles (`one`) in short CTAs, so that the next levels' launches find free SMs
                     spx::launch_update_sl(h->tmap_sla, h->tmap_slb, h->sl_rows, h->op_rows, h->dp, h->d_sl_tiles + c0, nc,
                                           h->d_colbase, h->d_relbase, h->d_slexp[0], h->d_slexp[ldlt ? 1 : 0], (double *)L, h->d_tcerr,
-                                          one ? kFarTiles : 0, wmax, st(0));
+                                          one ? kFarTiles : 0, wmax, st(nc, 0));
                     mk.mark(SPX_K_UPDATE_TC);
                     spx::launch_update_small(h->dp, h->d_tasks, h->d_sl_small + a0, na, (const double *)L,
-                                             (const double *)Bop, (double *)L, st(nc > 0 ? 1 : 0));
+                                             (const double *)Bop, (double *)L, st(na, nc > 0 ? 1 : 0));
                 } else if (!tc) {
-                    spx::launch_update<T>(h->dp, h->d_tasks, h->d_tiles + a0, na, L, Bop, L, 1, 0, st(0), 0);
+                    spx::launch_update<T>(h->dp, h->d_tasks, h->d_tiles + a0, na, L, Bop, L, 1, 0, st(na, 0), 0);
                     spx::launch_update<T>(h->dp, h->d_tasks, h->d_tiles + b0, nb, L, Bop, L, 1, 0,
-                                          st(na > 0 ? 1 : 0), 1);
+                                          st(nb, na > 0 ? 1 : 0), 1);
                 } else {
                     // the tensor-core tiles on the main stream, the CUDA-core ones beside them
                     spx::launch_update_tc(h->tmap, h->tmap_lo, op_kind, h->dp, h->d_tasks, tcbase + c0, nc,
-                                          (float *)L, 1, h->d_tcerr, st(0));
+                                          (float *)L, 1, h->d_tcerr, st(nc, 0));
                     mk.mark(SPX_K_UPDATE_TC);
                     spx::launch_update<T>(h->dp, h->d_tasks, h->d_tcsmall + a0, na, L, Bop, L, 1, 0,
-                                          st(nc > 0 ? 1 : 0), 0);
+                                          st(na, nc > 0 ? 1 : 0), 0);
                     spx::launch_update<T>(h->dp, h->d_tasks, h->d_tcsmall + b0, nb, L, Bop, L, 1, 0,
-                                          st((nc > 0) + (na > 0)), 1);
+                                          st(nb, (nc > 0) + (na > 0)), 1);
                 }
                 cnt += (na > 0) + (nb > 0) + (nc > 0);
                 h->class_launches[SPX_K_UPDATE] += (na > 0) + (nb > 0);
