@@ -405,13 +405,20 @@ bool panel_slices(const spx::Plan &P, int32_t q)
 // count on one launch for a small FP64 factor still get it.
 constexpr double kSliceMinFlops = 4e8;
 
-// Selected inversion: panels whose product Z_RR Lh has at least this many
-// multiply-adds go to the tensor cores by slices.
-constexpr double kSelinvMinMacs = 65536.0;
-bool selinv_slices(const spx::Plan &P, int32_t q)
+// Selected inversion by slices: panels whose product Z_RR Lh has at least
+// kSelinvMinMacs multiply-adds, in levels where those come to kSelinvLevelMacs:
+// a level's slices take about 33 us whatever their work, the FP64 units of all
+// SMs do 4e6 multiply-adds in half that.  Selected inverse in ms, all on the FP64
+// unit / panels by their own size alone / with the line at 1e6 / 4e6 / 1.6e7: 10^3
+// grid 0.55 / 0.65 / 0.44 / 0.44 / 0.44, 12^3 0.82 / 0.87 / 0.66 / 0.65 / 0.65,
+// 20^3 at most 16 wide 2.68 / 2.75 / 2.56 / 2.33 / 2.57, 22^3 4.96 / 2.46 / 2.43 /
+// 2.42 / 3.37, 48^3 257 / 47.3 / 47.3 / 47.2 / 47.3.  (kSelinvMinMacs at 262,144:
+// 22^3 2.63, 48^3 48.1.)
+constexpr double kSelinvMinMacs = 65536.0, kSelinvLevelMacs = 4e6;
+double selinv_macs(const spx::Plan &P, int32_t q)
 {
     const double m = (double)P.ph[q] - P.pw[q];
-    return m * m * P.pw[q] >= kSelinvMinMacs;
+    return m * m * P.pw[q];
 }
 
 // Algorithmic work of every panel and update task, as the kernel classes
@@ -3093,9 +3100,14 @@ spx_status spx_selected_inverse(spx_handle h, void *cuda_stream)
         h->sv64_ptr.assign(P.nlevels + 1, 0);
         h->sv_blocks.assign(P.nlevels, 1);
         for (int32_t l = 0; l < P.nlevels; ++l) {
+            double macs = 0.0;
+            for (int32_t q = P.level_ptr[l]; q < P.level_ptr[l + 1]; ++q) {
+                const double mq = selinv_macs(P, P.level_panels[q]);
+                macs += mq >= kSelinvMinMacs ? mq : 0.0;
+            }
             for (int32_t q = P.level_ptr[l]; q < P.level_ptr[l + 1]; ++q) {
                 const int32_t k = P.level_panels[q], w = P.pw[k], hk = P.ph[k];
-                const bool sl = selinv_slices(P, k);
+                const bool sl = macs >= kSelinvLevelMacs && selinv_macs(P, k) >= kSelinvMinMacs;
                 if (sl) h->sv_blocks[l] = std::max(h->sv_blocks[l], (hk - w + 63) / 64);
                 for (int32_t r0 = w; r0 < hk; r0 += sl ? 128 : 64) (sl ? c128 : c64).push_back(RowChunk{k, r0});
             }

@@ -547,7 +547,8 @@ __device__ __forceinline__ void ldl_diag_block(const DevPlan &p, int pid, T *__r
         }
         dvf[tid] = from_f64<T>(dv[tid]);
         rvf[tid] = from_f64<T>(rsv[tid]);
-        if constexpr (kExps && ldlt) rmax[tid] = lead_exp(__double2hiint(dv[tid])) >> 1;
+        if constexpr (kExps && ldlt)
+            if (rowexp) rmax[tid] = lead_exp(__double2hiint(dv[tid])) >> 1;
     }
     __syncthreads();
     for (int idx = tid; idx < W * W; idx += NT) {
