@@ -459,8 +459,9 @@ typedef struct {
     int64_t factor_elems;   /* stored elements of L plus U^T over all systems */
     double flops;           /* exact-pattern LU flops over all systems: sum 2(c_j-1)^2+(c_j-1) */
     int32_t precision;      /* spx_precision of the last run */
-    int32_t ctas_per_sm;    /* launch configuration in use ... */
-    int32_t leaf_width;     /* panels at most this wide go one per warp (0: none) */
+    int32_t ctas_per_sm;    /* launch configuration in use (unset: as many CTAs as hold the batch at once,
+                               two to the most that fit) ... */
+    int32_t leaf_width;     /* panels at most this wide with at most 32 rows below go one per warp (0: none) */
     int32_t rows_per_thread;/* rows of the update tile per thread (1, 2 or 4) */
     double tuned_ms;        /* run time of the configuration spx_batch_tune chose (0: not tuned) */
     double analyze_ms;      /* host time of spx_batch_analyze */

@@ -306,7 +306,13 @@ RunCfg current_cfg(spx_batch b, int elem)
 {
     RunCfg c{b->ctas_per_sm, b->leaf_width, b->rows_per_thread};
     const int mx = spx::batch_max_ctas_per_sm(elem, (int)b->n_max, c.rt);
-    if (c.ctas <= 0 || c.ctas > mx) c.ctas = mx;
+    // as many CTAs an SM as hold all systems at once, two at least (the kernel for
+    // fewer CTAs has more registers a thread): FP32, two / three / four, ms: 300
+    // systems of 8 to 16 a side 0.20 / 0.27 / 0.32, 400 of 4 to 5 0.11 / 0.08 / 0.09, 456
+    // of 80 13.4 / 9.0 / 10.6, 800 of 8 to 16 0.39 / 0.35 / 0.34, 4096 of 12 to 80
+    // 33.7 / 29.3 / 27.7
+    if (c.ctas <= 0) c.ctas = std::max(2, (int)std::min<int64_t>(mx, ((int64_t)b->nsys + b->num_sms - 1) / b->num_sms));
+    c.ctas = std::min(c.ctas, mx);
     return c;
 }
 
@@ -344,7 +350,7 @@ spx_status launch(spx_batch b, const double *vals, const double *B, double *X, i
     std::memcpy(key.data() + sizeof(a), &cfg, sizeof(cfg));
     std::memcpy(key.data() + sizeof(a) + sizeof(cfg), &elem, sizeof(elem));
     // sets the kernel's shared-memory attribute too (outside the capture)
-    if (spx::batch_max_ctas_per_sm(elem, (int)b->n_max, cfg.rt) < cfg.ctas)
+    if (spx::batch_max_ctas_per_sm(elem, (int)b->n_max, cfg.rt, cfg.ctas) < cfg.ctas)
         return bfail(b, SPX_ERR_ARG, "more CTAs per SM than fit");
     if (!b->exec || key != b->exec_key) {
         if (b->exec) {
@@ -354,7 +360,7 @@ spx_status launch(spx_batch b, const double *vals, const double *B, double *X, i
         cudaGraph_t g = nullptr;
         BCU(cudaStreamBeginCapture(b->hs, cudaStreamCaptureModeThreadLocal));
         cudaMemsetAsync(b->d_queue, 0, 4 * sizeof(unsigned), b->hs);
-        spx::launch_batch(a, elem, cfg.rt, b->num_sms * cfg.ctas, (int)b->n_max, b->hs);
+        spx::launch_batch(a, elem, cfg.rt, cfg.ctas, b->num_sms * cfg.ctas, (int)b->n_max, b->hs);
         cudaError_t le = cudaGetLastError();
         cudaError_t e = cudaStreamEndCapture(b->hs, &g);
         if (le != cudaSuccess) {

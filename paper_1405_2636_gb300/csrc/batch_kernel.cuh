@@ -63,8 +63,10 @@ constexpr int kBatchMaxWidth = 64;    // widest panel of a batched system
 constexpr int kBatchLeafMax = 16;     // widest panel one warp may take
 
 size_t batch_smem_bytes(int elem_bytes, int n_max);
-int batch_max_ctas_per_sm(int elem_bytes, int n_max, int rows_per_thread);
-void launch_batch(const BatchArgs &a, int elem_bytes, int rows_per_thread, int grid, int n_max,
+// CTAs that fit an SM of the kernel compiled for `ctas` of them.
+constexpr int kBatchMaxCtas = 4;
+int batch_max_ctas_per_sm(int elem_bytes, int n_max, int rows_per_thread, int ctas = kBatchMaxCtas);
+void launch_batch(const BatchArgs &a, int elem_bytes, int rows_per_thread, int ctas, int grid, int n_max,
                   cudaStream_t s);
 
 }  // namespace spx

@@ -20,8 +20,11 @@
 // What bounds it: chains.  A system's panels of a level rarely fill the CTA's
 // warps, each is a string of loads, pivots and barriers, and of 19 resident
 // warps' cycles a scheduler spends 6.5 at barriers and 5.9 on loads per issued
-// instruction, so FP32 runs four CTAs an SM (64 registers; three: 29.1 ms, four:
-// 27.7).  4096 systems (grids of 12 to 80 a side, FP32 with refinement) 37.5 ->
+// instruction, so FP32 batches of many systems run four CTAs an SM (64 registers;
+// three: 29.3 ms, four: 27.8), smaller ones as many as hold them all at once, with
+// the registers that this leaves (24 systems of 5 to 40 a side, FP32: 1.62 -> 1.23
+// ms; registers spilled, bytes of stores: 16 to 20 at two CTAs an SM, 56 to 68 at
+// three, 164 to 232 at four, 128 to 136 in FP64).  4096 systems (grids of 12 to 80 a side, FP32 with refinement) 37.5 ->
 // 27.7 ms, 24 systems (5 to 40 a side, FP64) 3.29 -> 2.66 ms, by narrow panels
 // and sweeps with their rows in registers and blocked pivots of the wide ones;
 // in FP64 the FP64 unit's rate for narrow panels bounds the leaves.
@@ -273,6 +276,7 @@ __device__ __forceinline__ void panel_warp8(const BClass &c, int p, T *Ls, T *Us
         if (lane < W) lu[lane * LDR + k] = a[k];
     }
     __syncwarp();
+    if (R == 0) return;                             // a root: no rows, no updates
     T x[W], y[W];
     constexpr bool kSplit = sizeof(T) == 8;
     if (kSplit && R <= 16) {                    // lanes 0 .. R-1: rows of L, R .. 2R-1: of U^T
@@ -520,7 +524,21 @@ __device__ __forceinline__ void bwd_panel_warp(const BClass &c, int p, const T *
     const T *Lp = Ls + c.pval[p];
     const T *Up = Us + c.pval[p];
     const int32_t *rows = c.rows + c.prow[p];
-    if (h > w) {
+    if (sizeof(T) == 8 && h > w && h - w <= 8) {
+        // few rows: a column a lane (in FP64 eight sums' shuffles cost more than the
+        // rows; in FP32 the branch costs as much as it saves)
+        for (int k = lane; k < w; k += 32) {
+            T s0 = wv[fc + k], s1 = (T)0;
+            int i = w;
+            for (; i + 1 < h; i += 2) {
+                s0 -= Up[i + (int64_t)k * h] * wv[rows[i]];
+                s1 -= Up[i + 1 + (int64_t)k * h] * wv[rows[i + 1]];
+            }
+            if (i < h) s0 -= Up[i + (int64_t)k * h] * wv[rows[i]];
+            wv[fc + k] = s0 + s1;
+        }
+        __syncwarp();
+    } else if (h > w) {
         for (int k0 = 0; k0 < w; k0 += 8) {
             const int kc = min(8, w - k0);
             T s[8];
@@ -716,8 +734,8 @@ __device__ __forceinline__ void process(const BatchArgs &a, int sid, T *region, 
     }
 }
 
-template <typename T, int RT>
-__global__ void __launch_bounds__(kBatchThreads, sizeof(T) == 8 ? 2 : 4) batch_lu_kernel(BatchArgs a)
+template <typename T, int RT, int CTAS>
+__global__ void __launch_bounds__(kBatchThreads, CTAS) batch_lu_kernel(BatchArgs a)
 {
     extern __shared__ double smd[];
     double *red = smd;
@@ -733,12 +751,6 @@ __global__ void __launch_bounds__(kBatchThreads, sizeof(T) == 8 ? 2 : 4) batch_l
     }
 }
 
-template <typename T, int RT>
-void set_smem_attr(size_t bytes)
-{
-    cudaFuncSetAttribute(batch_lu_kernel<T, RT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 }  // namespace
 
 size_t batch_smem_bytes(int elem_bytes, int n_max)
@@ -749,51 +761,53 @@ size_t batch_smem_bytes(int elem_bytes, int n_max)
     return sizeof(double) * kRedDoubles + (size_t)elem_bytes * (size_t)elems;
 }
 
-template <typename T, int RT>
-static int max_ctas(size_t smem)
+// fn(kernel) with the kernel for `ctas` CTAs an SM: its registers are what that
+// many leave (FP32: 128, 80 or 64 a thread for up to two, three, four; FP64, whose
+// shared memory lets two on an SM, 128).
+template <typename T, int RT, typename F>
+static auto with_ctas(int ctas, F fn)
 {
-    set_smem_attr<T, RT>(smem);
-    int blocks = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, batch_lu_kernel<T, RT>, kBatchThreads, smem) !=
-        cudaSuccess)
-        return 0;
-    return blocks;
+    if constexpr (sizeof(T) == 4) {
+        if (ctas > 3) return fn(batch_lu_kernel<T, RT, 4>);
+        if (ctas == 3) return fn(batch_lu_kernel<T, RT, 3>);
+    }
+    return fn(batch_lu_kernel<T, RT, 2>);
 }
 
-int batch_max_ctas_per_sm(int elem_bytes, int n_max, int rows_per_thread)
+template <typename F>
+static auto with_kernel(int elem_bytes, int rows_per_thread, int ctas, F fn)
+{
+    if (elem_bytes == 8) {
+        if (rows_per_thread == 1) return with_ctas<double, 1>(ctas, fn);
+        if (rows_per_thread == 2) return with_ctas<double, 2>(ctas, fn);
+        return with_ctas<double, 4>(ctas, fn);
+    }
+    if (rows_per_thread == 1) return with_ctas<float, 1>(ctas, fn);
+    if (rows_per_thread == 2) return with_ctas<float, 2>(ctas, fn);
+    return with_ctas<float, 4>(ctas, fn);
+}
+
+int batch_max_ctas_per_sm(int elem_bytes, int n_max, int rows_per_thread, int ctas)
 {
     const size_t smem = batch_smem_bytes(elem_bytes, n_max);
-    if (elem_bytes == 8) {
-        if (rows_per_thread == 1) return max_ctas<double, 1>(smem);
-        if (rows_per_thread == 2) return max_ctas<double, 2>(smem);
-        return max_ctas<double, 4>(smem);
-    }
-    if (rows_per_thread == 1) return max_ctas<float, 1>(smem);
-    if (rows_per_thread == 2) return max_ctas<float, 2>(smem);
-    return max_ctas<float, 4>(smem);
+    return with_kernel(elem_bytes, rows_per_thread, ctas, [&](auto *kernel) {
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        int blocks = 0;
+        return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks, kernel, kBatchThreads, smem) == cudaSuccess
+                   ? blocks
+                   : 0;
+    });
 }
 
 // The shared-memory attribute is set by batch_max_ctas_per_sm, which the
 // caller runs first (outside any stream capture).
-template <typename T, int RT>
-static void launch_t(const BatchArgs &a, int grid, size_t smem, cudaStream_t s)
-{
-    batch_lu_kernel<T, RT><<<grid, kBatchThreads, smem, s>>>(a);
-}
-
-void launch_batch(const BatchArgs &a, int elem_bytes, int rows_per_thread, int grid, int n_max,
+void launch_batch(const BatchArgs &a, int elem_bytes, int rows_per_thread, int ctas, int grid, int n_max,
                   cudaStream_t s)
 {
-    const size_t smem = batch_smem_bytes(elem_bytes, n_max);
-    if (elem_bytes == 8) {
-        if (rows_per_thread == 1) launch_t<double, 1>(a, grid, smem, s);
-        else if (rows_per_thread == 2) launch_t<double, 2>(a, grid, smem, s);
-        else launch_t<double, 4>(a, grid, smem, s);
-    } else {
-        if (rows_per_thread == 1) launch_t<float, 1>(a, grid, smem, s);
-        else if (rows_per_thread == 2) launch_t<float, 2>(a, grid, smem, s);
-        else launch_t<float, 4>(a, grid, smem, s);
-    }
+    with_kernel(elem_bytes, rows_per_thread, ctas, [&](auto *kernel) {
+        kernel<<<grid, kBatchThreads, batch_smem_bytes(elem_bytes, n_max), s>>>(a);
+        return 0;
+    });
 }
 
 }  // namespace spx
