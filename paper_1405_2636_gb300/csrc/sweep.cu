@@ -506,13 +506,14 @@ __device__ __forceinline__ void chunk_dot4(const T *Lc, const T *Xs, int k, int 
 }  // namespace
 
 // Shared memory: two 64 x 64 matrices, two vectors of the widest panel (at
-// least 64 rows) x NC, the partial sums.  Four CTAs an SM in FP32, three in
-// FP64 (one fewer measured slower in FP64, one more in FP32, where registers spill).
-template <typename T>
-constexpr int kCtas = sizeof(T) == 8 ? 3 : 4;
+// least 64 rows) x NC, the partial sums.  Four CTAs an SM in FP32 (one more
+// measured slower, where registers spill), three for one FP64 column (two
+// measured slower), two for eight, as many as 82 KB of shared memory let on.
+template <typename T, int NC>
+constexpr int kCtas = sizeof(T) == 4 ? 4 : NC == 1 ? 3 : 2;
 
 template <typename T, int NC>
-__global__ void __launch_bounds__(kQThreads, kCtas<T>)
+__global__ void __launch_bounds__(kQThreads, kCtas<T, NC>)
     fwd_queue_kernel(DevPlan p, SweepQueue q, const T *__restrict__ Dinv, int unit,
                      const T *__restrict__ L, T *Y, T *Z, int nrhs)
 {
@@ -629,7 +630,7 @@ __global__ void __launch_bounds__(kQThreads, kCtas<T>)
 // lu: 0 Cholesky (M = Linv^T), 1 LU (M = U^{-1}), 2 LDL^T
 // (X_p = l^{-T} (D^{-1} Z_p - Tacc_p), 1/d on the diagonal of Dinv).
 template <typename T, int NC>
-__global__ void __launch_bounds__(kQThreads, kCtas<T>)
+__global__ void __launch_bounds__(kQThreads, kCtas<T, NC>)
     bwd_queue_kernel(DevPlan p, SweepQueue q, const T *__restrict__ Dinv, int lu,
                      const T *__restrict__ Lop, const T *__restrict__ Z, T *Tacc, T *X, int nrhs)
 {
