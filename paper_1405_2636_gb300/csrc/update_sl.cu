@@ -69,9 +69,10 @@ __global__ void __launch_bounds__(kSlThreads, 1)
     extern __shared__ unsigned char smraw[];
     unsigned char *base =
         reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smraw) + 1023) & ~(uintptr_t)1023);
-    __shared__ __align__(8) uint64_t full[kSlots], empty[kSlots], acc_full[kAcc], acc_empty[kAcc];
+    __shared__ __align__(8) uint64_t full[kSlots], empty[kSlots], acc_full[kAcc], acc_empty[kAcc], drained;
     __shared__ uint32_t s_tmem;
     __shared__ volatile int s_fail;
+    __shared__ int s_lt, s_slice;                      // the first load that was not issued
     __shared__ int64_t s_coff[kEpi][kEC], s_rel[kEpi][kEC];
     __shared__ int32_t s_eb[kEpi][kEC];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -81,6 +82,7 @@ __global__ void __launch_bounds__(kSlThreads, 1)
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], 1);
         }
+        mbar_init(&drained, 1);
         for (int b = 0; b < kAcc; ++b) {
             mbar_init(&acc_full[b], 1);
             mbar_init(&acc_empty[b], kEpi);
@@ -100,11 +102,11 @@ __global__ void __launch_bounds__(kSlThreads, 1)
 
     if (warp == kEpi) {
         if (elect_one()) {
-            int lt = 0;
+            int lt = 0, next = 0;
             bool ok = true;
             for (int t = blockIdx.x; t < count && ok; t += gridDim.x) {
                 const SlTile tl = tiles[t];
-                for (int kx = 0; kx == 0 || (kWide && kx < tl.k && ok); kx += kK, ++lt) {
+                for (int kx = 0; ok && (kx == 0 || (kWide && kx < tl.k)); kx += kK) {
 #pragma unroll
                     for (int i = 0; i < kSlices; ++i) {
                         const int s = i < 2 ? i : 8 - i;   // 0, 1, 6, 5, 4, 3, 2: the order they fall free in
@@ -112,6 +114,7 @@ __global__ void __launch_bounds__(kSlThreads, 1)
                         const int u = s < 2 ? lt >> 1 : lt;   // earlier uses of this buffer
                         if (u >= 1 && !mbar_wait_or(&empty[slot], (uint32_t)(u - 1) & 1u, &s_fail)) {
                             ok = false;
+                            next = i;
                             break;
                         }
                         unsigned char *dst = base + slot * kSlotBytes;
@@ -121,9 +124,12 @@ __global__ void __launch_bounds__(kSlThreads, 1)
                         tma_load_2d(dst, &mapa, &full[slot], 0, (int)(s * oprows) + ra);
                         tma_load_2d(dst + kABytes, &mapb, &full[slot], 0, (int)(s * oprows) + rb);
                     }
+                    lt += ok;
                 }
             }
             if (!ok) s_fail = 1;
+            s_lt = lt;
+            s_slice = next;
         }
     } else if (warp == kEpi + 1) {
         if (elect_one()) {
@@ -192,6 +198,7 @@ __global__ void __launch_bounds__(kSlThreads, 1)
                 }
             }
             if (!ok) s_fail = 1;
+            mma_commit(&drained);
         }
     } else {
         uint32_t ng = 0;
@@ -279,6 +286,18 @@ __global__ void __launch_bounds__(kSlThreads, 1)
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    if (s_fail) {
+        // one of the roles gave up: no MMA and no load may be left in flight when the
+        // accumulators are freed and the CTA's shared memory is another's
+        mbar_wait(&drained, 0);
+        for (int i = 0; i < kSlices; ++i) {
+            const int s = i < 2 ? i : 8 - i, n = s_lt + (i < s_slice ? 1 : 0);   // (see the loads' order)
+            const int even = s < 2 ? (n + 1) / 2 : n, odd = s < 2 ? n / 2 : 0;
+            if (even > 0) mbar_wait(&full[s], (uint32_t)(even - 1) & 1u);
+            if (odd > 0) mbar_wait(&full[7 + s], (uint32_t)(odd - 1) & 1u);
+        }
+        __syncthreads();
+    }
     if (threadIdx.x == 0 && s_fail) atomicExch(err, 1);
     if (warp == 0)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kSlCols));
@@ -545,6 +564,7 @@ __global__ void __launch_bounds__(kTrThreads, 1)
             }
         }
     }
+    if (s_fail) mbar_wait(&done[0], phase ^ 1u);   // no MMA in flight when the accumulators are freed
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (tid == 0 && s_fail) atomicExch(err, 1);
@@ -742,6 +762,7 @@ __global__ void __launch_bounds__(kTrThreads, 1)
             else atomicAdd(dst + (int64_t)c * h, acc[q]);
         }
     }
+    if (s_fail) mbar_wait(&done[0], phase ^ 1u);   // no MMA in flight when the accumulators are freed
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (tid == 0 && s_fail) atomicExch(err, 1);
@@ -869,6 +890,7 @@ __global__ void __launch_bounds__(kTrThreads, 1)
             if (c < a) atomicAdd(&Z[pv + c + (int64_t)a * h], acc[q]);
         }
     }
+    if (s_fail) mbar_wait(&done[0], phase ^ 1u);   // no MMA in flight when the accumulators are freed
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (tid == 0 && s_fail) atomicExch(err, 1);
