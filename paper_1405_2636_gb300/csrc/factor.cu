@@ -399,8 +399,10 @@ size_t potrf_wide_smem(int wmax)
 // stays).  A block whose inverse fixed point cannot hold has it formed from the
 // stored factor (in all 68 us for FP64, 49 for FP32); one whose factor it cannot
 // hold goes the FP64 way, after the time lost here.
-template <typename T>
-__global__ void __launch_bounds__(256) potrf_mid_kernel(DevPlan p, const int32_t *__restrict__ panels,
+// One CTA an SM where the panels are no more than SMs (FP64: 172 registers; in
+// 128 the chain spills, 64^3 diagonal blocks 17.4 and 17.9 ms), else two.
+template <typename T, int CTAS>
+__global__ void __launch_bounds__(256, CTAS) potrf_mid_kernel(DevPlan p, const int32_t *__restrict__ panels,
                                                         T *__restrict__ L, T *__restrict__ Dinv,
                                                         const double *replace_tau_p, int64_t *err_col,
                                                         unsigned long long *nrepl, int32_t *rowexp)
@@ -491,16 +493,25 @@ void launch_potrf(const DevPlan &p, const int32_t *panels, int count, int wmax, 
     if (wmax <= 16) return launch_ldl<T, 16>(p, panels, count, L, Dinv, replace_tau, err_col, nrepl, rowexp, s);
     if (wmax <= 32) return launch_ldl<T, 32>(p, panels, count, L, Dinv, replace_tau, err_col, nrepl, rowexp, s);
     static bool once = false;
+    static int nsm = 0;
     if (!once) {
-        cudaFuncSetAttribute(potrf_mid_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaFuncSetAttribute(potrf_mid_kernel<T, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)std::max(fx::smem_bytes(64), ldl_smem_bytes<T, 64>()));
+        cudaFuncSetAttribute(potrf_mid_kernel<T, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)std::max(fx::smem_bytes(64), ldl_smem_bytes<T, 64>()));
+        int dev = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
         cudaFuncSetAttribute(potrf_wide_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)std::max(potrf_wide_smem(kMaxWidth), potrf_wide_smem(fx::kMaxW)));
         once = true;
     }
     if (wmax <= 64) {
         const size_t smem = std::max(fx::smem_bytes(wmax), ldl_smem_bytes<T, 64>());
-        potrf_mid_kernel<T><<<count, 256, smem, s>>>(p, panels, L, Dinv, replace_tau, err_col, nrepl, rowexp);
+        if (count <= nsm)
+            potrf_mid_kernel<T, 1><<<count, 256, smem, s>>>(p, panels, L, Dinv, replace_tau, err_col, nrepl, rowexp);
+        else
+            potrf_mid_kernel<T, 2><<<count, 256, smem, s>>>(p, panels, L, Dinv, replace_tau, err_col, nrepl, rowexp);
         return;
     }
     potrf_wide_kernel<T><<<count, 256, potrf_wide_smem(wmax), s>>>(p, panels, L, Dinv, replace_tau, err_col, nrepl,
