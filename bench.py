@@ -612,6 +612,62 @@ def run_update_study(torch, spx, inputs, peaks: dict) -> dict:
 
 
 # ---------------------------------------------------------------------------
+# the printed line
+# ---------------------------------------------------------------------------
+LINE_BYTES = 4096      # a line that fits the pipes and records it passes through
+DETAILS = "bench_details.json"
+
+
+def _short(v):
+    """Floats to five digits, containers through."""
+    if isinstance(v, float):
+        return float(f"{v:.5g}")
+    if isinstance(v, dict):
+        return {k: _short(x) for k, x in v.items()}
+    return [_short(x) for x in v] if isinstance(v, (list, tuple)) else v
+
+
+def _workload_ms(full: dict) -> dict:
+    """The further workloads' times."""
+    out = {}
+    if "batched_lu" in full:
+        out["batched_lu"] = {k: full["batched_lu"][k]["ms"] for k in ("fp32_refined", "fp64")}
+    if "differentiation" in full:
+        out["differentiation"] = {k: full["differentiation"][k + "_ms"]
+                                  for k in ("forward", "backward", "selected_inverse")}
+    for k in ("ldlt", "elasticity"):
+        if k in full:
+            out[k] = {m: r["ms_per_step"] for m, r in full[k]["modes"].items()}
+    return out
+
+
+def headline(full: dict) -> dict:
+    """The run's one printed line, at most LINE_BYTES long: the contract's keys in full,
+    of the modes and further workloads their times and errors.  `full` (every step's
+    time, kernel classes of all modes, the update study, rooflines) goes to the
+    details file."""
+    keep = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+            "vs_baseline", "dtype", "data", "config", "fp64_ms_per_step", "speedup_mixed_over_fp64", "e2e",
+            "gpu_launches", "clocks", "details")
+    line = {k: full[k] for k in keep if k in full}
+    per_mode = ("ms_per_step", "factor_ms", "solve_ms", "time_to_solve_gflops", "host_backward_error", "refine_iters",
+                "launches_per_step", "e2e_ms")
+    # in this order, as far as the line's length allows
+    more = {
+        "modes": {m: _short({k: r[k] for k in per_mode if k in r}) for m, r in full.get("modes", {}).items()},
+        "roofline": _short(full.get("roofline")),
+        "kernel_ms": {m: {c: round(st["ms"], 3) for c, st in ks.items() if st["ms"] > 0}
+                      for m, ks in full.get("kernel_stats", {}).items()},
+        "workload_ms": _short(_workload_ms(full)),
+        "cpu_baseline": _short(full.get("cpu_baseline")),
+    }
+    for k, v in more.items():
+        if v and len(json.dumps({**line, k: v})) < LINE_BYTES:
+            line[k] = v
+    return line
+
+
+# ---------------------------------------------------------------------------
 # the GPU arm
 # ---------------------------------------------------------------------------
 def main():
@@ -816,7 +872,9 @@ def main():
         "clocks": clocks,
     }
     line.update(extra)
-    print(json.dumps(line), flush=True)
+    with open(os.path.join(ROOT, DETAILS), "w") as f:
+        json.dump(line, f, indent=1)
+    print(json.dumps(headline(dict(line, details=DETAILS))), flush=True)
     if world > 1:
         torch.distributed.destroy_process_group()
 
