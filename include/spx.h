@@ -82,9 +82,10 @@ typedef struct {
     int32_t queue_panels;   /* levels of the panel tree run as one persistent launch over a device-side
                                task queue (Cholesky, LDL^T; panels at most 64 wide): > 0 = the top levels
                                holding at most this many panels; < 0 = none (every level launched on its
-                               own); 0 = default (the policy that measured fastest): the whole tree for an
-                               FP64 factor whose updates come to less than 4e8 flops, none for larger
-                               ones and for the single-precision factors */
+                               own); 0 = default: the whole tree for an FP64 factor whose updates come to
+                               less than 4e8 flops, so that it is one launch whatever the tree's depth
+                               (with < 0 such a factor of 8^3 to 22^3 unknowns took half to two thirds of
+                               the time), none for larger ones and for the single-precision factors */
     double pivot_tau;       /* LU static-pivot threshold; < 0 = sqrt(2^-52) * ||A||_inf at factorize */
     int32_t deterministic;  /* 1: bit-reproducible factors -- the updates of a level run in rounds, one
                                task per target panel per round in task order, so that every target

@@ -487,10 +487,11 @@ int queue_start_level(const spx::Plan &P, int qmax)
 
 // The queue region a factorization in `prec` uses.  qopt > 0: the top
 // levels with at most qopt panels; qopt < 0: none; qopt = 0 (default): the
-// whole tree (as far as panels are at most 64 wide) for an FP64 factor,
-// where the queue measured faster than the level walk (its update tiles are
-// long FP64 products), and none for the single-precision factors, whose
-// short tensor-core and FP32 tiles ran faster as per-level launches.
+// whole tree (as far as panels are at most 64 wide) for an FP64 factor that
+// does not take the slices (kSliceMinFlops; against the level walk on the
+// CUDA cores the queue measured faster there), and none for the
+// single-precision factors, whose short tensor-core and FP32 tiles ran faster
+// as per-level launches.
 int queue_policy_level(const spx::Plan &P, int qopt, int prec)
 {
     if (qopt < 0 || (qopt == 0 && prec != SPX_FP64)) return P.nlevels;
@@ -1439,7 +1440,11 @@ void enqueue_part_queue(spx_handle h, T *L, T *Dinv, T *W, void *opc, void *opc_
                                 h->tmap, h->tmap_lo, opc, opc_lo, h->kpad, op_kind, s);
 }
 
-constexpr int kFarTiles = 4;        // tiles a CTA of the far FP64 slice updates
+// Tiles a CTA of the far FP64 slice updates: short CTAs, so that the next levels'
+// launches find free SMs.  Factorization in ms at 2 / 4 / 8 / 16 / one CTA an SM:
+// 64^3 66.0 / 61.3 / 58.3 / 56.5 / 59.6, 48^3 20.4 / 19.2 / 19.3 / 19.4 / 19.4, LDL^T
+// 32^3 x 2 17.6 / 16.7 / 17.3 / 17.3 / 17.4, default options 8.64 at all.
+constexpr int kFarTiles = 4;
 constexpr int kWhole = INT32_MIN;   // enqueue_factorization: the whole factorization
 
 template <typename T>

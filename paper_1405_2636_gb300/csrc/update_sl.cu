@@ -55,8 +55,10 @@ __device__ __forceinline__ int slot_of(int s, int lt) { return (s < 2 && (lt & 1
 // What bounds it: a full tile's 28 pairs take 28 x 4 MMAs of 32 cycles
 // (3,584 cycles), its drain about 50 integer instructions an element
 // (3,200 cycles a warp scheduler), beside each other.  64^3 grid, 64-wide
-// panels: all updates 36.8 ms (4.2e11 flops, 11 TFLOP/s; the FP64 unit's tiles
-// in the task queue took most of that factorization's 537 ms, now 62).
+// panels: all updates 36.5 ms (4.2e11 flops, 11 TFLOP/s; the FP64 unit's tiles
+// in the task queue took most of that factorization's 537 ms, now 61.5).  Registers
+// (96 a thread for 18 warps) spill: 36 bytes, for panels wider than 64 with their
+// carried sums 196.
 // ---------------------------------------------------------------------------
 template <bool kWide>
 __global__ void __launch_bounds__(kSlThreads, 1)
@@ -332,7 +334,7 @@ __global__ void __launch_bounds__(kSlThreads, 1)
 // instructions an element) and, at the top of the tree, where a level has a
 // few dozen CTAs, by latency and instruction fetches: 8 elements a thread
 // and one loop over both operands keep the code short (a 64-row CTA 17 us; 128
-// rows with straight-line code 35).  64^3 grid: 12.1 ms for 245 levels.
+// rows with straight-line code 35).  64^3 grid: 11.9 ms for 245 levels.
 // ---------------------------------------------------------------------------
 constexpr int kTrRows = 64;
 constexpr int kTrThreads = 512;
@@ -585,7 +587,8 @@ __global__ void __launch_bounds__(kTrThreads, 1)
 // Bound by the integer work (about 68 instructions an entry of Z, 72 a result
 // and block); the FP64 unit would take 300,000 cycles for a block that this
 // does in about 15,000.  48^3 grid: the whole selected inverse 257 -> 46 ms, of
-// which these products 39 (150 levels of about 33 us fixed cost each).
+// which these products 39 (150 levels of about 33 us fixed cost each).  Registers
+// (128 a thread) spill 240 bytes.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kTrThreads, 1)
     selinv_sl_kernel(DevPlan p, const RowChunk *__restrict__ chunks, const int64_t *__restrict__ colbase,
