@@ -397,10 +397,12 @@ size_t potrf_wide_smem(int wmax)
 // one a lane (64 wide: 67 -> 48 us for an FP64 factor, 51 -> 47 for FP32; up to
 // 32 columns both take the same time, 23 to 26 us, and the smaller kernel
 // stays).  A block whose inverse fixed point cannot hold has it formed from the
-// stored factor (in all 68 us for FP64, 49 for FP32); one whose factor it cannot
+// stored factor (in all 69 us for FP64, 50 for FP32); one whose factor it cannot
 // hold goes the FP64 way, after the time lost here.
-// One CTA an SM where the panels are no more than SMs (FP64: 172 registers; in
-// 128 the chain spills, 64^3 diagonal blocks 17.4 and 17.9 ms), else two.
+// FP64 factors: one CTA an SM where the panels are no more than SMs (174 registers;
+// in 128 the chain spills, 64^3 diagonal blocks 17.4 and 17.75 ms), else two, and
+// always two for FP32 factors, whose other launches of the level want the
+// registers (64^3 TF32 factorization 28.24 ms with one, 27.93 with two).
 template <typename T, int CTAS>
 __global__ void __launch_bounds__(256, CTAS) potrf_mid_kernel(DevPlan p, const int32_t *__restrict__ panels,
                                                         T *__restrict__ L, T *__restrict__ Dinv,
@@ -508,7 +510,7 @@ void launch_potrf(const DevPlan &p, const int32_t *panels, int count, int wmax, 
     }
     if (wmax <= 64) {
         const size_t smem = std::max(fx::smem_bytes(wmax), ldl_smem_bytes<T, 64>());
-        if (count <= nsm)
+        if (sizeof(T) == 8 && count <= nsm)
             potrf_mid_kernel<T, 1><<<count, 256, smem, s>>>(p, panels, L, Dinv, replace_tau, err_col, nrepl, rowexp);
         else
             potrf_mid_kernel<T, 2><<<count, 256, smem, s>>>(p, panels, L, Dinv, replace_tau, err_col, nrepl, rowexp);

@@ -30,7 +30,7 @@
 //
 // A 64-wide FP64 block takes 49 us (FP64 unit: 69), FP32 47 (53; both start as
 // the same integers); 128 wide 0.18 ms (0.58 on the FP64 unit).  With the inverse
-// in floating point 68 us and 49, 0.40 ms and 0.25 (the whole block a second time
+// in floating point 69 us and 50, 0.40 ms and 0.25 (the whole block a second time
 // on the FP64 unit: 111 and 92, 0.74 and 0.60).  What bounds it: per 8 columns about 6,600 cycles of one warp's
 // dependent instructions, a third of them the reciprocal square roots.
 #pragma once
@@ -372,7 +372,7 @@ __device__ __forceinline__ void bar_some(int threads)
 // finds stays its own until a barrier joins all threads' words, so that all leave
 // at the same barrier: a shared flag, read behind one barrier, could already hold
 // what a faster warp finds before the next.  (leave_out is such a flag and decides
-// nothing: it saves work on an inverse that is not used, between barriers that
+// nothing: it saves rows of an inverse that is not used, between barriers that
 // every thread passes.)
 // rowexp (or null): the exponents of about sqrt(a_ii).
 enum Outcome { kRefused, kNoInverse, kDone };
@@ -460,7 +460,7 @@ __device__ Outcome diag_block(T *__restrict__ D, T *__restrict__ Mi, int w, int 
         if (nx == nw) rank8(a, LD, W8, lb, kDB * (b + 2), W8, 32 * wi + lane, 32 * nw);
         else if (wi >= nx) rank8(a, LD, W8, lb, kDB * (b + 2), W8, 32 * (wi - nx) + lane, 32 * (nw - nx));
         bar_some(32 * nw);
-        if (!*leave_out) inverse_sums(a, LD, W8, b, lb, limx, 32 * wi + lane, 32 * nw);
+        inverse_sums(a, LD, W8, b, lb, limx, 32 * wi + lane, 32 * nw);
     };
     for (int b = 0; b < nb; ++b) {
         const int kb = kDB * b;
